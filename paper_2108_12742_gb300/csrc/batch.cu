@@ -148,9 +148,12 @@ __global__ void __launch_bounds__(256, batch_min_blocks<R>()) batch_kernel(const
         A.inc_in = stage == 0 ? nullptr : B.inc[stage - 1] + off;
         A.inc_out = stage == 2 ? nullptr : B.inc[stage] + off;
         A.stage = stage;
+        set_component_pointers(A, sizeof(R) == 4);
         A.mode = kModeCombine | (stage == 2 || per_stage ? kModeAlpha : 0);
+        TileConst<R> k;
+        tile_const<ORDER, R>(A, a_stage, dt, k);
         for (long long tile = 0; tile < A.ntiles; ++tile)
-          sweep_tile<NV, ORDER, R, true>(A, tile_geo(A, tile), smem_raw, a_stage, dt, amax, nfall);
+          sweep_tile<NV, ORDER, R, true, false, false, false, kShapeXCombine>(A, tile_geo(A, tile), smem_raw, k, amax, nfall);
         if constexpr (NV > 1) {
           if (stage == 2)
             alpha = block_max(amax[0], s_red);
@@ -197,10 +200,9 @@ namespace {
 
 template <int NV, int ORDER, typename R>
 cudaError_t launch_batch_t(const BatchArgs& b, int block, size_t smem, int sms, cudaStream_t s) {
-  cudaError_t e = raise_smem_limit(batch_kernel<NV, ORDER, R>, smem);
-  if (e != cudaSuccess) return e;
   int per_sm = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_kernel<NV, ORDER, R>, block, smem);
+  cudaError_t e = sweep_setup(reinterpret_cast<const void*>(batch_kernel<NV, ORDER, R>), block, smem,
+                              &per_sm);
   if (e != cudaSuccess) return e;
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
   const int grid = std::min(b.nprob, sms * per_sm);
@@ -296,7 +298,7 @@ BatchArgs make_args(enoao_ctx* c, int nsteps, double cfl) {
 enoao_status enqueue_batch(enoao_ctx* c, int nsteps, double cfl) {
   BatchState* b = c->batch;
   const int f32 = c->cfg.precision == ENOAO_FP32_BULK;
-  const size_t smem = sweep_smem_bytes(b->nv, c->cfg.order, f32, 1, b->ts,
+  const size_t smem = sweep_smem_bytes(b->nv, f32, 1,
                                        sweep_row_pitch(b->nv, c->cfg.order, f32, 0, 1, b->ts));
   cudaError_t e = launch_batch(b->nv, c->cfg.order, f32, make_args(c, nsteps, cfl), b->block, smem,
                                c->sms, c->s);

@@ -291,22 +291,57 @@ bool fp32(const enoao_ctx* c) { return c->cfg.precision == ENOAO_FP32_BULK; }
 
 int halo(int order) { return order / 2 + 2; }
 
-// Tile lengths are 2^k - 1 cells so that the 2^k faces of a line fill whole
-// warps in the per-face phase.
+// Default tile of axis d for an FP32-bulk sweep of this grid: the candidate
+// of the least modelled time.  A tile costs a fixed part, a part per face (the
+// ones not proven smooth) and, per phase, as many rounds as its cells (phase
+// 1: with the halo) or faces take over the threads of a line; the sweep takes
+// as many tiles as the resident blocks do in turn, and one more (the tail).
+// Candidates fill whole rounds, so ragged lengths and small grids -- which want
+// many small tiles -- come out of the same rule.  Tiles whose shared memory
+// would leave fewer than seven blocks an SM are not considered.  y and z tiles
+// of 8 lines use half of each 128-byte line they touch (256^3 z sweep: 8 x 31
+// 1.18 ms, 16 x 16 0.82 ms); x tiles of one or two lines were up to 10 %
+// behind four (4096^2 ENO-AO7 x sweep: 1 x 374 0.67, 2 x 118 0.60, 4 x 86 0.56 ms).
+void pick_tile(const enoao_ctx* c, int d, int* ta_out, int* ts_out) {
+  const int G = halo(c->cfg.order);
+  const long long nd = c->cfg.n[d], lines = c->ncell / nd;
+  const long long na = d == 0 ? lines : c->cfg.n[0], nb = lines / na;
+  double best = 1e300;
+  for (int ta = d == 0 ? 1 : 8; ta <= (d == 0 ? 4 : 16); ta *= 2) {
+    if (c->cfg.ndim == 1 && ta > 1) break;
+    const int tpl = 128 / ta;  // threads of a line
+    for (int k = 1; k <= 16; ++k) {
+      for (int ts : {tpl * k - 2 * G, tpl * k - 1}) {
+        if (ts < 8) continue;
+        const int se = sweep_row_pitch(c->nv, c->cfg.order, 1, d, ta, ts);
+        if (sweep_smem_bytes(c->nv, 1, ta, se) > 33 * 1024) continue;
+        const double tiles = (double)((nd + ts - 1) / ts) * ((na + ta - 1) / ta) * nb;
+        const int r1 = (ts + 2 * G + tpl - 1) / tpl, r2 = (ts + 1 + tpl - 1) / tpl,
+                  r3 = (ts + tpl - 1) / tpl;
+        double t = (80 + 130 * r1 + 90 * r2 + 80 * r3 + ta * (ts + 1)) * (1 + tiles / (8.0 * c->sms));
+        if (d > 0 && ta == 8) t *= 1.25;
+        if (d == 0 && ta < 4 && c->cfg.ndim > 1) t *= ta == 1 ? 1.1 : 1.04;
+        if (t < best) best = t, *ta_out = ta, *ts_out = ts;
+      }
+    }
+  }
+}
+
+// FP64 and per-field sweeps: tile lengths are 2^k - 1 cells, so that the 2^k
+// faces of a line fill whole warps in the per-face phase.
 void default_tiles(enoao_ctx* c) {
-  const bool f32 = fp32(c);
+  const bool f32 = fp32(c), prove = f32 && !consts(c).field;
   for (int d = 0; d < c->cfg.ndim; ++d) {
-    // FP32 2D ENO-AO5: 2 x 191 (x) and 8 x 31 (y) tiles take the LEAN kernel
-    // at eight blocks per SM (measured fastest on 4096^2 Euler data)
-    const bool lean2d = f32 && c->cfg.ndim == 2 && c->cfg.order == 5;
-    if (d == 0) {
-      c->ta[d] = c->cfg.ndim == 1 ? 1 : (lean2d ? 2 : 4);
-      c->ts[d] = lean2d ? 191 : 63;
+    c->block[d] = 128;
+    if (prove) {
+      pick_tile(c, d, &c->ta[d], &c->ts[d]);
+    } else if (d == 0) {
+      c->ta[d] = c->cfg.ndim == 1 ? 1 : 4;
+      c->ts[d] = 63;
     } else {
       c->ta[d] = f32 ? 8 : 32;
-      c->ts[d] = f32 ? (lean2d ? 31 : 47) : 15;
+      c->ts[d] = f32 ? 47 : 15;
     }
-    c->block[d] = 128;
   }
 }
 
@@ -317,9 +352,12 @@ enoao_status check_tiles(enoao_ctx* c, int d, int ta, int ts) {
     return fail(c, ENOAO_EINVAL, "axis %d needs 8, 16, 32 or 64 lines per tile", d);
   if (d == 0 && ta != 1 && ta != 2 && ta != 4 && ta != 8)
     return fail(c, ENOAO_EINVAL, "axis 0 needs 1, 2, 4 or 8 lines per tile");
-  size_t smem = sweep_smem_bytes(c->nv, c->cfg.order, fp32(c), ta, ts,
-                                 sweep_row_pitch(c->nv, c->cfg.order, fp32(c), d, ta, ts));
-  if (smem > 200 * 1024)
+  const int field = consts(c).field;
+  size_t smem = sweep_smem_bytes(
+      c->nv, fp32(c), ta, sweep_row_pitch(c->nv, c->cfg.order, fp32(c), d, ta, ts, field), field);
+  // (FP32 bulk keeps a value per cell more than the 200 KB that tiles may take
+  // were set for)
+  if (smem > (fp32(c) ? 216 : 200) * 1024)
     return fail(c, ENOAO_EINVAL, "tile %dx%d needs %zu bytes of shared memory", ta, ts, smem);
   return ENOAO_OK;
 }
@@ -471,7 +509,7 @@ enoao_status fill_sweep_args(enoao_ctx* c, int d, int stage, int mode, const dou
   a.stage = stage;
   a.ta = ta;
   a.ts = ts;
-  a.se = sweep_row_pitch(c->nv, c->cfg.order, fp32(c), d, a.ta, a.ts);
+  a.se = sweep_row_pitch(c->nv, c->cfg.order, fp32(c), d, a.ta, a.ts, consts(c).field);
   const long long nd = c->cfg.n[d];
   a.nfaces = c->ncell / nd * (nd + 1);
   a.tiles_s = (nd + a.ts - 1) / a.ts;
@@ -491,6 +529,7 @@ enoao_status fill_sweep_args(enoao_ctx* c, int d, int stage, int mode, const dou
   a.delta = c->cfg.delta;
   a.tie_rel = c->cfg.tie_rel;
   set_derived_constants(a);
+  set_component_pointers(a, fp32(c));
   a.redo_passes = c->redo_passes >= 0 ? c->redo_passes : 64 * c->nv;
   return ENOAO_OK;
 }
@@ -503,49 +542,23 @@ enoao_status launch_sweep(enoao_ctx* c, int d, int stage, int mode, const double
                                     c->ts[d], a);
   if (r0 != ENOAO_OK) return r0;
   CUtensorMap tmap;
-  const size_t smem0 = sweep_smem_bytes(c->nv, c->cfg.order, fp32(c), a.ta, a.ts, a.se);
+  const size_t smem0 = sweep_smem_bytes(c->nv, fp32(c), a.ta, a.se, consts(c).field);
   bool tma = encode_tile_map(c, d, list, u_in, a, &tmap);
   if (tma && smem0 + (size_t)a.tma_raw_bytes > 200 * 1024) tma = false;  // no room for the box
   const size_t smem = smem0 + (tma ? (size_t)a.tma_raw_bytes : 0);
   const int block = c->block[d];
   int per_sm = 1;
-  cudaError_t e;
-  const int nv = c->nv, order = c->cfg.order;
   a.field = consts(c).field;
-  if (fp32(c)) {
-    // ENO-AO5 tiles that let seven (or eight) blocks share an SM take the
-    // LEAN kernel (re-decisions out of line, 64 registers); measured faster there
-    if (!a.field && !list && !tma && order == 5 && smem * 7 <= 220 * 1024) {
-      int lean_per_sm = 0;
-      if (sweep_configure_fp32(nv, order, smem, 2) == cudaSuccess &&
-          sweep_occupancy_fp32(nv, order, block, smem, &lean_per_sm, 2) == cudaSuccess &&
-          lean_per_sm >= 7)
-        a.lean = 1;
-      cudaGetLastError();
-    }
-    const int variant = tma ? 1 : (a.lean ? 2 : 0);
-    e = a.field ? sweep_configure_fp32_field(nv, order, smem)
-                : sweep_configure_fp32(nv, order, smem, variant);
-    if (e == cudaSuccess)
-      e = a.field ? sweep_occupancy_fp32_field(nv, order, block, smem, &per_sm)
-                  : sweep_occupancy_fp32(nv, order, block, smem, &per_sm, variant);
-  } else {
-    e = a.field ? sweep_configure_fp64_field(nv, order, smem) : sweep_configure_fp64(nv, order, smem);
-    if (e == cudaSuccess)
-      e = a.field ? sweep_occupancy_fp64_field(nv, order, block, smem, &per_sm)
-                  : sweep_occupancy_fp64(nv, order, block, smem, &per_sm);
-  }
+  const int variant = fp32(c) ? (a.field ? kSweepFp32Field
+                                         : (tma ? kSweepFp32Tma : (list ? kSweepFp32List : kSweepFp32)))
+                              : (a.field ? kSweepFp64Field : kSweepFp64);
+  const void* kernel = sweep_kernel_for(c->nv, c->cfg.order, sweep_shape(d, mode), variant);
+  cudaError_t e = sweep_setup(kernel, block, smem, &per_sm);
   if (e != cudaSuccess) return fail(c, ENOAO_ECUDA, "sweep setup: %s", cudaGetErrorString(e));
   if (per_sm < 1) return fail(c, ENOAO_EINVAL, "sweep tile does not fit on an SM");
   long long grid = std::min<long long>(a.ntiles, (long long)c->sms * per_sm);
   if (grid < 1) grid = 1;
-  if (a.field)
-    e = fp32(c) ? sweep_launch_fp32_field(nv, order, a, (int)grid, block, smem, c->s)
-                : sweep_launch_fp64_field(nv, order, a, (int)grid, block, smem, c->s);
-  else
-    e = fp32(c) ? sweep_launch_fp32(nv, order, a, (int)grid, block, smem, c->s,
-                                    tma ? &tmap : nullptr)
-                : sweep_launch_fp64(nv, order, a, (int)grid, block, smem, c->s);
+  e = sweep_launch(kernel, a, (int)grid, block, smem, c->s, tma ? &tmap : nullptr);
   if (e != cudaSuccess) return fail(c, ENOAO_ECUDA, "sweep launch: %s", cudaGetErrorString(e));
   if (after_sweep) CU(c, cudaEventRecord(after_sweep, c->s));
   if (list) {
@@ -583,25 +596,19 @@ enoao_status launch_fused_stage(enoao_ctx* c, int stage, const double* in, doubl
                       out, nullptr, nullptr, false, ft[2], ft[3], ay);
   if (r != ENOAO_OK) return r;
   const int nv = c->nv, order = c->cfg.order, block = 128;
-  const size_t sx = sweep_smem_bytes(nv, order, true, ax.ta, ax.ts, ax.se);
-  const size_t sy = sweep_smem_bytes(nv, order, true, ay.ta, ay.ts, ay.se);
+  const size_t sx = sweep_smem_bytes(nv, true, ax.ta, ax.se);
+  const size_t sy = sweep_smem_bytes(nv, true, ay.ta, ay.se);
   const size_t smem = sx > sy ? sx : sy;
-  int lean = 0, per_sm = 0;
-  if (order == 5 && smem * 7 <= 220 * 1024) {
-    int p = 0;
-    if (fused2d_configure_fp32(nv, order, smem, 1) == cudaSuccess &&
-        fused2d_occupancy_fp32(nv, order, block, smem, &p, 1) == cudaSuccess && p >= 7)
-      lean = 1;
-    cudaGetLastError();
-  }
-  cudaError_t e = fused2d_configure_fp32(nv, order, smem, lean);
-  if (e == cudaSuccess) e = fused2d_occupancy_fp32(nv, order, block, smem, &per_sm, lean);
+  int per_sm = 0;
+  const void* kernel = fused2d_kernel_for(nv, order);
+  cudaError_t e = sweep_setup(kernel, block, smem, &per_sm);
   if (e != cudaSuccess) return fail(c, ENOAO_ECUDA, "fused stage setup: %s", cudaGetErrorString(e));
   if (per_sm < 1) return fail(c, ENOAO_EINVAL, "fused stage tiles do not fit on an SM");
   const long long tiles = ax.tiles_s * ay.tiles_s;
   long long grid = std::min<long long>(tiles, (long long)c->sms * per_sm);
   if (grid < 1) grid = 1;
-  e = fused2d_launch_fp32(nv, order, ax, ay, (int)grid, block, smem, c->s, lean);
+  void* args[2] = {&ax, &ay};
+  e = cudaLaunchKernel(kernel, dim3((unsigned)grid), dim3(block), args, smem, c->s);
   if (e != cudaSuccess) return fail(c, ENOAO_ECUDA, "fused stage launch: %s", cudaGetErrorString(e));
   return ENOAO_OK;
 }

@@ -59,7 +59,43 @@ constexpr int kModeAlpha = 8;      // accumulate alpha of u_out: for the next st
                                    // (stage 2) or the next stage (stages 0, 1)
 constexpr int kModeFlux = 16;      // write interface fluxes (and choices)
 
+// The arrays of a sweep by component, in sweep order (momentum along the
+// swept axis first, tangential momenta cyclic): set_component_pointers.  Kernels
+// address a cell as one multiply-add onto these.
+struct ComponentPtrs {
+  const double* u_in[kMaxNv];
+  const double* u0[kMaxNv];
+  double* u_out[kMaxNv];
+  void* rhs[kMaxNv];
+  const float* inc_in[kMaxNv];
+  float* inc_out[kMaxNv];
+};
+
+// Shapes of a sweep kernel: the axis class and mode it is compiled for (the
+// first axis stores L(u), later ones add theirs, the last one combines; 1D
+// combines at once).  Sizes, stage, boundary and alpha stay arguments.  One
+// kernel for every mode kept the values of all of them live and recomputed
+// under the register cap; the compiled shapes issue a fifth fewer instructions.
+enum SweepShape {
+  kShapeAny = 0,   // everything from the arguments (per-field, TMA staging)
+  kShapeXStore,
+  kShapeXCombine,
+  kShapeYStore,    // y or z, adding to the earlier axes
+  kShapeYCombine,
+  kShapeFlux       // interface fluxes, any axis
+};
+inline int sweep_shape(int dir, int mode) {
+  if (mode & kModeFlux) return kShapeFlux;
+  if (mode == kModeRhsStore) return dir == 0 ? kShapeXStore : kShapeAny;
+  if (mode == (kModeRhsStore | kModeRhsAdd)) return dir > 0 ? kShapeYStore : kShapeAny;
+  const int m = mode & ~kModeAlpha;
+  if (m == kModeCombine) return dir == 0 ? kShapeXCombine : kShapeAny;
+  if (m == (kModeCombine | kModeRhsAdd)) return dir > 0 ? kShapeYCombine : kShapeAny;
+  return kShapeAny;
+}
+
 struct SweepArgs {
+  ComponentPtrs comp;
   const double* u_in;   // U^(s): stencil source, [nv][N]
   const double* u0;     // U^n for the Runge-Kutta combine
   double* u_out;        // combined state
@@ -92,7 +128,6 @@ struct SweepArgs {
   int ta, ts;           // tile: lines x faces
   int se;               // shared-memory row pitch in cells (sweep_row_pitch)
   int field;            // 1: per-field splitting constants (st->alpha_f), Euler only
-  int lean;             // FP32 bulk, ENO-AO5, in-sweep re-decision: the seven-block variant
   int tma_box;          // TMA: box extent along the swept axis (cells, with alignment slack)
   unsigned tma_bytes;   // TMA: bytes of one box
   int tma_raw_bytes;    // TMA: shared memory reserved for the box (a multiple of 128)
@@ -126,48 +161,57 @@ __host__ __device__ inline void set_derived_constants(SweepArgs& a) {
   a.inv_dx_f = (float)a.inv_dx;
 }
 
-// Host-side entry points of the instantiation units (sweep_fp64.cu,
-// sweep_fp32.cu); return cudaError_t values.
+// Component pointers of a SweepArgs from its arrays, ndim, dir, cstride and the
+// bulk precision (fp32: element size of rhs).
+__host__ __device__ inline void set_component_pointers(SweepArgs& a, bool fp32) {
+  for (int c = 0; c < kMaxNv; ++c) {
+    const int k = c >= 1 && c <= a.ndim ? 1 + (a.dir + c - 1) % a.ndim : c;
+    const long long off = a.cstride * k;
+    a.comp.u_in[c] = a.u_in + off;
+    a.comp.u0[c] = a.u0 + off;
+    a.comp.u_out[c] = a.u_out + off;
+    a.comp.rhs[c] = static_cast<char*>(a.rhs) + off * (fp32 ? 4 : 8);
+    a.comp.inc_in[c] = a.inc_in + off;
+    a.comp.inc_out[c] = a.inc_out + off;
+  }
+}
+
+// Host-side interface of the instantiation units.
 }  // namespace enoao
 #include <cuda.h>
 #include <cuda_runtime.h>
 namespace enoao {
-// tmap: the stencil source as a tensor map for TMA staging of raw tiles (FP32
-// bulk sweeps that re-decide in the sweep), or NULL for direct loads.
-cudaError_t sweep_launch_fp64(int nv, int order, const SweepArgs& a, int grid, int block,
-                              size_t smem, cudaStream_t s);
-cudaError_t sweep_launch_fp32(int nv, int order, const SweepArgs& a, int grid, int block,
-                              size_t smem, cudaStream_t s, const CUtensorMap* tmap = nullptr);
-cudaError_t sweep_configure_fp64(int nv, int order, size_t smem);
-// variant: 0 the regular in-sweep / listing kernels, 1 TMA staging, 2 LEAN
-cudaError_t sweep_configure_fp32(int nv, int order, size_t smem, int variant = 0);
-cudaError_t sweep_occupancy_fp64(int nv, int order, int block, size_t smem, int* per_sm);
-cudaError_t sweep_occupancy_fp32(int nv, int order, int block, size_t smem, int* per_sm,
-                                 int variant = 0);
+// The sweep kernel for a system, order, shape and variant, or NULL: FP32 bulk
+// re-deciding its near-ties in the sweep, the same with raw tiles staged by
+// TMA, FP32 bulk listing them for the grid-wide pass, FP64, and either
+// precision with per-field splitting constants (Euler systems).
+enum SweepVariant { kSweepFp32, kSweepFp32Tma, kSweepFp32List, kSweepFp64, kSweepFp32Field, kSweepFp64Field };
+const void* sweep_kernel_for(int nv, int order, int shape, int variant);
+// by instantiation unit
+const void* sweep_fp32_o5(int nv, int shape, int variant);
+const void* sweep_fp32_o7(int nv, int shape, int variant);
+const void* sweep_fp32_list_o5(int nv, int shape);
+const void* sweep_fp32_list_o7(int nv, int shape);
+const void* sweep_fp64(int nv, int order, int shape);
+const void* sweep_fp32_field(int nv, int order);
+const void* sweep_fp64_field(int nv, int order);
+// the fused 2D stage kernel (both axes in one launch; FP32 bulk, nv 1 or 4)
+const void* fused2d_kernel_for(int nv, int order);
 cudaError_t redo_launch_fp32(int nv, int order, const SweepArgs& a, int grid, cudaStream_t s);
-// per-field splitting constants (a.field; Euler systems, nv 3..5)
-cudaError_t sweep_launch_fp64_field(int nv, int order, const SweepArgs& a, int grid, int block,
-                                    size_t smem, cudaStream_t s);
-cudaError_t sweep_launch_fp32_field(int nv, int order, const SweepArgs& a, int grid, int block,
-                                    size_t smem, cudaStream_t s);
-cudaError_t sweep_configure_fp64_field(int nv, int order, size_t smem);
-cudaError_t sweep_configure_fp32_field(int nv, int order, size_t smem);
-cudaError_t sweep_occupancy_fp64_field(int nv, int order, int block, size_t smem, int* per_sm);
-cudaError_t sweep_occupancy_fp32_field(int nv, int order, int block, size_t smem, int* per_sm);
-// the fused 2D stage kernel (both axes in one launch; FP32 bulk, nv 1 or 4):
-// ax the x sweep's arguments, ay the y sweep's; lean: the seven-block ENO-AO5 form
-cudaError_t fused2d_launch_fp32(int nv, int order, const SweepArgs& ax, const SweepArgs& ay,
-                                int grid, int block, size_t smem, cudaStream_t s, int lean);
-cudaError_t fused2d_configure_fp32(int nv, int order, size_t smem, int lean);
-cudaError_t fused2d_occupancy_fp32(int nv, int order, int block, size_t smem, int* per_sm,
-                                   int lean);
+
+// tmap: the stencil source as a tensor map for TMA staging, or NULL.
+inline cudaError_t sweep_launch(const void* kernel, const SweepArgs& a, int grid, int block,
+                                size_t smem, cudaStream_t s, const CUtensorMap* tmap = nullptr) {
+  CUtensorMap none{};  // direct loads: the map is not read
+  void* args[2] = {const_cast<SweepArgs*>(&a), tmap ? const_cast<CUtensorMap*>(tmap) : &none};
+  return cudaLaunchKernel(kernel, dim3(grid), dim3(block), args, smem, s);
+}
 
 // Raises a kernel's dynamic shared-memory limit to at least smem, never
 // lowers it: the limit belongs to the kernel, not to one launch, and the
 // axes and tiles of one kernel (and launches captured earlier into a graph)
 // need different sizes.
-template <typename Kernel>
-cudaError_t raise_smem_limit(Kernel* kernel, size_t smem) {
+inline cudaError_t raise_smem_limit(const void* kernel, size_t smem) {
   cudaFuncAttributes fa;
   cudaError_t e = cudaFuncGetAttributes(&fa, kernel);
   if (e != cudaSuccess) return e;
@@ -175,20 +219,30 @@ cudaError_t raise_smem_limit(Kernel* kernel, size_t smem) {
   return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
 }
 
-// Dynamic shared memory of one sweep block: per extended cell, the split
-// differences (2 nv), the face corrections (nv), the Roe ingredients (nv for
-// the Euler equations) and, in FP32 bulk mode, one word of near-tie flags.
+// Readies a kernel for smem bytes of dynamic shared memory and gives the
+// blocks of it that share an SM.
+inline cudaError_t sweep_setup(const void* kernel, int block, size_t smem, int* per_sm) {
+  if (!kernel) return cudaErrorInvalidValue;
+  cudaError_t e = raise_smem_limit(kernel, smem);
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, kernel, block, smem);
+  return e;
+}
+
+// Cell slots of a tile's shared-memory planes: a multiple of four, so that
+// every plane starts on a 16-byte boundary.
+__host__ __device__ constexpr int tile_cells(int ta, int se) { return (ta * se + 3) & ~3; }
+
 // Row pitch (cells) of a tile's shared-memory rows.  x sweeps read along a
 // row (any pitch); y/z sweeps put lines on lanes, so the pitch must spread a
 // warp's lanes over distinct banks: odd for 32- and 64-line tiles, for 8-byte
-// elements and for FP32 four-component cells (one 16-byte vector per cell:
+// elements and for FP32 Euler cells (16-byte vectors:
 // each quarter-warp access then covers eight distinct 16-byte bank groups),
-// 2 (mod 4) for other 16-line FP32 tiles (a warp spans two cells of 16 lines).
-inline int sweep_row_pitch(int nv, int order, int fp32, int dir, int ta, int ts) {
+// 2 (mod 4) for 16-line FP32 tiles kept in planes (a warp spans two cells of 16 lines).
+inline int sweep_row_pitch(int nv, int order, int fp32, int dir, int ta, int ts, int field = 0) {
   const int G = order / 2 + 2;
   int se = ts + 2 * G;
   if (dir == 0) return se;
-  if (fp32 && ta == 16 && nv != 4) {
+  if (fp32 && ta == 16 && (nv == 1 || (field && nv != 4))) {
     while (se % 4 != 2) ++se;
   } else {
     if (se % 2 == 0) ++se;
@@ -196,11 +250,18 @@ inline int sweep_row_pitch(int nv, int order, int fp32, int dir, int ta, int ts)
   return se;
 }
 
-inline size_t sweep_smem_bytes(int nv, int order, int fp32, int ta, int ts, int se) {
-  (void)ts;
-  const size_t cells = (size_t)ta * (size_t)se;
-  const int per = 3 * nv + (nv > 1 ? nv : 0) + (fp32 ? 1 : 0);
-  return cells * per * (fp32 ? 4 : 8);
+// Dynamic shared memory of one sweep block: per extended cell the split
+// differences and the face correction (three vectors), the Roe ingredients
+// (Euler equations), in FP32 bulk with one splitting constant the magnitude of
+// the pair's differences, and in FP32 bulk a word of the face list.  The FP32
+// vectors of the 1D system are four values wide, the spare ones taking the
+// magnitude and two of its Roe ingredients.
+inline size_t sweep_smem_bytes(int nv, int fp32, int ta, int se, int field = 0) {
+  const size_t cells = (size_t)tile_cells(ta, se);
+  const int prims = nv > 1 ? nv : 0;
+  if (!fp32) return cells * (size_t)(3 * nv + prims) * 8;
+  if (field) return cells * (size_t)(4 * nv + 1) * 4;
+  return cells * (size_t)(nv == 3 ? 14 : 3 * nv + prims + 2) * 4;
 }
 
 }  // namespace enoao

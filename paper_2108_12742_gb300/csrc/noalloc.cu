@@ -202,13 +202,11 @@ extern "C" enoao_status enoao_step_noalloc(const enoao_config* cfg, const double
   a.tie_rel = cfg->tie_rel;
   set_derived_constants(a);
   a.redo_passes = 64 * nv;
-  const size_t smem = sweep_smem_bytes(nv, cfg->order, f32, a.ta, a.ts, a.se);
+  const size_t smem = sweep_smem_bytes(nv, f32, a.ta, a.se);
   const int block = 128;
   int per_sm = 1;
-  e = f32 ? sweep_configure_fp32(nv, cfg->order, smem) : sweep_configure_fp64(nv, cfg->order, smem);
-  if (e == cudaSuccess)
-    e = f32 ? sweep_occupancy_fp32(nv, cfg->order, block, smem, &per_sm)
-            : sweep_occupancy_fp64(nv, cfg->order, block, smem, &per_sm);
+  const void* kernel = sweep_kernel_for(nv, cfg->order, kShapeXCombine, f32 ? kSweepFp32 : kSweepFp64);
+  e = sweep_setup(kernel, block, smem, &per_sm);
   if (e != cudaSuccess) return nofail(ENOAO_ECUDA, std::string("sweep setup: ") + cudaGetErrorString(e));
   const int grid = (int)std::max<long long>(1, std::min<long long>(a.ntiles, (long long)sms * per_sm));
   // stage 0: U1 = U^n + dt L(U^n); stage 1: U2 = 3/4 U^n + 1/4 (U1 + dt L(U1));
@@ -228,9 +226,9 @@ extern "C" enoao_status enoao_step_noalloc(const enoao_config* cfg, const double
     a.inc_in = stage == 0 ? nullptr : (stage == 1 ? I0 : I1);
     a.inc_out = stage == 0 ? I0 : (stage == 1 ? I1 : nullptr);
     a.stage = stage;
+    set_component_pointers(a, f32);
     a.mode = kModeCombine;
-    e = f32 ? sweep_launch_fp32(nv, cfg->order, a, grid, block, smem, s)
-            : sweep_launch_fp64(nv, cfg->order, a, grid, block, smem, s);
+    e = sweep_launch(kernel, a, grid, block, smem, s);
     if (e != cudaSuccess) return nofail(ENOAO_ECUDA, std::string("sweep launch: ") + cudaGetErrorString(e));
   }
   int err = 0;

@@ -106,6 +106,18 @@ __device__ __forceinline__ double brcp(double a) { return 1.0 / a; }
 __device__ __forceinline__ float brcp(float a) { return __fdividef(1.0f, a); }
 __device__ __forceinline__ double bdiv(double a, double b) { return a / b; }
 __device__ __forceinline__ float bdiv(float a, float b) { return __fdividef(a, b); }
+// A product that is rounded before whatever is added to it, in every kernel.
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+// a b + c d with the first product fused.  Sums of products are written out
+// with fma, dot2 and mul_rn from the state to the choice: which product the
+// compiler fuses by itself changes from one kernel to the next, and every
+// kernel must give the same bits -- the re-decision passes most of all, which
+// re-derive the FP32 pick of a near-tie from its window.
+template <typename T>
+__device__ __forceinline__ T dot2(T a, T b, T c, T d) {
+  return fma(a, b, mul_rn(c, d));
+}
 // Absolute value (a sign-bit operation, no floating-point instruction).
 __device__ __forceinline__ double rabs(double a) { return fabs(a); }
 __device__ __forceinline__ float rabs(float a) { return fabsf(a); }
@@ -201,7 +213,7 @@ __device__ __forceinline__ R eno_select(const R (&d)[8], R delta, R tie_rel, con
     // its nonzero coefficients: d[2..5] (ENO-AO5), d[1..6] (ENO-AO7)
 #pragma unroll
     for (int i = ORDER == 5 ? 2 : 1; i <= (ORDER == 5 ? 5 : 6); ++i)
-      corr += bcoef_top<ORDER, R>(i) * d[i];
+      corr = fma(bcoef_top<ORDER, R>(i), d[i], corr);
     if constexpr (CHECK) {
       // its bound: the Pascal sums of e over its two differences, written out
       R qa, qb;
@@ -321,7 +333,7 @@ __device__ __forceinline__ R eno_select(const R (&d)[8], R delta, R tie_rel, con
       marginal = m;
     }
 #pragma unroll
-    for (int i = LO; i <= HI; ++i) corr += bcoef<R>(pick, i) * d[i];
+    for (int i = LO; i <= HI; ++i) corr = fma(bcoef<R>(pick, i), d[i], corr);
   }
   pick_out = pick;
   return corr;
@@ -364,26 +376,37 @@ __device__ __forceinline__ void flux_diff(const T (&qa)[NV], const T (&qb)[NV], 
     const T ib = brcp(qb[0]);
     const T u = qa[1] * ia;
     T vt[NT > 0 ? NT : 1], dvt[NT > 0 ? NT : 1];
-    const T du = (dq[1] - u * dq[0]) * ib;
-    T v2 = u * u, vdv = u * du, dv2 = du * du;
+    const T du = fma(-u, dq[0], dq[1]) * ib;
 #pragma unroll
     for (int t = 0; t < NT; ++t) {
       vt[t] = qa[2 + t] * ia;
-      dvt[t] = (dq[2 + t] - vt[t] * dq[0]) * ib;
-      v2 += vt[t] * vt[t];
-      vdv += vt[t] * dvt[t];
-      dv2 += dvt[t] * dvt[t];
+      dvt[t] = fma(-vt[t], dq[0], dq[2 + t]) * ib;
     }
-    const T ke_a = T(0.5) * qa[0] * v2;
-    const T dke = T(0.5) * dq[0] * v2 + qb[0] * (vdv + T(0.5) * dv2);
-    const T pa = gm1 * (qa[NV - 1] - ke_a);
-    const T dp = gm1 * (dq[NV - 1] - dke);
+    T v2, dke2;  // |v|^2, and v . dv + |dv|^2 / 2
+    if constexpr (NT == 0) {
+      v2 = mul_rn(u, u);
+      dke2 = fma(u, du, T(0.5) * mul_rn(du, du));
+    } else {
+      v2 = dot2(u, u, vt[0], vt[0]);
+      T vdv = dot2(u, du, vt[0], dvt[0]);
+      T dv2 = dot2(du, du, dvt[0], dvt[0]);
+#pragma unroll
+      for (int t = 1; t < NT; ++t) {
+        v2 = fma(vt[t], vt[t], v2);
+        vdv = fma(vt[t], dvt[t], vdv);
+        dv2 = fma(dvt[t], dvt[t], dv2);
+      }
+      dke2 = fma(T(0.5), dv2, vdv);
+    }
+    const T dke = dot2(T(0.5) * dq[0], v2, qb[0], dke2);
+    const T ea = fma(T(-0.5) * qa[0], v2, qa[NV - 1]);  // internal energy
+    const T de = dq[NV - 1] - dke;
     const T ub = u + du;
     dF[0] = dq[1];
-    dF[1] = dq[1] * ub + qa[1] * du + dp;
+    dF[1] = fma(gm1, de, dot2(dq[1], ub, qa[1], du));
 #pragma unroll
-    for (int t = 0; t < NT; ++t) dF[2 + t] = dq[2 + t] * ub + qa[2 + t] * du;
-    dF[NV - 1] = (dq[NV - 1] + dp) * ub + (qa[NV - 1] + pa) * du;
+    for (int t = 0; t < NT; ++t) dF[2 + t] = dot2(dq[2 + t], ub, qa[2 + t], du);
+    dF[NV - 1] = dot2(fma(gm1, de, dq[NV - 1]), ub, fma(gm1, ea, qa[NV - 1]), du);
   }
 }
 
@@ -417,11 +440,10 @@ __device__ __forceinline__ void roe_prims(const T (&q)[NV], T gm1, T (&pr)[NV]) 
 #pragma unroll
     for (int i = 1; i < NV - 1; ++i) {
       pr[i] = q[i] * ir;
-      ke += q[i] * pr[i];
+      ke = fma(q[i], pr[i], ke);
     }
-    const T p = gm1 * (q[NV - 1] - T(0.5) * ke);
     pr[0] = bsqrt(q[0]);
-    pr[NV - 1] = (q[NV - 1] + p) * ir;
+    pr[NV - 1] = fma(gm1, fma(T(-0.5), ke, q[NV - 1]), q[NV - 1]) * ir;  // (E + p) / rho
   }
 }
 
@@ -437,20 +459,23 @@ __device__ __forceinline__ void roe_eigen(const T (&pl)[NV], const T (&prr)[NV],
   constexpr int NT = NV - 3;
   const T inv = brcp(pl[0] + prr[0]);
   const T wl = pl[0] * inv, wr = prr[0] * inv;
-  E.u = wl * pl[1] + wr * prr[1];
-  T q2 = E.u * E.u;
+  E.u = dot2(wl, pl[1], wr, prr[1]);
 #pragma unroll
-  for (int t = 0; t < NT; ++t) {
-    E.vt[t] = wl * pl[2 + t] + wr * prr[2 + t];
-    q2 += E.vt[t] * E.vt[t];
+  for (int t = 0; t < NT; ++t) E.vt[t] = dot2(wl, pl[2 + t], wr, prr[2 + t]);
+  T q2;
+  if constexpr (NT < 2) {
+    q2 = mul_rn(E.u, E.u);
+    if constexpr (NT == 1) q2 = fma(E.vt[0], E.vt[0], q2);
+  } else {
+    q2 = fma(E.vt[1], E.vt[1], dot2(E.u, E.u, E.vt[0], E.vt[0]));
   }
-  E.H = wl * pl[NV - 1] + wr * prr[NV - 1];
+  E.H = dot2(wl, pl[NV - 1], wr, prr[NV - 1]);
   E.q2 = q2;
-  const T c2 = gm1 * (E.H - T(0.5) * q2);
+  const T c2 = gm1 * fma(T(-0.5), q2, E.H);
   E.c = bsqrt(c2);
   E.ic = brcp(E.c);
   E.b1 = bdiv(gm1, c2);
-  E.b2 = T(0.5) * q2 * E.b1;
+  E.b2 = mul_rn(T(0.5) * q2, E.b1);
 }
 
 // The constant c ? 1 : 0 (and c ? 1 : -1) by an integer select: a
@@ -473,8 +498,8 @@ __device__ __forceinline__ void left_row(const Eigen<NV, T>& E, int v, T (&L)[NV
   constexpr int NT = NV - 3;
   if (v == 0 || v == NV - 1) {
     const T s = sign_if<T>(v == 0);
-    L[0] = T(0.5) * (E.b2 + s * E.u * E.ic);
-    L[1] = T(0.5) * (-E.b1 * E.u - s * E.ic);
+    L[0] = T(0.5) * fma(s * E.u, E.ic, E.b2);
+    L[1] = T(0.5) * fma(-E.b1, E.u, -(s * E.ic));
 #pragma unroll
     for (int t = 0; t < NT; ++t) L[2 + t] = T(-0.5) * E.b1 * E.vt[t];
     L[NV - 1] = T(0.5) * E.b1;
@@ -517,7 +542,7 @@ __device__ __forceinline__ void right_col(const Eigen<NV, T>& E, int v, T (&Rc)[
     Rc[1] = E.u + s * E.c;
 #pragma unroll
     for (int t = 0; t < NT; ++t) Rc[2 + t] = E.vt[t];
-    Rc[NV - 1] = E.H + s * E.u * E.c;
+    Rc[NV - 1] = fma(s * E.u, E.c, E.H);
   } else if (v == 1) {
     Rc[0] = T(1);
     Rc[1] = E.u;
@@ -584,15 +609,29 @@ __device__ __forceinline__ TileGeo tile_geo(const SweepArgs& A, long long tile) 
   return g;
 }
 
-// Loads the permuted state of one cell.  COHERENT loads go through L2 (the
-// batched kernel reads states it wrote itself); otherwise the read-only
-// path is used (a sweep never writes the array it stencils from).
+// Cell index within a component.  The Euler systems index with 32 bits (2^32
+// cells of three or more FP64 components in three state arrays do not fit the
+// device's memory), so that an access is one multiply-add onto a component's
+// uniform base; scalar arrays can be longer.
+template <int NV>
+struct CellIndex {
+  using type = unsigned;
+};
+template <>
+struct CellIndex<1> {
+  using type = unsigned long long;
+};
+template <int NV>
+using cell_t = typename CellIndex<NV>::type;
+
+// Loads the input state of one cell in sweep order.  COHERENT loads go
+// through L2 (the batched kernel reads states it wrote itself); otherwise the
+// read-only path is used (a sweep never writes the array it stencils from).
 template <int NV, bool COHERENT = false>
-__device__ __forceinline__ void load_state(const double* __restrict__ U, long long ncell,
-                                           long long cell, int dir, double (&q)[NV]) {
+__device__ __forceinline__ void load_state(const SweepArgs& A, cell_t<NV> cell, double (&q)[NV]) {
 #pragma unroll
   for (int c = 0; c < NV; ++c) {
-    const double* p = U + perm_comp<NV>(c, dir) * ncell + cell;
+    const double* p = A.comp.u_in[c] + cell;
     q[c] = COHERENT ? __ldcg(p) : __ldg(p);
   }
 }
@@ -613,8 +652,7 @@ __device__ __forceinline__ int redo_group(const SweepArgs& A, const TileGeo& g, 
   const long long line = g.base + (g.a0 + a) * g.stride_a;
   const int rr = r < 2 * G ? r : 2 * G - 1;
   double q[NV];
-  load_state<NV, COHERENT>(A.u_in, A.cstride, line + bc_map(sj - G + 1 + rr, g.nd, A.bc) * g.stride_d,
-                           A.dir, q);
+  load_state<NV, COHERENT>(A, line + bc_map(sj - G + 1 + rr, g.nd, A.bc) * g.stride_d, q);
   double L[NV];
   if constexpr (NV > 1) {
     double ql[NV], qr[NV], pl[NV], prr[NV];
@@ -642,7 +680,7 @@ __device__ __forceinline__ int redo_group(const SweepArgs& A, const TileGeo& g, 
     flux_diff<NV, double>(q, qn, dq, gm1, A.adv_speed, dF);
     const double sa = sgn == 0 ? alpha : -alpha;
 #pragma unroll
-    for (int c = 0; c < NV; ++c) w += L[c] * (0.5 * (dF[c] + sa * dq[c]));
+    for (int c = 0; c < NV; ++c) w = fma(L[c], 0.5 * fma(sa, dq[c], dF[c]), w);
   }
   // window difference k (between cells k and k+1) sits in group lane k
   double d[8];
@@ -675,8 +713,7 @@ __device__ __forceinline__ int redo_lane(const SweepArgs& A, const TileGeo& g, i
   // window cell r (0..2G-1) is cell sj - G + 1 + r of the line; the face lies
   // between cells G-1 and G
   auto load_cell = [&](int r, double (&q)[NV]) {
-    load_state<NV, COHERENT>(A.u_in, A.cstride, line + bc_map(sj - G + 1 + r, g.nd, A.bc) * g.stride_d,
-                             A.dir, q);
+    load_state<NV, COHERENT>(A, line + bc_map(sj - G + 1 + r, g.nd, A.bc) * g.stride_d, q);
   };
   double L[NV];
   if constexpr (NV > 1) {
@@ -711,7 +748,7 @@ __device__ __forceinline__ int redo_lane(const SweepArgs& A, const TileGeo& g, i
     flux_diff<NV, double>(qlo, qhi, dq, gm1, A.adv_speed, dF);
     double w = 0.0;
 #pragma unroll
-    for (int c = 0; c < NV; ++c) w += L[c] * (0.5 * (dF[c] + sa * dq[c]));
+    for (int c = 0; c < NV; ++c) w = fma(L[c], 0.5 * fma(sa, dq[c], dF[c]), w);
     d[i] = sgn == 0 ? w : -w;
     if (i < GE::HI) {
       const int k = sgn == 0 ? i + G - 5 : G + 3 - i;
@@ -738,11 +775,6 @@ __device__ __forceinline__ int nth_set_bit(unsigned x, int n) {
   for (int i = 0; i < n && x; ++i) x &= x - 1;
   return x ? __ffs(x) - 1 : -1;
 }
-
-template <int NV>
-struct NPrim {
-  static constexpr int value = NV > 1 ? NV : 0;
-};
 
 // Runs body(a, e) over the items of a TA x cnt tile.  x sweeps (sfast):
 // each thread keeps one line a and strides along e (lanes along the line);
@@ -779,29 +811,47 @@ __device__ __forceinline__ void item_start(int lgTA, bool sfast, int& a, int& e0
   }
 }
 
-// Per-cell vectors in shared memory.  FP32 four-component states (2D Euler)
-// are stored as one float4 per cell, so a cell moves in one 128-bit access;
-// every other case keeps one plane per component.  Both layouts take NV
-// values of R per cell slot.
-template <int NV, typename R>
+// Whether a sweep variant proves most faces to take the top candidate before
+// any projection (phase 2a below): FP32 bulk with one splitting constant.
+template <typename R, bool FIELD>
+constexpr bool kProve = sizeof(R) == 4 && !FIELD;
+
+// Per-cell vectors in shared memory.  FP32 vectors of the Euler equations are
+// one float4 per cell, so a cell moves in one 128-bit access: the 1D system
+// has a fourth value to spare (kSpare: phase 1 keeps a bound of the proof
+// there), the 3D system keeps its fifth in a plane behind the float4s.  FP64,
+// scalar and per-field 1D and 3D sweeps keep one plane per component.
+template <int NV, typename R, bool FIELD>
 struct CellVec {
-  static constexpr bool kAoS = sizeof(R) == 4 && NV == 4;
+  static constexpr bool kAoS = sizeof(R) == 4 && (NV == 4 || (NV >= 3 && !FIELD));
+  static constexpr bool kSpare = kAoS && NV == 3;
+  static constexpr int kSlots = kSpare ? 4 : NV;  // values of R per cell
   __device__ __forceinline__ static void load(const R* base, int cells, int i, R (&v)[NV]) {
     if constexpr (kAoS) {
       const float4 t = reinterpret_cast<const float4*>(base)[i];
-      v[0] = t.x, v[1] = t.y, v[2] = t.z, v[3] = t.w;
+      v[0] = t.x, v[1] = t.y, v[2] = t.z;
+      if constexpr (NV >= 4) v[3] = t.w;
+      if constexpr (NV == 5) v[4] = base[4 * cells + i];
     } else {
 #pragma unroll
       for (int c = 0; c < NV; ++c) v[c] = base[c * cells + i];
     }
   }
   __device__ __forceinline__ static void store(R* base, int cells, int i, const R (&v)[NV]) {
-    if constexpr (kAoS) {
+    if constexpr (kSpare) {  // the fourth value stays
+      reinterpret_cast<float2*>(base)[2 * i] = make_float2(v[0], v[1]);
+      base[4 * i + 2] = v[2];
+    } else if constexpr (kAoS) {
       reinterpret_cast<float4*>(base)[i] = make_float4(v[0], v[1], v[2], v[3]);
+      if constexpr (NV == 5) base[4 * cells + i] = v[4];
     } else {
 #pragma unroll
       for (int c = 0; c < NV; ++c) base[c * cells + i] = v[c];
     }
+  }
+  // with the spare fourth value of the 1D system
+  __device__ __forceinline__ static void store4(R* base, int i, const R (&v)[NV], R w) {
+    reinterpret_cast<float4*>(base)[i] = make_float4(v[0], v[1], v[2], w);
   }
 };
 
@@ -809,11 +859,13 @@ struct CellVec {
 // bulk precision (phase 1): dq = qb - qa rounded once from FP64, the flux
 // difference in difference form, and (dF +- alpha dq)/2 written as
 // dF/2 +- (alpha/2) dq (the same bits: halving is exact).
+// Returns sum_c max(|fp_c|, |fm_c|) = sum_c |dF_c|/2 + alpha |dq_c|/2, the
+// magnitude that bounds the FP32 rounding of both (unused results cost nothing).
 template <int NV, typename R>
-__device__ __forceinline__ void split_diff(const double (&qa64)[NV], const double (&qb64)[NV],
-                                           const R (&qa)[NV], const R (&qb)[NV], R gm1, R adv,
-                                           R halpha, R (&fp)[NV], R (&fm)[NV]) {
-  R dq[NV], dF[NV];
+__device__ __forceinline__ R split_diff(const double (&qa64)[NV], const double (&qb64)[NV],
+                                        const R (&qa)[NV], const R (&qb)[NV], R gm1, R adv,
+                                        R halpha, R (&fp)[NV], R (&fm)[NV]) {
+  R dq[NV], dF[NV], m = R(0);
 #pragma unroll
   for (int c = 0; c < NV; ++c) dq[c] = to_bulk<R>(qb64[c] - qa64[c]);
   flux_diff<NV, R>(qa, qb, dq, gm1, adv, dF);
@@ -822,7 +874,9 @@ __device__ __forceinline__ void split_diff(const double (&qa64)[NV], const doubl
     const R hdF = R(0.5) * dF[c];
     fp[c] = fma(halpha, dq[c], hdF);
     fm[c] = fma(-halpha, dq[c], hdF);
+    m = fma(halpha, rabs(dq[c]), m + rabs(hdF));
   }
+  return m;
 }
 
 // The same pair of cells for per-field splitting: dF/2 and dq/2 (exact
@@ -913,32 +967,79 @@ __device__ __forceinline__ void bulk_state_check(const SweepArgs& A, long long c
   }
 }
 
+// The axis class and the mode bits that a sweep kernel of a given shape
+// (enoao_internal.h) knows at compile time; kShapeAny takes both from its
+// arguments.
+template <int SHAPE>
+__device__ __forceinline__ bool shape_x(const SweepArgs& A) {
+  if constexpr (SHAPE == kShapeXStore || SHAPE == kShapeXCombine) return true;
+  if constexpr (SHAPE == kShapeYStore || SHAPE == kShapeYCombine) return false;
+  return A.dir == 0;
+}
+template <int SHAPE>
+__device__ __forceinline__ int shape_mode(const SweepArgs& A) {
+  if constexpr (SHAPE == kShapeXStore) return kModeRhsStore;
+  if constexpr (SHAPE == kShapeXCombine) return kModeCombine | (A.mode & kModeAlpha);
+  if constexpr (SHAPE == kShapeYStore) return kModeRhsStore | kModeRhsAdd;
+  if constexpr (SHAPE == kShapeYCombine) return kModeCombine | kModeRhsAdd | (A.mode & kModeAlpha);
+  if constexpr (SHAPE == kShapeFlux) return kModeFlux;
+  return A.mode;
+}
+
 // Number of alpha maxima a sweep accumulates: |u_d| + c per axis, or with
 // per-field constants |u_d - c|, |u_d|, |u_d + c| per axis.
 template <bool FIELD>
 constexpr int kAmax = FIELD ? 9 : 3;
 
-// The shared-memory planes of a tile (per extended cell: the split
-// differences df+ and df-, the face correction C, the Roe ingredients and,
-// in FP32 bulk, one word of near-tie flags) and the projected windows of its
-// faces, shared by the tile's phases and the out-of-line re-decision.
+// Entry of a tile's face list: line, face and the near-tie flags of the face's
+// choices (bit field * 2 + sign).
+__device__ __forceinline__ unsigned face_entry(int a, int f) {
+  return (unsigned)a << 26 | (unsigned)f << 10;
+}
+__device__ __forceinline__ int entry_line(unsigned e) { return (int)(e >> 26); }
+__device__ __forceinline__ int entry_face(unsigned e) { return (int)(e >> 10 & 0xffffu); }
+__device__ __forceinline__ unsigned entry_flags(unsigned e) { return e & 0x3ffu; }
+
+// The shared-memory planes of a tile, sizes as sweep_smem_bytes: per extended
+// cell the split differences df+ and df-, the face correction C, the Roe
+// ingredients, with kProve the magnitude of the pair's split differences, and
+// in FP32 bulk one word for the face list (faces not proven, or with flagged
+// choices).  The 1D system keeps the magnitude with df+ and two of its three
+// Roe ingredients with df- and C (the spare values).  Shared by the tile's
+// phases and the out-of-line re-decision.
 template <int NV, int ORDER, typename R, bool FIELD>
 struct TileView {
   using GE = Geo<ORDER>;
-  using CV = CellVec<NV, R>;
+  using CV = CellVec<NV, R, FIELD>;
   static constexpr bool FP32 = sizeof(R) == 4;
+  static constexpr bool PROVE = kProve<R, FIELD>;
   R* dfp;
   R* dfm;
   R* Cf;
-  R* prim;
-  unsigned* fixmask;
+  R* prim;         // 1D FP32: the third ingredient only
+  float* mag;      // PROVE, all but 1D Euler
+  unsigned* list;  // FP32
   int cells, SE;
-  __device__ __forceinline__ TileView(unsigned char* smem_raw, int ta, int se) : cells(ta * se), SE(se) {
+  __device__ __forceinline__ TileView(unsigned char* smem_raw, int ta, int se)
+      : cells(tile_cells(ta, se)), SE(se) {
     dfp = reinterpret_cast<R*>(smem_raw);
-    dfm = dfp + NV * cells;
-    Cf = dfm + NV * cells;
-    prim = Cf + NV * cells;
-    fixmask = reinterpret_cast<unsigned*>(prim + NPrim<NV>::value * cells);
+    dfm = dfp + CV::kSlots * cells;
+    Cf = dfm + CV::kSlots * cells;
+    prim = Cf + CV::kSlots * cells;
+    R* p = prim + (NV == 1 ? 0 : (CV::kSpare ? 1 : NV)) * cells;
+    mag = reinterpret_cast<float*>(p);
+    if constexpr (PROVE && NV != 3) p += cells;
+    list = reinterpret_cast<unsigned*>(p);
+  }
+  // Roe ingredients of the cell at slot i
+  __device__ __forceinline__ void load_prims(int i, R (&pr)[NV]) const {
+    if constexpr (CV::kSpare) {
+      pr[0] = dfm[4 * i + 3];
+      pr[1] = Cf[4 * i + 3];
+      pr[2] = prim[i];
+    } else {
+      CV::load(prim, cells, i, pr);
+    }
   }
   __device__ __forceinline__ int sidx(int a, int e) const { return a * SE + e; }
   // Projected window of face j (extended cells) onto the field with left
@@ -955,7 +1056,7 @@ struct TileView {
       CV::load(src, cells, e, x);
       R acc = R(0);
 #pragma unroll
-      for (int c = 0; c < NV; ++c) acc += L[c] * x[c];
+      for (int c = 0; c < NV; ++c) acc = fma(L[c], x[c], acc);
       d[i] = sgn == 0 ? acc : -acc;
     }
   }
@@ -973,8 +1074,8 @@ struct TileView {
       R acc = R(0), mag = R(0);
 #pragma unroll
       for (int c = 0; c < NV; ++c) {
-        acc += L[c] * x[c];
-        mag += rabs(L[c]) * rabs(x[c]);
+        acc = fma(L[c], x[c], acc);
+        mag = fma(rabs(L[c]), rabs(x[c]), mag);
       }
       d[i] = sgn == 0 ? acc : -acc;
       m[i] = mag;
@@ -994,9 +1095,9 @@ struct TileView {
         R x[NV];
         CV::load(src, cells, e, x);
         const R xv = shear_comp<NV>(x, v);
-        const R acc = xv - w * x[0];
+        const R acc = fma(-w, x[0], xv);
         d[i] = sgn == 0 ? acc : -acc;
-        if constexpr (FP32) m[i] = rabs(xv) + rabs(w) * rabs(x[0]);
+        if constexpr (FP32) m[i] = fma(rabs(w), rabs(x[0]), rabs(xv));
       }
     }
   }
@@ -1019,8 +1120,8 @@ struct TileView {
       if constexpr (NV >= 4) {
         if (shear) {
           const R fv = shear_comp<NV>(xF, v), qv = shear_comp<NV>(xq, v);
-          aF = fv - w * xF[0];
-          aq = qv - w * xq[0];
+          aF = fma(-w, xF[0], fv);
+          aq = fma(-w, xq[0], qv);
           if constexpr (FP32) {
             mF = rabs(fv) + rabs(w) * rabs(xF[0]);
             mq = rabs(qv) + rabs(w) * rabs(xq[0]);
@@ -1030,8 +1131,8 @@ struct TileView {
       if (!shear) {
 #pragma unroll
         for (int c = 0; c < NV; ++c) {
-          aF += L[c] * xF[c];
-          aq += L[c] * xq[c];
+          aF = fma(L[c], xF[c], aF);
+          aq = fma(L[c], xq[c], aq);
           if constexpr (FP32) {
             mF += rabs(L[c]) * rabs(xF[c]);
             mq += rabs(L[c]) * rabs(xq[c]);
@@ -1065,6 +1166,153 @@ struct TileView {
   }
 };
 
+// Roe average and eigenvectors of the face at slot i (between cells i and i+1).
+template <int NV, int ORDER, typename R, bool FIELD>
+__device__ __forceinline__ void face_eigen(const TileView<NV, ORDER, R, FIELD>& tv, int i, R gm1,
+                                           Eigen<NV, R>& E) {
+  R pl[NV], prr[NV];
+  tv.load_prims(i, pl);
+  tv.load_prims(i + 1, prr);
+  roe_eigen<NV, R>(pl, prr, gm1, E);
+}
+
+// Phase 2a on one face (between cells j and j+1 of its line; x is its slot):
+// proves that every characteristic field takes the top candidate for both
+// signs, and if so gives the correction C they make, with the operations (and
+// the bits) of choose_face but without its indicators, selection and bounds.
+//
+// The top candidate's indicator is at most |L_v . D|, D the undivided
+// difference of df+- over the window's five (ENO-AO7: seven) middle pairs; D
+// carries an FP32 error of at most feps times the Pascal sum P of the pairs'
+// magnitudes, so |L_v . D| one of at most K feps P, K the largest entry of the
+// left rows.  When |L_v . D| + K feps P is below delta by more than the
+// near-tie margin, principle 1 of Sec. 3.2 picks the top candidate without a
+// near-tie.  One difference decides a field instead of two per candidate and
+// their bounds; the faces of resolved flow end here (98 to 99.5 % of 2D data
+// at 2048^2 and more), the others go to the tile's face list.
+template <int NV, int ORDER, bool FIELD>
+__device__ __forceinline__ bool prove_top(const TileView<NV, ORDER, float, FIELD>& tv, int x,
+                                          float gm1, float limit, float (&C)[NV]) {
+  using CV = CellVec<NV, float, FIELD>;
+  constexpr int H = ORDER == 7 ? 3 : 2;  // pairs j-H .. j+H
+  constexpr float feps = (NV + 8) * FLT_EPSILON;
+  constexpr float bw[4] = {1.0f, ORDER == 7 ? -6.0f : -4.0f, ORDER == 7 ? 15.0f : 6.0f, -20.0f};
+  // window entries i whose Table-1 coefficients are nonzero
+  constexpr int B0 = ORDER == 5 ? 2 : 1, B1 = ORDER == 5 ? 5 : 6;
+  constexpr int ND = NV == 1 ? 1 : 3;       // dense rows: u-c, entropy, u+c
+  constexpr int NS = NV > 3 ? NV - 3 : 0;   // shear fields
+  float L[ND][NV], vt[NS > 0 ? NS : 1], K = 1.0f;
+  Eigen<NV, float> E;
+  if constexpr (NV > 1) {
+    face_eigen<NV, ORDER, float, FIELD>(tv, x, gm1, E);
+    left_row<NV, float>(E, 0, L[0]);
+    left_row<NV, float>(E, 1, L[1]);
+    left_row<NV, float>(E, NV - 1, L[2]);
+#pragma unroll
+    for (int t = 0; t < NS; ++t) {
+      vt[t] = E.vt[t];
+      K = fmaxf(K, fabsf(vt[t]));
+    }
+    // (the acoustic rows' later entries are halves of the entropy row's)
+    K = fmaxf(K, fmaxf(fmaxf(fabsf(L[0][0]), fabsf(L[2][0])), fmaxf(fabsf(L[0][1]), fabsf(L[2][1]))));
+#pragma unroll
+    for (int c = 0; c < NV; ++c) K = fmaxf(K, fabsf(L[1][c]));
+  } else {
+    L[0][0] = 1.0f;
+  }
+  float m[2 * H + 1];
+  float cv[ND], cs[NS > 0 ? NS : 1];  // values of the dense and the shear fields
+  bool ok = true;
+  float most = 0.0f;  // the largest |L_v . D|
+#pragma unroll
+  for (int sgn = 0; sgn < 2; ++sgn) {
+    const float* src = sgn == 0 ? tv.dfp : tv.dfm;
+    float D[NV], corr[ND], corrs[NS > 0 ? NS : 1];
+#pragma unroll
+    for (int c = 0; c < NV; ++c) D[c] = 0.0f;
+#pragma unroll
+    for (int v = 0; v < ND; ++v) corr[v] = 0.0f;
+#pragma unroll
+    for (int t = 0; t < NS; ++t) corrs[t] = 0.0f;
+    // pair j + k: window entry 4 + k of f^+ (sign 0), 4 - k of f^- (sign 1,
+    // negated); in the order of the entries
+#pragma unroll
+    for (int i = 4 - H; i <= 4 + H; ++i) {
+      const int k = sgn == 0 ? i - 4 : 4 - i;
+      float p[NV];
+      if constexpr (CV::kSpare) {
+        const float4 t = reinterpret_cast<const float4*>(src)[x + k];
+        p[0] = t.x, p[1] = t.y, p[2] = t.z;
+        if (sgn == 0) m[k + H] = t.w;
+      } else {
+        CV::load(src, tv.cells, x + k, p);
+        if (sgn == 0) m[k + H] = tv.mag[x + k];
+      }
+      const float w = bw[k <= 0 ? k + H : H - k];
+#pragma unroll
+      for (int c = 0; c < NV; ++c) D[c] = fmaf(w, p[c], D[c]);
+      if (i >= B0 && i <= B1) {
+        const float b = bcoef_top<ORDER, float>(i);
+#pragma unroll
+        for (int v = 0; v < ND; ++v) {
+          float acc = 0.0f;
+#pragma unroll
+          for (int c = 0; c < NV; ++c) acc = fmaf(L[v][c], p[c], acc);
+          corr[v] = fmaf(b, sgn == 0 ? acc : -acc, corr[v]);
+        }
+#pragma unroll
+        for (int t = 0; t < NS; ++t) {
+          const float acc = fmaf(-vt[t], p[0], p[2 + t]);
+          corrs[t] = fmaf(b, sgn == 0 ? acc : -acc, corrs[t]);
+        }
+      }
+    }
+#pragma unroll
+    for (int v = 0; v < ND; ++v) {
+      float d = 0.0f;
+#pragma unroll
+      for (int c = 0; c < NV; ++c) d = fmaf(L[v][c], D[c], d);
+      most = fmaxf(most, fabsf(d));
+      ok = ok && d == d;  // fmaxf drops a NaN
+      cv[v] = sgn == 0 ? corr[v] : cv[v] + corr[v];
+    }
+#pragma unroll
+    for (int t = 0; t < NS; ++t) {
+      const float d = fmaf(-vt[t], D[0], D[2 + t]);
+      most = fmaxf(most, fabsf(d));
+      cs[t] = sgn == 0 ? corrs[t] : cs[t] + corrs[t];
+    }
+  }
+  float P;
+  if constexpr (ORDER == 7)
+    P = fmaf(20.0f, m[3], fmaf(15.0f, m[2] + m[4], fmaf(6.0f, m[1] + m[5], m[0] + m[6])));
+  else
+    P = fmaf(6.0f, m[2], fmaf(4.0f, m[1] + m[3], m[0] + m[4]));
+  if constexpr (NV == 1) {
+    C[0] = cv[0];
+  } else {
+    // the fields in order: u-c, entropy, shear..., u+c
+#pragma unroll
+    for (int c = 0; c < NV; ++c) C[c] = 0.0f;
+    float Rc[NV];
+    right_col<NV, float>(E, 0, Rc);
+#pragma unroll
+    for (int c = 0; c < NV; ++c) C[c] = fmaf(Rc[c], cv[0], C[c]);
+    right_col<NV, float>(E, 1, Rc);
+#pragma unroll
+    for (int c = 0; c < NV; ++c) C[c] = fmaf(Rc[c], cv[1], C[c]);
+#pragma unroll
+    for (int t = 0; t < NS; ++t) {
+      C[2 + t] += cs[t];
+      C[NV - 1] = fmaf(vt[t], cs[t], C[NV - 1]);
+    }
+    right_col<NV, float>(E, NV - 1, Rc);
+#pragma unroll
+    for (int c = 0; c < NV; ++c) C[c] = fmaf(Rc[c], cv[ND - 1], C[c]);
+  }
+  return ok && fmaf(K * feps, P, most) <= limit;  // false for NaN
+}
+
 // The raw state of a tile staged in shared memory by TMA: conserved
 // component c of line a at extended cell e is p[c rc + a ra + (e + xoff) re]
 // (the layout of the copied box; xoff is the alignment slack of x boxes).
@@ -1076,8 +1324,169 @@ struct NoHook {
   __device__ __forceinline__ void operator()() const {}
 };
 
-// One tile of a sweep (phases 1-3 above).  alpha_d and dt are the splitting
-// constant of the swept axis and the step size; amax accumulates |u_d| + c of
+// What every tile of a stage's sweep shares: the splitting constant of the
+// swept axis, the step size, and what follows from them in the bulk precision
+// (made once, by one thread, and kept in shared memory: made per tile they
+// cost every thread conversions on the FP64 unit).
+template <typename R>
+struct TileConst {
+  double alpha_d, dt;
+  R alpha;
+  float dt32, wdt32;    // FP32 bulk combine: dt and the stage's weight of dt L
+  float limit;          // bound of prove_top
+};
+template <int ORDER, typename R>
+__device__ __forceinline__ void tile_const(const SweepArgs& A, double alpha_d, double dt,
+                                           TileConst<R>& k) {
+  k.alpha_d = alpha_d;
+  k.dt = dt;
+  k.alpha = (R)alpha_d;
+  k.dt32 = f32_rn(dt);
+  k.wdt32 = f32_rn((A.stage == 0 ? 1.0 : (A.stage == 1 ? 0.25 : 2.0 / 3.0)) * dt);
+  // below delta by more than the near-tie margin (and the bound's own rounding)
+  k.limit = A.delta_f - fmaf(A.tie_rel_f, A.delta_f, 1e-3f * A.delta_f);
+}
+
+// Whether the tile is the one that writes face f (the face between two tiles
+// belongs to the one on its right, the last face to the last).
+__device__ __forceinline__ bool owns_face(const SweepArgs& A, const TileGeo& g, int f) {
+  const long long gface = g.s0 + f;  // face index between cells gface-1 and gface
+  return (gface <= g.nd) && (f < A.ts || gface == g.nd);
+}
+// Index of face f of line a in the face arrays.
+__device__ __forceinline__ long long face_index(const TileGeo& g, int a, int f) {
+  return g.fbase + (g.a0 + a) * g.fstride_a + (g.s0 + f) * g.fstride_d;
+}
+
+// Phase 2 of one face: its correction C by projection and selection of every
+// field and sign; returns the choices that are near-ties (FP32 bulk).
+template <int NV, int ORDER, typename R, bool COHERENT, bool FIELD, int SHAPE>
+__device__ __forceinline__ unsigned choose_face(const SweepArgs& A, const TileGeo& g,
+                                                const TileView<NV, ORDER, R, FIELD>& tv,
+                                                const TileConst<R>& K, const int a, const int f) {
+  using CV = CellVec<NV, R, FIELD>;
+  constexpr int G = Geo<ORDER>::G;
+  constexpr bool FP32 = sizeof(R) == 4;
+  const StepState* st = A.st;
+  const int cells = tv.cells, mode = shape_mode<SHAPE>(A);
+  R* const dfm = tv.dfm;
+  R* const Cf = tv.Cf;
+  auto sidx = [&](int aa, int e) { return tv.sidx(aa, e); };
+  const R gm1 = bconst<R>(A.gm1, A.gm1_f);
+  const R delta = bconst<R>(A.delta, A.delta_f);
+  const R tie_rel = bconst<R>(A.tie_rel, A.tie_rel_f);
+  // splitting constant of field v: alpha, or per field max |u_d - c|, |u_d|, |u_d + c|
+  R alo = K.alpha, amid = K.alpha, ahi = K.alpha;
+  if constexpr (FIELD) {
+    alo = (R)st->alpha_f[A.dir][0];
+    amid = (R)st->alpha_f[A.dir][1];
+    ahi = (R)st->alpha_f[A.dir][2];
+  }
+  auto afield = [&](int v) { return v == 0 ? alo : (v == NV - 1 ? ahi : amid); };
+  const int j = G - 1 + f;  // face j+1/2 in extended cells
+  Eigen<NV, R> E;
+  if constexpr (NV > 1) face_eigen<NV, ORDER, R, FIELD>(tv, sidx(a, j), gm1, E);
+  const bool own = owns_face(A, g, f);
+  R C[NV];
+#pragma unroll
+  for (int c = 0; c < NV; ++c) C[c] = R(0);
+  unsigned fix = 0;
+#pragma unroll 1
+  for (int v = 0; v < NV; ++v) {
+    // shear fields (2D/3D Euler) have a sparse left row e_v - w e_0
+    const bool shear = NV >= 4 && v >= 2 && v <= NV - 2;
+    R L[NV], w = R(0);
+    if constexpr (NV > 1) {
+      left_row<NV, R>(E, v, L);
+      if constexpr (NV >= 4) w = -L[0];
+    } else {
+      L[0] = R(1);
+    }
+    // f^+ then mirrored f^- window, one live at a time
+    R cv = R(0);
+    const R av = afield(v);
+    if constexpr (FIELD) {
+      // the face's centre part: - alpha_v L dq/2 of the face's own pair
+      R xq[NV];
+      CV::load(dfm, cells, sidx(a, j), xq);
+      R aq = R(0);
+      if constexpr (NV >= 4) {
+        if (shear) aq = shear_comp<NV>(xq, v) - w * xq[0];
+      }
+      if (!shear) {
+#pragma unroll
+        for (int c = 0; c < NV; ++c) aq += L[c] * xq[c];
+      }
+      cv = -av * aq;
+    }
+#pragma unroll
+    for (int sgn = 0; sgn < 2; ++sgn) {
+      R d[8], mag[8];
+      tv.field_window(a, j, sgn, v, L, w, av, d, mag);
+      int pick;
+      bool marg = false;
+      R corr = eno_select<ORDER, R, FP32>(d, delta, tie_rel, mag, R(NV + 8) * R(FLT_EPSILON),
+                                          pick, marg);
+      if constexpr (FP32) {
+        if (marg) fix |= 1u << (v * 2 + sgn);  // re-decided in FP64 (phase 2b or the pass)
+      }
+      if ((mode & kModeFlux) && A.idx_out && own)
+        A.idx_out[(v * 2 + sgn) * A.nfaces + face_index(g, a, f)] = (int8_t)pick;
+      cv += corr;
+    }
+    if constexpr (NV >= 4) {
+      if (shear) {
+        // column v of R is e_v + w e_{NV-1}
+#pragma unroll
+        for (int c = 2; c < NV - 1; ++c) C[c] += c == v ? cv : R(0);
+        C[NV - 1] = fma(w, cv, C[NV - 1]);
+        continue;
+      }
+    }
+    if constexpr (NV > 1) {
+      R Rc[NV];
+      right_col<NV, R>(E, v, Rc);
+#pragma unroll
+      for (int c = 0; c < NV; ++c) C[c] = fma(Rc[c], cv, C[c]);
+    } else {
+      C[0] += cv;
+    }
+  }
+  CV::store(Cf, cells, sidx(a, j), C);
+  return fix;
+}
+
+// Phase 2 of the faces on the tile's list (FP32 bulk, kProve), one per
+// thread; their near-ties go into the list's entries.  Returns whether this
+// thread met one.
+template <int NV, int ORDER, bool COHERENT, int SHAPE>
+__device__ __forceinline__ bool listed_faces(const SweepArgs& A, const TileGeo& g,
+                                             unsigned char* smem_raw, const TileConst<float>& K,
+                                             int n) {
+  const TileView<NV, ORDER, float, false> tv(smem_raw, A.ta, A.se);
+  bool any = false;
+  for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    const unsigned entry = tv.list[i];
+    const unsigned fix = choose_face<NV, ORDER, float, COHERENT, false, SHAPE>(
+        A, g, tv, K, entry_line(entry), entry_face(entry));
+    if (fix) {
+      tv.list[i] = entry | fix;
+      any = true;
+    }
+  }
+  return any;
+}
+// The same out of line: most tiles have no such face, and the projection and
+// selection code then neither sets the register budget of the other phases nor
+// stands between them in the instruction cache.
+template <int NV, int ORDER, bool COHERENT, int SHAPE>
+__device__ __noinline__ bool listed_faces_call(const SweepArgs& A, const TileGeo& g,
+                                               unsigned char* smem_raw, const TileConst<float>& K,
+                                               int n) {
+  return listed_faces<NV, ORDER, COHERENT, SHAPE>(A, g, smem_raw, K, n);
+}
+
+// One tile of a sweep (phases 1-3 above).  amax accumulates |u_d| + c of
 // combined states (last stage), nfall counts FP64 re-decisions.  FIELD: each
 // characteristic field splits with its own constant (st->alpha_f): phase 1
 // keeps dF/2 and dq/2, the split follows the projection, and the face's
@@ -1089,26 +1498,20 @@ struct NoHook {
 // fixed field/sign order.  Out of line: only tiles with flagged choices call
 // it, and its FP64 code does not raise the register footprint of the common
 // path.  Ends with a block barrier.
-template <int NV, int ORDER, bool COHERENT, bool FIELD>
+template <int NV, int ORDER, bool COHERENT, bool FIELD, int SHAPE>
 __device__ __forceinline__ void redecide_tile(const SweepArgs& A, const TileGeo& g,
-                                              unsigned char* smem_raw, double alpha_d,
+                                              unsigned char* smem_raw, int nlist, double alpha_d,
                                               unsigned long long& nfall) {
   using R = float;
   using GE = Geo<ORDER>;
-  using CV = CellVec<NV, R>;
+  using CV = CellVec<NV, R, FIELD>;
   constexpr int G = GE::G;
   StepState* st = A.st;
-  const int TA = A.ta, SE = A.se;
-  const TileView<NV, ORDER, R, FIELD> tv(smem_raw, TA, SE);
+  const TileView<NV, ORDER, R, FIELD> tv(smem_raw, A.ta, A.se);
   R* Cf = tv.Cf;
-  R* prim = tv.prim;
-  unsigned* fixmask = tv.fixmask;
   const int cells = tv.cells;
-  auto sidx = [&](int a, int e) { return a * SE + e; };
-  const bool sfast = A.dir == 0;
-  const int lgTA = __ffs(TA) - 1;
-  const int nts = g.nts;
-  const int mode = A.mode;
+  auto sidx = [&](int a, int e) { return tv.sidx(a, e); };
+  const int mode = shape_mode<SHAPE>(A);
   const R gm1 = bconst<R>(A.gm1, A.gm1_f);
   const R delta = bconst<R>(A.delta, A.delta_f);
   const R tie_rel = bconst<R>(A.tie_rel, A.tie_rel_f);
@@ -1127,92 +1530,107 @@ __device__ __forceinline__ void redecide_tile(const SweepArgs& A, const TileGeo&
   auto field_window = [&](int a, int j, int sgn, int v, const R (&L)[NV], R w, R av, R (&d)[8],
                           R (&mag)[8]) { tv.field_window(a, j, sgn, v, L, w, av, d, mag); };
     constexpr int W = 2 * G <= 8 ? 8 : 16;  // lanes per re-decision group
+    constexpr int NG = 32 / W;
     const unsigned FULL = 0xffffffffu;
-    const int cnt = nts + 1;
     const int bd = blockDim.x, tid = threadIdx.x, lane = tid & 31;
-    int al, e0, estep;  // this thread's line, first face and face stride (as for_items)
-    if (sfast) {
-      const int lgTpl = __ffs(bd) - 1 - lgTA;
-      al = tid >> lgTpl;
-      e0 = tid & ((1 << lgTpl) - 1);
-      estep = 1 << lgTpl;
-    } else {
-      al = tid & (TA - 1);
-      e0 = tid >> lgTA;
-      estep = bd >> lgTA;
-    }
-    // estep is a power of two (blocks of 128 threads): no integer division,
-    // which runs partly on the FP64 unit
-    const int rounds = (cnt + estep - 1) >> (__ffs(estep) - 1);  // the same for every lane
-    for (int rd = 0; rd < rounds; ++rd) {
-      const int f = e0 + rd * estep;
-      const bool valid = f < cnt && g.a0 + al < g.na;
-      const int j = G - 1 + f;
-      unsigned fix = valid ? fixmask[sidx(al, j)] : 0u;
-      if (!__any_sync(FULL, fix != 0u)) continue;
-      // Re-decide every flagged choice of the warp: in each pass, group gi
-      // takes the lowest flagged choice of the gi-th lane that still has one,
-      // and that lane collects the result from group gi.  Every pass clears at
-      // least one of the at most 32 * 2 NV flags, so the default bound (64 NV
-      // passes) is never reached; a smaller bound (a test knob) can be: then
-      // the error word says so and the choices left keep their FP32 pick.
-      constexpr int NG = 32 / W;
-      unsigned todo = fix;
-      unsigned long long picks = 0ull;
-      // Many flags in the warp: each lane re-decides its own choices alone
-      // (as many rounds as the busiest lane has flags) instead of the warp
-      // serving NG choices per pass; a lone re-decision costs about 2.5x
-      // (ENO-AO5) or 3x (ENO-AO7) a cooperative pass.
-      const unsigned total = __reduce_add_sync(FULL, (unsigned)__popc(fix));
-      const unsigned most = __reduce_max_sync(FULL, (unsigned)__popc(fix));
-      if (most * (ORDER == 7 ? 6u : 5u) < 2u * ((total + NG - 1) / NG)) {
-        while (todo) {
-          const int kk = __ffs(todo) - 1;
-          todo &= todo - 1;
-          const int pick = redo_lane<NV, ORDER, COHERENT>(A, g, al, g.s0 + f - 1, kk >> 1, kk & 1,
-                                                          alpha64(kk >> 1));
-          picks |= (unsigned long long)pick << (4 * kk);
-          ++nfall;
-        }
+    // The flagged entries to the front of the list (one warp, in place: an
+    // entry never moves behind one not yet read), so that the choices of a
+    // warp's 32 faces below fill its lanes.
+    __shared__ int s_nflag;
+    if (tid < 32) {
+      int n = 0;
+      for (int base = 0; base < nlist; base += 32) {
+        const unsigned e = base + lane < nlist ? tv.list[base + lane] : 0u;
+        const unsigned m = __ballot_sync(FULL, entry_flags(e) != 0u);
+        if (entry_flags(e)) tv.list[n + __popc(m & ((1u << lane) - 1u))] = e;
+        n += __popc(m);
+        __syncwarp();
       }
-      const int pass_limit = A.redo_passes;
-      for (int pass = 0; pass <= pass_limit; ++pass) {
-        const unsigned have = __ballot_sync(FULL, todo != 0u);
-        if (!have) break;
-        if (pass == pass_limit) {
+      if (lane == 0) s_nflag = n;
+    }
+    __syncthreads();
+    const int nflag = s_nflag;
+    for (int base = tid - lane; base < nflag; base += bd) {  // the same for every lane
+      const unsigned entry = base + lane < nflag ? tv.list[base + lane] : 0u;
+      const int al = entry_line(entry), f = entry_face(entry);
+      const int j = G - 1 + f;
+      unsigned fix = entry_flags(entry);
+      // The warp's T choices in rounds.  Many left: one per lane (redo_lane),
+      // 32 in a round -- an instruction of the FP64 unit costs the same
+      // whatever its active lanes.  A few left: NG per round, each by W lanes
+      // together (redo_group), which takes about 2/5 (ENO-AO5) or 1/3 of the
+      // instructions of a lone re-decision.  Every round clears at least one
+      // choice, so the default bound (64 NV rounds) is never reached; a
+      // smaller bound (a test knob) can be: then the error word says so and
+      // the choices left keep their FP32 pick.
+      const int m = __popc(fix);
+      int pre = m;  // inclusive, then exclusive prefix sum over the lanes
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(FULL, pre, o);
+        if (lane >= o) pre += t;
+      }
+      const int T = __shfl_sync(FULL, pre, 31);
+      pre -= m;
+      unsigned long long picks = 0ull;
+      int done = 0;
+      for (int pass = 0; done < T; ++pass) {
+        if (pass >= A.redo_passes) {
           if (lane == 0) atomicOr(&st->err, kErrTimeout);
           break;
         }
-        const int src = nth_set_bit(have, lane / W);
-        const int srcl = src < 0 ? 0 : src;
-        const int k = __shfl_sync(FULL, todo ? __ffs(todo) - 1 : 0, srcl);
-        int ga = __shfl_sync(FULL, al, srcl);
-        int gf = __shfl_sync(FULL, f, srcl);
-        if (src < 0) {  // idle group: a valid face of the tile, result unused
-          ga = 0;
-          gf = 0;
+        const bool lone = T - done > (ORDER == 7 ? 3 : 2) * NG;
+        const int per = lone ? 32 : NG;
+        // this lane's (its group's) choice of the round: number ci, of the
+        // face of lane jl
+        const int ci = done + (lone ? lane : lane / W);
+        int jl = 0;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {  // the last lane whose first choice is <= ci
+          const int pq = __shfl_sync(FULL, pre, jl + o);
+          if (pq <= ci) jl += o;
         }
-        const int pick = redo_group<NV, ORDER, COHERENT, W>(A, g, ga, g.s0 + gf - 1, k >> 1, k & 1,
-                                                            alpha64(k >> 1), lane & (W - 1));
-        // my rank among the lanes with work tells which group (if any) took it
-        const int rank = __popc(have & ((1u << lane) - 1u));
-        const int mine = __shfl_sync(FULL, pick, (rank < NG ? rank : 0) * W);
-        if (todo != 0u && rank < NG) {
-          const int kk = __ffs(todo) - 1;
-          todo &= ~(1u << kk);
-          picks |= (unsigned long long)mine << (4 * kk);
-          ++nfall;
+        const unsigned mj = __shfl_sync(FULL, fix, jl);
+        const int prej = __shfl_sync(FULL, pre, jl);
+        const int aj = __shfl_sync(FULL, al, jl), fj = __shfl_sync(FULL, f, jl);
+        const bool valid = ci < T;
+        const int kb = valid ? nth_set_bit(mj, ci - prej) : 0;
+        // (a group without a choice works on the face of the last one, unused)
+        const int k = kb < 0 ? 0 : kb;
+        int pick = 0;
+        if (lone) {
+          if (valid)
+            pick = redo_lane<NV, ORDER, COHERENT>(A, g, aj, g.s0 + fj - 1, k >> 1, k & 1,
+                                                  alpha64(k >> 1));
+        } else {
+          pick = redo_group<NV, ORDER, COHERENT, W>(A, g, aj, g.s0 + fj - 1, k >> 1, k & 1,
+                                                    alpha64(k >> 1), lane & (W - 1));
         }
+        __syncwarp();
+        // each face's lane collects its choices of the round
+        unsigned todo = fix;
+        int most = __reduce_max_sync(FULL, (unsigned)m);
+        for (int t = 0; t < most; ++t) {
+          const int c = pre + t - done;
+          const int src = c >= 0 && c < per ? (lone ? c : c * W) : 0;
+          const int got = __shfl_sync(FULL, pick, src);
+          const int kk = todo ? __ffs(todo) - 1 : 0;
+          todo &= todo - 1;
+          if (t < m && c >= 0 && c < per) {
+            picks |= (unsigned long long)got << (4 * kk);
+            ++nfall;
+          }
+        }
+        done += per;
       }
-      fix &= ~todo;  // choices left by a pass bound keep their FP32 pick
+      // choices left by a pass bound keep their FP32 pick
+      const int have = done - pre < 0 ? 0 : (done - pre < m ? done - pre : m);
+      for (int t = m; t > have; --t) fix &= ~(1u << (31 - __clz(fix)));
       if (!fix) continue;
       // apply the changed choices of this face
       Eigen<NV, R> E;
       if constexpr (NV > 1) {
-        R pl[NV], prr[NV];
-        CV::load(prim, cells, sidx(al, j), pl);
-        CV::load(prim, cells, sidx(al, j + 1), prr);
-        roe_eigen<NV, R>(pl, prr, gm1, E);
+        face_eigen<NV, ORDER, R, FIELD>(tv, sidx(al, j), gm1, E);
       }
       const long long gface = g.s0 + f;
       const bool own = (gface <= g.nd) && (f < A.ts || gface == g.nd);
@@ -1241,17 +1659,17 @@ __device__ __forceinline__ void redecide_tile(const SweepArgs& A, const TileGeo&
         if (pick != pick_old) {
           R corr = R(0);
 #pragma unroll
-          for (int i = GE::LO; i <= GE::HI; ++i) corr += bcoef<R>(pick, i) * d[i];
+          for (int i = GE::LO; i <= GE::HI; ++i) corr = fma(bcoef<R>(pick, i), d[i], corr);
           const R dv = corr - corr_old;
           if (shear) {
 #pragma unroll
             for (int c = 2; c < NV - 1; ++c) dC[c] += c == v ? dv : R(0);
-            dC[NV - 1] += w * dv;
+            dC[NV - 1] = fma(w, dv, dC[NV - 1]);
           } else if constexpr (NV > 1) {
             R Rc[NV];
             right_col<NV, R>(E, v, Rc);
 #pragma unroll
-            for (int c = 0; c < NV; ++c) dC[c] += Rc[c] * dv;
+            for (int c = 0; c < NV; ++c) dC[c] = fma(Rc[c], dv, dC[c]);
           } else {
             dC[0] += dv;
           }
@@ -1275,20 +1693,20 @@ __device__ __forceinline__ void redecide_tile(const SweepArgs& A, const TileGeo&
 // The same, not inlined (only one copy of the code, called by the tiles that
 // have flags): where the FP64 re-decision code would otherwise set the
 // register budget of the whole tile.
-template <int NV, int ORDER, bool COHERENT, bool FIELD>
+template <int NV, int ORDER, bool COHERENT, bool FIELD, int SHAPE>
 __device__ __noinline__ void redecide_tile_call(const SweepArgs& A, const TileGeo& g,
-                                                unsigned char* smem_raw, double alpha_d,
+                                                unsigned char* smem_raw, int nlist, double alpha_d,
                                                 unsigned long long& nfall) {
-  redecide_tile<NV, ORDER, COHERENT, FIELD>(A, g, smem_raw, alpha_d, nfall);
+  redecide_tile<NV, ORDER, COHERENT, FIELD, SHAPE>(A, g, smem_raw, nlist, alpha_d, nfall);
 }
 
-// TMA: phase 1 reads the tile's raw state from rt instead of global memory,
-// and hook() runs once every thread is past phase 1 (the raw buffer is then
-// free for the next tile's copy).
+// TMA: phase 1 reads the tile's raw state from rt instead of global memory.
+// hook() runs before the tile's last barrier, with TMA once every thread is
+// past phase 1 (the raw buffer is then free for the next tile's copy).
 template <int NV, int ORDER, typename R, bool COHERENT = false, bool DEFER = false,
-          bool FIELD = false, bool TMA = false, typename Hook = NoHook, bool LEAN = false>
+          bool FIELD = false, bool TMA = false, int SHAPE = kShapeAny, typename Hook = NoHook>
 __device__ __forceinline__ void sweep_tile(const SweepArgs& A, const TileGeo& g,
-                                           unsigned char* smem_raw, double alpha_d, double dt,
+                                           unsigned char* smem_raw, const TileConst<R>& K,
                                            double (&amax)[kAmax<FIELD>],
                                            unsigned long long& nfall, const RawTile& rt = RawTile{},
                                            Hook hook = Hook{}) {
@@ -1296,21 +1714,27 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& A, const TileGeo& g,
   using GE = Geo<ORDER>;
   constexpr int G = GE::G;
   constexpr bool FP32 = sizeof(R) == 4;
-  constexpr int NP = NPrim<NV>::value;
+  constexpr bool PROVE = kProve<R, FIELD>;
+  // the code of faces not proven and of near-ties out of line
+  constexpr bool CALL = PROVE && SHAPE != kShapeAny && !COHERENT;
   StepState* st = A.st;
   const int TA = A.ta, TS = A.ts;
-  const int SE = A.se;  // row pitch (>= TS + 2G), chosen on the host for conflict-free banks
-  const int cells = TA * SE;
-  R* dfp = reinterpret_cast<R*>(smem_raw);
-  R* dfm = dfp + NV * cells;
-  R* Cf = dfm + NV * cells;
-  R* prim = Cf + NV * cells;
-  // FP32 only: near-tie flags per face (one word per cell slot)
-  unsigned* fixmask = reinterpret_cast<unsigned*>(prim + NP * cells);
+  // row pitch A.se (>= TS + 2G), chosen on the host for conflict-free banks
+  const TileView<NV, ORDER, R, FIELD> tv(smem_raw, TA, A.se);
+  const int cells = tv.cells;
+  R* const dfp = tv.dfp;
+  R* const dfm = tv.dfm;
+  R* const Cf = tv.Cf;
+  R* const prim = tv.prim;
+  // FP32 bulk: faces on the tile's list (those not proven in phase 2a, or
+  // all with flagged choices)
+  __shared__ int s_nlist;
+  if (FP32 && threadIdx.x == 0) s_nlist = 0;
 
   const int dir = A.dir;
-  const bool sfast = dir == 0;
-  const R alpha = (R)alpha_d;
+  const bool sfast = shape_x<SHAPE>(A);
+  const double alpha_d = K.alpha_d, dt = K.dt;
+  const R alpha = K.alpha;
   const R halpha = R(0.5) * alpha;
   // splitting constant of field v: alpha, or per field max |u_d - c|, |u_d|, |u_d + c|
   R alo = alpha, amid = alpha, ahi = alpha;
@@ -1329,27 +1753,30 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& A, const TileGeo& g,
   const R adv = bconst<R>(A.adv_speed, A.adv_f);
   const R delta = bconst<R>(A.delta, A.delta_f);
   const R tie_rel = bconst<R>(A.tie_rel, A.tie_rel_f);
-  const int mode = A.mode;
+  const int mode = shape_mode<SHAPE>(A);
   const double inv_dx = A.inv_dx;
   const R inv_dx_r = bconst<R>(inv_dx, A.inv_dx_f);
   // FP32 bulk combine: dt and the stage's weight of dt L in FP32
-  const float dt32 = f32_rn(dt);
-  const float wdt32 = f32_rn((A.stage == 0 ? 1.0 : (A.stage == 1 ? 0.25 : 2.0 / 3.0)) * dt);
+  const float dt32 = K.dt32, wdt32 = K.wdt32;
   const float inc_w = A.stage == 1 ? -0.75f : -f32_rn(1.0 / 12.0);  // weight of the carried increment
   // Shared-memory rows of SE cells per line for every axis: unit stride
   // along the swept axis (window offsets are immediates); SE is odd, so the
   // y/z sweeps, whose lanes run across lines, hit distinct banks.
-  auto sidx = [&](int a, int e) { return a * SE + e; };
-  using CV = CellVec<NV, R>;
+  auto sidx = [&](int a, int e) { return tv.sidx(a, e); };
+  using CV = CellVec<NV, R, FIELD>;
   const int lgTA = __ffs(TA) - 1;  // TA is a power of two (checked on the host)
   (void)TS;
-  const TileView<NV, ORDER, R, FIELD> tv(smem_raw, TA, SE);
   // Projected window of field v (the same arithmetic in phase 2 and in the
   // phase-2b check of a flagged choice, which must reproduce its pick).
   auto field_window = [&](int a, int j, int sgn, int v, const R (&L)[NV], R w, R av, R (&d)[8],
                           R (&mag)[8]) { tv.field_window(a, j, sgn, v, L, w, av, d, mag); };
   const int nts = g.nts;
   const int sext = nts + 2 * G;  // extended cells in use
+  // extended cell e of line a is cell ext0 + a sa + e sd, except ghosts of a
+  // tile at the end of its lines
+  const bool edge = A.bc != kBcHalo && (g.s0 < G || g.s0 + nts + G > g.nd);
+  const cell_t<NV> sa = g.stride_a, sd = g.stride_d;
+  const cell_t<NV> ext0 = g.base + g.a0 * g.stride_a + (g.s0 - G) * g.stride_d;
 
   // ---------------- phase 1: split differences and Roe ingredients
   {
@@ -1361,30 +1788,43 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& A, const TileGeo& g,
 #pragma unroll
         for (int c = 0; c < NV; ++c) q[c] = p[perm_comp<NV>(c, dir) * rt.rc];
       } else {
-        const long long la = g.base + (g.a0 + a) * g.stride_a;
-        load_state<NV, COHERENT>(A.u_in, A.cstride,
-                                 la + bc_map(g.s0 - G + ee, g.nd, A.bc) * g.stride_d, dir, q);
+        cell_t<NV> cell = ext0 + (cell_t<NV>)a * sa + (cell_t<NV>)ee * sd;
+        if (edge)
+          cell = g.base + (g.a0 + a) * g.stride_a + bc_map(g.s0 - G + ee, g.nd, A.bc) * g.stride_d;
+        load_state<NV, COHERENT>(A, cell, q);
       }
     };
     // cell e's Roe ingredients, and the split differences of the pair (e, e+1)
     auto prim_out = [&](int a, int e, const R (&qa)[NV]) {
-      if constexpr (NP > 0) {
+      if constexpr (NV > 1) {
         if (e >= G - 1 && e <= G + nts) {
           R pr[NV];
           roe_prims<NV, R>(qa, gm1, pr);
-          CV::store(prim, cells, sidx(a, e), pr);
+          if constexpr (CV::kSpare) {
+            dfm[4 * sidx(a, e) + 3] = pr[0];
+            Cf[4 * sidx(a, e) + 3] = pr[1];
+            prim[sidx(a, e)] = pr[2];
+          } else {
+            CV::store(prim, cells, sidx(a, e), pr);
+          }
         }
       }
     };
     auto pair_out = [&](int a, int e, const double (&qa64)[NV], const R (&qa)[NV],
                         const double (&qb64)[NV], const R (&qb)[NV]) {
-      R fp[NV], fm[NV];
+      R fp[NV], fm[NV], m = R(0);
       if constexpr (FIELD)
         split_parts<NV, R>(qa64, qb64, qa, qb, gm1, adv, fp, fm);  // dF/2, dq/2
       else
-        split_diff<NV, R>(qa64, qb64, qa, qb, gm1, adv, halpha, fp, fm);
-      CV::store(dfp, cells, sidx(a, e), fp);
-      CV::store(dfm, cells, sidx(a, e), fm);
+        m = split_diff<NV, R>(qa64, qb64, qa, qb, gm1, adv, halpha, fp, fm);
+      if constexpr (CV::kSpare) {
+        CV::store4(dfp, sidx(a, e), fp, m);
+        CV::store(dfm, cells, sidx(a, e), fm);  // its spare value: a Roe ingredient
+      } else {
+        CV::store(dfp, cells, sidx(a, e), fp);
+        CV::store(dfm, cells, sidx(a, e), fm);
+        if constexpr (PROVE) tv.mag[sidx(a, e)] = m;
+      }
     };
     if (sfast) {
       // x sweeps: lanes along the line (coalesced), one pair per item
@@ -1412,7 +1852,7 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& A, const TileGeo& g,
       // left cell of the next), the run's last pair reaching one cell on
       int a, j0, step;
       item_start(lgTA, false, a, j0, step);
-      const int run = (cnt + step - 1) / step;
+      const int run = (cnt + step - 1) >> (__ffs(step) - 1);  // step is a power of two
       int e = j0 * run;
       const int e_end = min(e + run, cnt);
       if (g.a0 + a < g.na && e < e_end) {
@@ -1441,131 +1881,83 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& A, const TileGeo& g,
     }
   }
   __syncthreads();
-  hook();
+  if constexpr (TMA) hook();
 
-  // ---------------- phase 2: per face choice and back-projection
+  // ---------------- phase 2a (FP32 bulk): prove the smooth faces, list the others
+  const int nfaces_tile = nts + 1;
   bool any_fix = false;  // FP32 bulk: this thread flagged a near-tie
-  {
-    const int cnt = nts + 1;
-    for_items(lgTA, cnt, sfast, [&](const int a, const int f) {
+  if constexpr (PROVE) {
+    for_items(lgTA, nfaces_tile, sfast, [&](const int a, const int f) {
       if (g.a0 + a >= g.na) return;
-      const int j = G - 1 + f;  // face j+1/2 in extended cells
-      Eigen<NV, R> E;
-      if constexpr (NV > 1) {
-        R pl[NV], prr[NV];
-        CV::load(prim, cells, sidx(a, j), pl);
-        CV::load(prim, cells, sidx(a, j + 1), prr);
-        roe_eigen<NV, R>(pl, prr, gm1, E);
-      }
-      const long long gface = g.s0 + f;  // face index between cells gface-1 and gface
-      const bool own = (gface <= g.nd) && (f < A.ts || gface == g.nd);
+      const int x = sidx(a, G - 1 + f);
       R C[NV];
-#pragma unroll
-      for (int c = 0; c < NV; ++c) C[c] = R(0);
-      unsigned fix = 0;
-#pragma unroll 1
-      for (int v = 0; v < NV; ++v) {
-        // shear fields (2D/3D Euler) have a sparse left row e_v - w e_0
-        const bool shear = NV >= 4 && v >= 2 && v <= NV - 2;
-        R L[NV], w = R(0);
-        if constexpr (NV > 1) {
-          left_row<NV, R>(E, v, L);
-          if constexpr (NV >= 4) w = -L[0];
-        } else {
-          L[0] = R(1);
+      if (prove_top<NV, ORDER, FIELD>(tv, x, gm1, K.limit, C)) {
+        CV::store(Cf, cells, x, C);
+        if ((mode & kModeFlux) && A.idx_out && owns_face(A, g, f)) {
+          const long long fc = face_index(g, a, f);
+          for (int k = 0; k < 2 * NV; ++k) A.idx_out[k * A.nfaces + fc] = (int8_t)(GE::NC - 1);
         }
-        // f^+ then mirrored f^- window, one live at a time
-        R cv = R(0);
-        const R av = afield(v);
-        if constexpr (FIELD) {
-          // the face's centre part: - alpha_v L dq/2 of the face's own pair
-          R xq[NV];
-          CV::load(dfm, cells, sidx(a, j), xq);
-          R aq = R(0);
-          if constexpr (NV >= 4) {
-            if (shear) aq = shear_comp<NV>(xq, v) - w * xq[0];
-          }
-          if (!shear) {
-#pragma unroll
-            for (int c = 0; c < NV; ++c) aq += L[c] * xq[c];
-          }
-          cv = -av * aq;
-        }
-#pragma unroll
-        for (int sgn = 0; sgn < 2; ++sgn) {
-          R d[8], mag[8];
-          field_window(a, j, sgn, v, L, w, av, d, mag);
-          int pick;
-          bool marg = false;
-          R corr = eno_select<ORDER, R, FP32>(d, delta, tie_rel, mag, R(NV + 8) * R(FLT_EPSILON),
-                                              pick, marg);
-          if constexpr (FP32) {
-            if (marg) fix |= 1u << (v * 2 + sgn);  // re-decided in FP64 (phase 2b or the pass)
-          }
-          if ((mode & kModeFlux) && A.idx_out && own) {
-            const long long nf = A.nfaces;
-            const long long fc = g.fbase + (g.a0 + a) * g.fstride_a + gface * g.fstride_d;
-            A.idx_out[(v * 2 + sgn) * nf + fc] = (int8_t)pick;
-          }
-          cv += corr;
-        }
-        if constexpr (NV >= 4) {
-          if (shear) {
-            // column v of R is e_v + w e_{NV-1}
-#pragma unroll
-            for (int c = 2; c < NV - 1; ++c) C[c] += c == v ? cv : R(0);
-            C[NV - 1] += w * cv;
-            continue;
-          }
-        }
-        if constexpr (NV > 1) {
-          R Rc[NV];
-          right_col<NV, R>(E, v, Rc);
-#pragma unroll
-          for (int c = 0; c < NV; ++c) C[c] += Rc[c] * cv;
-        } else {
-          C[0] += cv;
-        }
-      }
-      const int sj = sidx(a, j);
-      CV::store(Cf, cells, sj, C);
-      if constexpr (FP32) {
-        fixmask[sj] = fix;
-        any_fix |= fix != 0u;
+      } else {
+        tv.list[atomicAdd(&s_nlist, 1)] = face_entry(a, f);
       }
     });
+    __syncthreads();
   }
-  if constexpr (!(FP32 && !DEFER)) __syncthreads();  // else the barrier of phase 2b's test
 
-  // ---------------- phase 2b (FP32 bulk, re-decision list): list the faces
-  // with flagged choices that this tile owns; the grid-wide pass corrects both
-  // cells of each, whichever tiles they lie in, so results do not depend on
-  // tiles.  Nothing here changes Cf: phase 3 uses the FP32 choices.
-  if constexpr (FP32 && DEFER) {
-    for_items(lgTA, nts + 1, sfast, [&](const int a, const int f) {
-      if (g.a0 + a >= g.na) return;
-      const unsigned fix = fixmask[sidx(a, G - 1 + f)];
-      const long long gface = g.s0 + f;
-      if (!fix || !((gface <= g.nd) && (f < A.ts || gface == g.nd))) return;
+  // ---------------- phase 2: per face choice and back-projection
+  {
+    if constexpr (PROVE) {
+      if (s_nlist > 0) {
+        if constexpr (CALL)
+          any_fix = listed_faces_call<NV, ORDER, COHERENT, SHAPE>(A, g, smem_raw, K, s_nlist);
+        else
+          any_fix = listed_faces<NV, ORDER, COHERENT, SHAPE>(A, g, smem_raw, K, s_nlist);
+      }
+    } else {
+      for_items(lgTA, nfaces_tile, sfast, [&](const int a, const int f) {
+        if (g.a0 + a >= g.na) return;
+        const unsigned fix = choose_face<NV, ORDER, R, COHERENT, FIELD, SHAPE>(A, g, tv, K, a, f);
+        if constexpr (FP32) {
+          if (fix) {
+            tv.list[atomicAdd(&s_nlist, 1)] = face_entry(a, f) | fix;
+            any_fix = true;
+          }
+        }
+      });
+    }
+  }
+
+  // ---------------- phase 2b (FP32 bulk): the faces with flagged choices
+  if constexpr (!FP32) {
+    __syncthreads();
+  } else if (PROVE && s_nlist == 0) {
+    // every face proven: C is complete since the barrier of phase 2a
+  } else if constexpr (DEFER) {
+    // list the faces that this tile owns for the grid-wide pass, which
+    // corrects both cells of each, whichever tiles they lie in, so results do
+    // not depend on tiles.  Nothing here changes Cf: phase 3 uses the FP32
+    // choices.
+    __syncthreads();
+    const int n = s_nlist;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+      const unsigned entry = tv.list[i], fix = entry_flags(entry);
+      if (!fix || !owns_face(A, g, entry_face(entry))) continue;
       const unsigned slot = atomicAdd(&st->redo_n, 1u);
       if (slot < A.redo_cap) {
-        const long long fc = g.fbase + (g.a0 + a) * g.fstride_a + gface * g.fstride_d;
+        const long long fc = face_index(g, entry_line(entry), entry_face(entry));
         A.redo[slot] = ((unsigned long long)fc << 16) | fix;
       } else {
         atomicOr(&st->err, kErrRedoFull);
       }
-    });
-  }
-
-  // ---------------- phase 2b (FP32 bulk, no list): FP64 re-decision of near-ties
-  // Only tiles with flagged choices run it.  LEAN kernels call it out of line,
-  // so that its FP64 code does not set the register budget of every tile.
-  if constexpr (FP32 && !DEFER) {
+    }
+  } else {
+    // FP64 re-decision of the tile's near-ties; only tiles with flagged
+    // choices run it.
     if (__syncthreads_or(any_fix)) {
-      if constexpr (LEAN)
-        redecide_tile_call<NV, ORDER, COHERENT, FIELD>(A, g, smem_raw, alpha_d, nfall);
+      if constexpr (CALL)
+        redecide_tile_call<NV, ORDER, COHERENT, FIELD, SHAPE>(A, g, smem_raw, s_nlist, alpha_d, nfall);
       else
-        redecide_tile<NV, ORDER, COHERENT, FIELD>(A, g, smem_raw, alpha_d, nfall);
+        redecide_tile<NV, ORDER, COHERENT, FIELD, SHAPE>(A, g, smem_raw, s_nlist, alpha_d, nfall);
     }
   }
 
@@ -1580,8 +1972,8 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& A, const TileGeo& g,
       const int j = G - 1 + f;
       const long long la = g.base + (g.a0 + a) * g.stride_a;
       double ql[NV], qr[NV], Fl[NV], Fr[NV];
-      load_state<NV, COHERENT>(A.u_in, A.cstride, la + bc_map(gface - 1, g.nd, A.bc) * g.stride_d, dir, ql);
-      load_state<NV, COHERENT>(A.u_in, A.cstride, la + bc_map(gface, g.nd, A.bc) * g.stride_d, dir, qr);
+      load_state<NV, COHERENT>(A, la + bc_map(gface - 1, g.nd, A.bc) * g.stride_d, ql);
+      load_state<NV, COHERENT>(A, la + bc_map(gface, g.nd, A.bc) * g.stride_d, qr);
       phys_flux<NV>(ql, A.gm1, A.adv_speed, Fl);
       phys_flux<NV>(qr, A.gm1, A.adv_speed, Fr);
       const long long fc = g.fbase + (g.a0 + a) * g.fstride_a + gface * g.fstride_d;
@@ -1604,7 +1996,7 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& A, const TileGeo& g,
     for_items(lgTA, cnt, sfast, [&](const int a, const int t) {
       if (g.a0 + a >= g.na) return;
       const int e = G + t;
-      const long long cell = g.base + (g.a0 + a) * g.stride_a + (g.s0 + t) * g.stride_d;
+      const cell_t<NV> cell = ext0 + (cell_t<NV>)a * sa + (cell_t<NV>)e * sd;
       R r[NV];
       {
         R p0[NV], m1[NV], c1[NV], c0[NV];
@@ -1616,78 +2008,97 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& A, const TileGeo& g,
 #pragma unroll
         for (int c = 0; c < NV; ++c) {
           const R s = p0[c] + m1[c] + (c1[c] - c0[c]);
-          r[c] = -s * inv_dx_r;
+          r[c] = mul_rn(-s, inv_dx_r);
         }
       }
-      // Every store of the cell comes after all its loads: the stores could
-      // alias the inputs as far as the compiler knows, so a load after a
-      // store would wait for it (one memory round trip per component).
-      if (!(mode & kModeCombine)) {
-        R* rb = reinterpret_cast<R*>(A.rhs);
-        R v[NV];
+      // Every load of the cell comes first, each array's under one uniform
+      // condition, so that all are in flight together; the stores follow (they
+      // could alias the inputs as far as the compiler knows, and a load after
+      // one would wait for it).
+      const bool add = mode & kModeRhsAdd, combine = mode & kModeCombine;
+      R o[NV];         // L(u) of the earlier axes
+      double ui[NV];   // the stage's input
+      float I[NV];     // FP32 bulk: the increment of the stage before
+      double u0[NV];   // FP64: U^n
+      if (add) {
+#pragma unroll
+        for (int c = 0; c < NV; ++c) o[c] = static_cast<const R*>(A.comp.rhs[c])[cell];
+      }
+      if (combine) {
+        // (the batched kernel reads stage states it wrote itself: through L2)
 #pragma unroll
         for (int c = 0; c < NV; ++c) {
-          const long long k = perm_comp<NV>(c, dir) * A.cstride + cell;
-          v[c] = (mode & kModeRhsAdd) ? rb[k] + r[c] : r[c];
+          const double* p = A.comp.u_in[c] + cell;
+          ui[c] = COHERENT ? __ldcg(p) : __ldg(p);
         }
+        if (A.stage > 0) {
 #pragma unroll
-        for (int c = 0; c < NV; ++c) rb[perm_comp<NV>(c, dir) * A.cstride + cell] = v[c];
+          for (int c = 0; c < NV; ++c) {
+            if constexpr (FP32) {
+              const float* p = A.comp.inc_in[c] + cell;
+              I[c] = COHERENT ? __ldcg(p) : __ldg(p);
+            } else {
+              const double* p = A.comp.u0[c] + cell;
+              u0[c] = COHERENT ? __ldcg(p) : __ldg(p);
+            }
+          }
+        }
+      }
+      // L(u) summed over the axes in the bulk precision
+      if (add) {
+#pragma unroll
+        for (int c = 0; c < NV; ++c) r[c] = o[c] + r[c];
+      }
+      if (!combine) {
+#pragma unroll
+        for (int c = 0; c < NV; ++c) static_cast<R*>(A.comp.rhs[c])[cell] = r[c];
         return;
       }
-      auto u0v = [&](const double* p) { return COHERENT ? __ldcg(p) : __ldg(p); };
       double up[NV], unew[NV];
       float inc[NV];  // FP32 bulk: the increment this stage carries on
+      if constexpr (FP32) {
+        // Each stage as its own input u_i plus an FP32 increment, the step's
+        // increments so far carried in FP32 (each is dt times an FP32-bulk
+        // L(u)): with I0 = dt L(u0) and I1 = I0 + dt L(u1),
+        //   u1 = u0 + I0
+        //   u2 = u1 + (1/4 dt L(u1) - 3/4 I0)
+        //   u3 = u2 + (2/3 dt L(u2) - 1/12 I1),
+        // which are 3/4 u0 + 1/4 (u1 + dt L(u1)) and 1/3 u0 + 2/3 (u2 +
+        // dt L(u2)) because u1 - u0 = I0 and u2 - u0 = I1 / 4 (up to FP64
+        // rounding of u1 and u2).  One FP64 add per component (the FP64 unit
+        // runs at 1/64 of the FP32 rate) and no read of U^n: the increments
+        // take the bytes U^n took, and u_i was just read by phase 1.
+        if (A.stage > 0) {
 #pragma unroll
-      for (int c = 0; c < NV; ++c) {
-        const long long k = perm_comp<NV>(c, dir) * A.cstride + cell;
-        // L(u) summed over the axes in the bulk precision, then one rounding
-        // to FP64 for the Runge-Kutta combine
-        R Lsum = r[c];
-        if (mode & kModeRhsAdd) Lsum = reinterpret_cast<const R*>(A.rhs)[k] + r[c];
-        // (the batched kernel reads stage states it wrote itself: through L2)
-        const double ui = COHERENT ? __ldcg(A.u_in + k) : __ldg(A.u_in + k);
-        const double* u0p = A.u0 + k;
-        double un;
-        if constexpr (FP32) {
-          // Each stage as its own input u_i plus an FP32 increment, the
-          // step's increments so far carried in FP32 (each is dt times an
-          // FP32-bulk L(u)): with I0 = dt L(u0) and I1 = I0 + dt L(u1),
-          //   u1 = u0 + I0
-          //   u2 = u1 + (1/4 dt L(u1) - 3/4 I0)
-          //   u3 = u2 + (2/3 dt L(u2) - 1/12 I1),
-          // which are 3/4 u0 + 1/4 (u1 + dt L(u1)) and 1/3 u0 + 2/3 (u2 +
-          // dt L(u2)) because u1 - u0 = I0 and u2 - u0 = I1 / 4 (up to FP64
-          // rounding of u1 and u2).  One FP64 add per component (the FP64
-          // unit runs at 1/64 of the FP32 rate) and no read of U^n: the
-          // increments take the bytes U^n took, and u_i was just read by
-          // phase 1.
-          float t = wdt32 * Lsum;
-          if (A.stage > 0) {
-            const float I = COHERENT ? __ldcg(A.inc_in + k) : __ldg(A.inc_in + k);
-            inc[c] = fmaf(dt32, Lsum, I);  // I1 (stored by stage 1 only)
-            t = fmaf(inc_w, I, t);
-          } else {
-            inc[c] = t;  // I0
+          for (int c = 0; c < NV; ++c) {
+            inc[c] = fmaf(dt32, r[c], I[c]);  // I1 (stored by stage 1 only)
+            up[c] = ui[c] + f64_of(fmaf(inc_w, I[c], wdt32 * r[c]));
           }
-          un = ui + f64_of(t);
         } else {
-          const double Lk = to_f64(Lsum);
-          if (A.stage == 0) {
-            un = ui + dt * Lk;
-          } else if (A.stage == 1) {
-            un = 0.75 * u0v(u0p) + 0.25 * (ui + dt * Lk);
-          } else {
-            un = (1.0 / 3.0) * u0v(u0p) + (2.0 / 3.0) * (ui + dt * Lk);
+#pragma unroll
+          for (int c = 0; c < NV; ++c) {
+            inc[c] = wdt32 * r[c];  // I0
+            up[c] = ui[c] + f64_of(inc[c]);
           }
         }
-        up[c] = un;
+      } else {
+#pragma unroll
+        for (int c = 0; c < NV; ++c) {
+          const double Lk = to_f64(r[c]);
+          if (A.stage == 0)
+            up[c] = ui[c] + dt * Lk;
+          else if (A.stage == 1)
+            up[c] = 0.75 * u0[c] + 0.25 * (ui[c] + dt * Lk);
+          else
+            up[c] = (1.0 / 3.0) * u0[c] + (2.0 / 3.0) * (ui[c] + dt * Lk);
+        }
       }
 #pragma unroll
-      for (int c = 0; c < NV; ++c) A.u_out[perm_comp<NV>(c, dir) * A.cstride + cell] = up[c];
+      for (int c = 0; c < NV; ++c) A.comp.u_out[c][cell] = up[c];
       if constexpr (FP32) {
         if (A.stage < 2) {
 #pragma unroll
-          for (int c = 0; c < NV; ++c) A.inc_out[perm_comp<NV>(c, dir) * A.cstride + cell] = inc[c];
+          for (int c = 0; c < NV; ++c) A.comp.inc_out[c][cell] = inc[c];
         }
       }
 #pragma unroll
@@ -1712,35 +2123,22 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& A, const TileGeo& g,
       }
     });
   }
+  if constexpr (!TMA) hook();
   __syncthreads();
 }
 
 // Minimum resident blocks per SM asked of the compiler for the FP32-bulk
-// sweep (caps its registers at 65536 / (128 * min blocks)): the sweep is
-// latency-bound, so six blocks (80 registers, a few spilled) beat four
-// without spills for ENO-AO5; ENO-AO7 keeps more live values and takes five.
-#ifndef ENOAO_FP32_MIN_BLOCKS_AO5
-#define ENOAO_FP32_MIN_BLOCKS_AO5 6
-#endif
-#ifndef ENOAO_FP32_MIN_BLOCKS_AO7
-#define ENOAO_FP32_MIN_BLOCKS_AO7 5
+// sweep (caps its registers at 65536 / (128 * min blocks)).
+#ifndef ENOAO_FP32_MIN_BLOCKS
+#define ENOAO_FP32_MIN_BLOCKS 8
 #endif
 // Per-field splitting keeps two projections per window cell live and takes
-// four blocks (128 registers).
-// With a TMA-staged raw tile a block needs more shared memory, and four of
-// them fill an SM: they get the registers (128, no spills; at 96 the
-// thread-0 copy issue spills).
-// LEAN (ENO-AO5 in-sweep re-decision, re-decisions out of line): 64
-// registers (no more spills than at 72), for tiles whose shared memory lets
-// seven or eight blocks share an SM.
-template <int ORDER, typename R, bool FIELD = false, bool TMA = false, bool LEAN = false>
+// four blocks (128 registers).  With a TMA-staged raw tile a block needs more
+// shared memory, and four of them fill an SM: they get the registers (128, no
+// spills; at 96 the thread-0 copy issue spills).
+template <typename R, bool FIELD = false, bool TMA = false>
 constexpr int sweep_min_blocks() {
-  return sizeof(R) == 8 ? 1
-                        : (FIELD ? 4
-                                 : (TMA ? 4
-                                        : (LEAN ? 8
-                                                : (ORDER == 5 ? ENOAO_FP32_MIN_BLOCKS_AO5
-                                                              : ENOAO_FP32_MIN_BLOCKS_AO7))));
+  return sizeof(R) == 8 ? 1 : (FIELD || TMA ? 4 : ENOAO_FP32_MIN_BLOCKS);
 }
 
 // Bound on the polls of a TMA completion barrier (a copy of a few tens of KB
@@ -1818,36 +2216,49 @@ __device__ __forceinline__ void sweep_epilogue(const SweepArgs& A, double (&amax
 }
 
 template <int NV, int ORDER, typename R, bool DEFER = false, bool FIELD = false, bool TMA = false,
-          bool LEAN = false>
-__global__ void __launch_bounds__(128, sweep_min_blocks<ORDER, R, FIELD, TMA, LEAN>())
+          int SHAPE = kShapeAny>
+__global__ void __launch_bounds__(128, sweep_min_blocks<R, FIELD, TMA>())
     sweep_kernel(const __grid_constant__ SweepArgs A, const __grid_constant__ CUtensorMap tmap) {
-  constexpr bool FP32 = sizeof(R) == 4;
   constexpr int G = Geo<ORDER>::G;
   StepState* st = A.st;
   if (st->skip) return;
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  const int mode = A.mode;
-  const double alpha_d = st->alpha[A.dir];
-  const double dt = st->dt;
+  __shared__ TileConst<R> s_k;
+  if (threadIdx.x == 0) tile_const<ORDER, R>(A, st->alpha[A.dir], st->dt, s_k);
   constexpr int KA = kAmax<FIELD>;
   double amax[KA];
 #pragma unroll
   for (int i = 0; i < KA; ++i) amax[i] = 0.0;
   unsigned long long nfall = 0;
-  // Dynamic tile queue: tiles differ in cost (FP64 re-decisions cluster at
-  // discontinuities), so blocks pull the next tile instead of striding.  The
-  // last block to leave resets the queue for the next launch on the stream.
-  __shared__ long long s_tile;
+  // Dynamic tile queue: tiles differ in cost (slow faces and FP64
+  // re-decisions cluster at discontinuities), so blocks pull their next tile
+  // instead of striding.  Thread 0 asks for it as the current tile starts and
+  // works out its geometry as that one ends, so that neither the atomic's
+  // round trip nor the index arithmetic stands between two tiles.  The last
+  // block to leave resets the queue for the next launch on the stream.
   if constexpr (!TMA) {
-    for (;;) {
-      if (threadIdx.x == 0) s_tile = (long long)atomicAdd(&st->tile_next, 1ull);
-      __syncthreads();
-      const long long tile = s_tile;
-      if (tile >= A.ntiles) break;
-      sweep_tile<NV, ORDER, R, false, DEFER, FIELD, false, NoHook, LEAN>(
-          A, tile_geo(A, tile), smem_raw, alpha_d, dt, amax, nfall);
+    __shared__ TileGeo s_geo[2];
+    __shared__ bool s_more[2];
+    if (threadIdx.x == 0) {
+      s_geo[0] = tile_geo(A, blockIdx.x);  // the grid has at most a block per tile
+      s_more[0] = true;
+    }
+    __syncthreads();
+    for (int b = 0; s_more[b]; b ^= 1) {
+      unsigned long long next = 0;
+      if (threadIdx.x == 0) next = atomicAdd(&st->tile_next, 1ull) + gridDim.x;
+      auto publish = [&]() {
+        if (threadIdx.x == 0) {
+          const bool more = next < (unsigned long long)A.ntiles;
+          s_more[b ^ 1] = more;
+          if (more) s_geo[b ^ 1] = tile_geo(A, (long long)next);
+        }
+      };
+      sweep_tile<NV, ORDER, R, false, DEFER, FIELD, false, SHAPE, decltype(publish)>(
+          A, s_geo[b], smem_raw, s_k, amax, nfall, RawTile{}, publish);
     }
   } else {
+    __shared__ long long s_tile;
     __shared__ __align__(8) unsigned long long s_bar;
     double* raw = reinterpret_cast<double*>(smem_raw);
     unsigned char* smem = smem_raw + A.tma_raw_bytes;
@@ -1911,9 +2322,8 @@ __global__ void __launch_bounds__(128, sweep_min_blocks<ORDER, R, FIELD, TMA, LE
           const long long sg = g.s0 - G + e;
           if (sg >= 0 && sg < g.nd) return;
           double q[NV];
-          load_state<NV, false>(A.u_in, A.cstride,
-                                g.base + (g.a0 + a) * g.stride_a + bc_map(sg, g.nd, A.bc) * g.stride_d,
-                                A.dir, q);
+          load_state<NV, false>(
+              A, g.base + (g.a0 + a) * g.stride_a + bc_map(sg, g.nd, A.bc) * g.stride_d, q);
           double* p = raw + a * rt.ra + (e + rt.xoff) * rt.re;
 #pragma unroll
           for (int c = 0; c < NV; ++c) p[perm_comp<NV>(c, A.dir) * rt.rc] = q[c];
@@ -1927,8 +2337,7 @@ __global__ void __launch_bounds__(128, sweep_min_blocks<ORDER, R, FIELD, TMA, LE
           if (t < A.ntiles) issue(t);
         }
       };
-      sweep_tile<NV, ORDER, R, false, DEFER, FIELD, true>(A, g, smem, alpha_d, dt, amax, nfall, rt,
-                                                          hook);
+      sweep_tile<NV, ORDER, R, false, DEFER, FIELD, true>(A, g, smem, s_k, amax, nfall, rt, hook);
     }
   }
   sweep_epilogue<NV, R, DEFER, FIELD>(A, amax, nfall);
@@ -1945,15 +2354,18 @@ __global__ void __launch_bounds__(128, sweep_min_blocks<ORDER, R, FIELD, TMA, LE
 // blocks never wait on one another.  Ax and Ay are the two axes' arguments
 // as separate launches would take them; the host makes the 2D tile a whole
 // number of both axes' sub-tiles (Ay.ts % Ax.ta == 0, Ax.ts % Ay.ta == 0).
-template <int NV, int ORDER, bool LEAN>
-__global__ void __launch_bounds__(128, sweep_min_blocks<ORDER, float, false, false, LEAN>())
+template <int NV, int ORDER>
+__global__ void __launch_bounds__(128, sweep_min_blocks<float>())
     fused2d_kernel(const __grid_constant__ SweepArgs Ax, const __grid_constant__ SweepArgs Ay) {
   using R = float;
   StepState* st = Ay.st;
   if (st->skip) return;
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  const double alpha_x = st->alpha[0], alpha_y = st->alpha[1];
-  const double dt = st->dt;
+  __shared__ TileConst<R> s_kx, s_ky;
+  if (threadIdx.x == 0) {
+    tile_const<ORDER, R>(Ax, st->alpha[0], st->dt, s_kx);
+    tile_const<ORDER, R>(Ay, st->alpha[1], st->dt, s_ky);
+  }
   double amax[3] = {0.0, 0.0, 0.0};
   unsigned long long nfall = 0;
   const long long tx = Ax.tiles_s, ty = Ay.tiles_s;  // 2D tiles along x and y
@@ -1968,14 +2380,14 @@ __global__ void __launch_bounds__(128, sweep_min_blocks<ORDER, float, false, fal
     for (int k = 0; k < kx; ++k) {
       const long long rows = Y * kx + k;  // row group of Ax.ta rows
       if (rows >= Ax.tiles_a) break;
-      sweep_tile<NV, ORDER, R, false, false, false, false, NoHook, LEAN>(
-          Ax, tile_geo(Ax, X + Ax.tiles_s * rows), smem_raw, alpha_x, dt, amax, nfall);
+      sweep_tile<NV, ORDER, R, false, false, false, false, kShapeXStore>(
+          Ax, tile_geo(Ax, X + Ax.tiles_s * rows), smem_raw, s_kx, amax, nfall);
     }
     for (int m = 0; m < ky; ++m) {
       const long long cols = X * ky + m;  // column group of Ay.ta columns
       if (cols >= Ay.tiles_a) break;
-      sweep_tile<NV, ORDER, R, false, false, false, false, NoHook, LEAN>(
-          Ay, tile_geo(Ay, Y + Ay.tiles_s * cols), smem_raw, alpha_y, dt, amax, nfall);
+      sweep_tile<NV, ORDER, R, false, false, false, false, kShapeYCombine>(
+          Ay, tile_geo(Ay, Y + Ay.tiles_s * cols), smem_raw, s_ky, amax, nfall);
     }
   }
   sweep_epilogue<NV, R, false, false>(Ay, amax, nfall);
@@ -2030,7 +2442,7 @@ __device__ __forceinline__ void face_change32(const SweepArgs& A, const TileGeo&
   const float gm1 = A.gm1_f, adv = A.adv_f;
   const float halpha = 0.5f * (float)alpha_d;
   auto cell = [&](long long gi, double (&q)[NV]) {
-    load_state<NV, false>(A.u_in, A.cstride, g.base + bc_map(gi, g.nd, A.bc) * g.stride_d, A.dir, q);
+    load_state<NV, false>(A, g.base + bc_map(gi, g.nd, A.bc) * g.stride_d, q);
   };
   const bool shear = NV >= 4 && v >= 2 && v <= NV - 2;
   float L[NV], Rc[NV], w = 0.0f;
@@ -2077,14 +2489,14 @@ __device__ __forceinline__ void face_change32(const SweepArgs& A, const TileGeo&
     float acc = 0.0f;
     if constexpr (NV >= 4) {
       if (shear) {
-        acc = shear_comp<NV>(x, v) - w * x[0];
+        acc = fma(-w, x[0], shear_comp<NV>(x, v));
       } else {
 #pragma unroll
-        for (int c = 0; c < NV; ++c) acc += L[c] * x[c];
+        for (int c = 0; c < NV; ++c) acc = fma(L[c], x[c], acc);
       }
     } else {
 #pragma unroll
-      for (int c = 0; c < NV; ++c) acc += L[c] * x[c];
+      for (int c = 0; c < NV; ++c) acc = fma(L[c], x[c], acc);
     }
     d[i] = sgn == 0 ? acc : -acc;
   }
@@ -2097,18 +2509,18 @@ __device__ __forceinline__ void face_change32(const SweepArgs& A, const TileGeo&
   changed = true;
   float corr = 0.0f;
 #pragma unroll
-  for (int i = GE::LO; i <= GE::HI; ++i) corr += bcoef<float>(pick64, i) * d[i];
+  for (int i = GE::LO; i <= GE::HI; ++i) corr = fma(bcoef<float>(pick64, i), d[i], corr);
   const float dv = corr - corr_old;
   if constexpr (NV >= 4) {
     if (shear) {  // column v of R is e_v + w e_{NV-1}
 #pragma unroll
       for (int c = 2; c < NV - 1; ++c) dC[c] += c == v ? dv : 0.0f;
-      dC[NV - 1] += w * dv;
+      dC[NV - 1] = fma(w, dv, dC[NV - 1]);
       return;
     }
   }
 #pragma unroll
-  for (int c = 0; c < NV; ++c) dC[c] += Rc[c] * dv;
+  for (int c = 0; c < NV; ++c) dC[c] = fma(Rc[c], dv, dC[c]);
 }
 
 // Adds s * dC (s = +-1/dx) to L(u) of one cell: to the stored L(u) of a
