@@ -291,35 +291,41 @@ bool fp32(const enoao_ctx* c) { return c->cfg.precision == ENOAO_FP32_BULK; }
 
 int halo(int order) { return order / 2 + 2; }
 
-// Default tile of axis d for an FP32-bulk sweep of this grid: the candidate
+// Default tile of axis d for a sweep of this grid (one splitting constant): the candidate
 // of the least modelled time.  A tile costs a fixed part, a part per face (the
 // ones not proven smooth) and, per phase, as many rounds as its cells (phase
 // 1: with the halo) or faces take over the threads of a line; the sweep takes
 // as many tiles as the resident blocks do in turn, and one more (the tail).
 // Candidates fill whole rounds, so ragged lengths and small grids -- which want
 // many small tiles -- come out of the same rule.  Tiles whose shared memory
-// would leave fewer than seven blocks an SM are not considered.  y and z tiles
-// of 8 lines use half of each 128-byte line they touch (256^3 z sweep: 8 x 31
-// 1.18 ms, 16 x 16 0.82 ms); x tiles of one or two lines were up to 10 %
+// would leave fewer than seven (FP64: three) blocks an SM are not considered.
+// FP32 y and z tiles of 8 lines use half of each 128-byte line they touch
+// (256^3 z sweep: 8 x 31 1.18 ms, 16 x 16 0.82 ms); FP64 sweeps, bound by the
+// FP64 unit, take 8 lines for the smaller halo (2048^2 y sweep: 32 x 15 1.73,
+// 16 x 40 1.60, 8 x 55 1.51 ms).  x tiles of one or two lines were up to 10 %
 // behind four (4096^2 ENO-AO7 x sweep: 1 x 374 0.67, 2 x 118 0.60, 4 x 86 0.56 ms).
 void pick_tile(const enoao_ctx* c, int d, int* ta_out, int* ts_out) {
   const int G = halo(c->cfg.order);
   const long long nd = c->cfg.n[d], lines = c->ncell / nd;
   const long long na = d == 0 ? lines : c->cfg.n[0], nb = lines / na;
   double best = 1e300;
+  const bool f32 = fp32(c);
   for (int ta = d == 0 ? 1 : 8; ta <= (d == 0 ? 4 : 16); ta *= 2) {
     if (c->cfg.ndim == 1 && ta > 1) break;
     const int tpl = 128 / ta;  // threads of a line
     for (int k = 1; k <= 16; ++k) {
       for (int ts : {tpl * k - 2 * G, tpl * k - 1}) {
         if (ts < 8) continue;
-        const int se = sweep_row_pitch(c->nv, c->cfg.order, 1, d, ta, ts);
-        if (sweep_smem_bytes(c->nv, 1, ta, se) > 33 * 1024) continue;
+        const int se = sweep_row_pitch(c->nv, c->cfg.order, f32, d, ta, ts);
+        if (sweep_smem_bytes(c->nv, f32, ta, se) > (f32 ? 33 : 72) * 1024) continue;
         const double tiles = (double)((nd + ts - 1) / ts) * ((na + ta - 1) / ta) * nb;
         const int r1 = (ts + 2 * G + tpl - 1) / tpl, r2 = (ts + 1 + tpl - 1) / tpl,
                   r3 = (ts + tpl - 1) / tpl;
-        double t = (80 + 130 * r1 + 90 * r2 + 80 * r3 + ta * (ts + 1)) * (1 + tiles / (8.0 * c->sms));
-        if (d > 0 && ta == 8) t *= 1.25;
+        double t = f32 ? (80 + 130 * r1 + 90 * r2 + 80 * r3 + ta * (ts + 1)) *
+                             (1 + tiles / (8.0 * c->sms))
+                       : (80 + 160 * r1 + 120 * r2 + 60 * r3 + 2 * ta * (ts + 1)) *
+                             (1 + tiles / (3.0 * c->sms));
+        if (d > 0 && ta == (f32 ? 8 : 16)) t *= 1.25;
         if (d == 0 && ta < 4 && c->cfg.ndim > 1) t *= ta == 1 ? 1.1 : 1.04;
         if (t < best) best = t, *ta_out = ta, *ts_out = ts;
       }
@@ -327,10 +333,10 @@ void pick_tile(const enoao_ctx* c, int d, int* ta_out, int* ts_out) {
   }
 }
 
-// FP64 and per-field sweeps: tile lengths are 2^k - 1 cells, so that the 2^k
-// faces of a line fill whole warps in the per-face phase.
+// Per-field sweeps: tile lengths are 2^k - 1 cells, so that the 2^k faces of a
+// line fill whole warps in the per-face phase.
 void default_tiles(enoao_ctx* c) {
-  const bool f32 = fp32(c), prove = f32 && !consts(c).field;
+  const bool f32 = fp32(c), prove = !consts(c).field;
   for (int d = 0; d < c->cfg.ndim; ++d) {
     c->block[d] = 128;
     if (prove) {
@@ -355,9 +361,9 @@ enoao_status check_tiles(enoao_ctx* c, int d, int ta, int ts) {
   const int field = consts(c).field;
   size_t smem = sweep_smem_bytes(
       c->nv, fp32(c), ta, sweep_row_pitch(c->nv, c->cfg.order, fp32(c), d, ta, ts, field), field);
-  // (FP32 bulk keeps a value per cell more than the 200 KB that tiles may take
-  // were set for)
-  if (smem > (fp32(c) ? 216 : 200) * 1024)
+  // (216 KB: the tiles that fitted 200 KB before a cell took a face-list word
+  // and, in FP32 bulk, a value more)
+  if (smem > 216 * 1024)
     return fail(c, ENOAO_EINVAL, "tile %dx%d needs %zu bytes of shared memory", ta, ts, smem);
   return ENOAO_OK;
 }

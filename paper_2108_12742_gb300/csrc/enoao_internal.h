@@ -253,13 +253,13 @@ inline int sweep_row_pitch(int nv, int order, int fp32, int dir, int ta, int ts,
 // Dynamic shared memory of one sweep block: per extended cell the split
 // differences and the face correction (three vectors), the Roe ingredients
 // (Euler equations), in FP32 bulk with one splitting constant the magnitude of
-// the pair's differences, and in FP32 bulk a word of the face list.  The FP32
+// the pair's differences, and a word of the face list.  The FP32
 // vectors of the 1D system are four values wide, the spare ones taking the
 // magnitude and two of its Roe ingredients.
 inline size_t sweep_smem_bytes(int nv, int fp32, int ta, int se, int field = 0) {
   const size_t cells = (size_t)tile_cells(ta, se);
   const int prims = nv > 1 ? nv : 0;
-  if (!fp32) return cells * (size_t)(3 * nv + prims) * 8;
+  if (!fp32) return cells * ((size_t)(3 * nv + prims) * 8 + 4);
   if (field) return cells * (size_t)(4 * nv + 1) * 4;
   return cells * (size_t)(nv == 3 ? 14 : 3 * nv + prims + 2) * 4;
 }

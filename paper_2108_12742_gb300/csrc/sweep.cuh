@@ -812,9 +812,9 @@ __device__ __forceinline__ void item_start(int lgTA, bool sfast, int& a, int& e0
 }
 
 // Whether a sweep variant proves most faces to take the top candidate before
-// any projection (phase 2a below): FP32 bulk with one splitting constant.
-template <typename R, bool FIELD>
-constexpr bool kProve = sizeof(R) == 4 && !FIELD;
+// any projection (phase 2a below): all with one splitting constant.
+template <bool FIELD>
+constexpr bool kProve = !FIELD;
 
 // Per-cell vectors in shared memory.  FP32 vectors of the Euler equations are
 // one float4 per cell, so a cell moves in one 128-bit access: the 1D system
@@ -986,6 +986,35 @@ __device__ __forceinline__ int shape_mode(const SweepArgs& A) {
   return A.mode;
 }
 
+// FP64 path: whether FP32 bounds show a new state to be physical and, when the
+// next alpha is being taken, its |u_d| + c to be no more than the maxima so
+// far.  The margins (1e-5 and 1e-6 of the summed magnitudes) cover the FP32
+// rounding of every operation; NaN, infinities and values beyond FP32's range
+// are never shown.
+template <int NV, int KA>
+__device__ __forceinline__ bool state_is_plain(const double (&u)[NV], float gm1, bool alpha,
+                                               const double (&amax)[KA]) {
+  const float rho = f32_rn(u[0]), E = f32_rn(u[NV - 1]);
+  float m[NV], m2 = 0.0f;
+#pragma unroll
+  for (int c = 1; c < NV - 1; ++c) {
+    m[c] = f32_rn(u[c]);
+    m2 = fmaf(m[c], m[c], m2);
+  }
+  const float ir = __fdividef(1.0f, rho), ke = 0.5f * m2 * ir;
+  const float ei = E - ke, sum = E + ke;
+  bool ok = rho > 1e-30f && sum < 1e30f && ei > 1e-5f * sum;
+  if (alpha) {
+    const float c = sqrtf((1.0f + gm1) * gm1 * fmaf(1e-6f, sum, ei) * ir);
+#pragma unroll
+    for (int d = 0; d < NV - 2; ++d) {
+      const float s = fmaf(fabsf(m[1 + d]), ir, c);
+      ok = ok && s * 1.00001f <= f32_rn(amax[d]);
+    }
+  }
+  return ok;
+}
+
 // Number of alpha maxima a sweep accumulates: |u_d| + c per axis, or with
 // per-field constants |u_d - c|, |u_d|, |u_d + c| per axis.
 template <bool FIELD>
@@ -1002,9 +1031,9 @@ __device__ __forceinline__ unsigned entry_flags(unsigned e) { return e & 0x3ffu;
 
 // The shared-memory planes of a tile, sizes as sweep_smem_bytes: per extended
 // cell the split differences df+ and df-, the face correction C, the Roe
-// ingredients, with kProve the magnitude of the pair's split differences, and
-// in FP32 bulk one word for the face list (faces not proven, or with flagged
-// choices).  The 1D system keeps the magnitude with df+ and two of its three
+// ingredients, in FP32 bulk with kProve the magnitude of the pair's split
+// differences, and one word for the face list (faces not proven, or with
+// flagged choices).  The 1D system keeps the magnitude with df+ and two of its three
 // Roe ingredients with df- and C (the spare values).  Shared by the tile's
 // phases and the out-of-line re-decision.
 template <int NV, int ORDER, typename R, bool FIELD>
@@ -1012,13 +1041,13 @@ struct TileView {
   using GE = Geo<ORDER>;
   using CV = CellVec<NV, R, FIELD>;
   static constexpr bool FP32 = sizeof(R) == 4;
-  static constexpr bool PROVE = kProve<R, FIELD>;
+  static constexpr bool MAG = FP32 && kProve<FIELD> && NV != 3;
   R* dfp;
   R* dfm;
   R* Cf;
   R* prim;         // 1D FP32: the third ingredient only
-  float* mag;      // PROVE, all but 1D Euler
-  unsigned* list;  // FP32
+  float* mag;      // MAG
+  unsigned* list;
   int cells, SE;
   __device__ __forceinline__ TileView(unsigned char* smem_raw, int ta, int se)
       : cells(tile_cells(ta, se)), SE(se) {
@@ -1028,7 +1057,7 @@ struct TileView {
     prim = Cf + CV::kSlots * cells;
     R* p = prim + (NV == 1 ? 0 : (CV::kSpare ? 1 : NV)) * cells;
     mag = reinterpret_cast<float*>(p);
-    if constexpr (PROVE && NV != 3) p += cells;
+    if constexpr (MAG) p += cells;
     list = reinterpret_cast<unsigned*>(p);
   }
   // Roe ingredients of the cell at slot i
@@ -1313,6 +1342,105 @@ __device__ __forceinline__ bool prove_top(const TileView<NV, ORDER, float, FIELD
   return ok && fmaf(K * feps, P, most) <= limit;  // false for NaN
 }
 
+// The same for the FP64 path: the proof in FP32 from the FP64 differences and
+// ingredients (narrowed on the integer units: the FP64 unit, 1/64 of the FP32
+// rate, bounds this path, and its issue slots are nine tenths idle), the
+// correction in FP64.  The proof only decides; what it cannot decide with its
+// margin -- the FP32 rounding of the differences, and of the left rows, which
+// the cancellation in c^2 = (gamma-1) (H - |v|^2/2) magnifies by up to
+// (gamma-1) H / c^2 -- goes through the FP64 indicators as before.  With every
+// field on the top candidate R L = I, so the values need no projection: C is
+// a sum of FP64 differences, 8 NV (ENO-AO7: 12 NV) operations instead of 500.
+template <int NV, int ORDER, bool FIELD>
+__device__ __forceinline__ bool prove_top(const TileView<NV, ORDER, double, FIELD>& tv, int x,
+                                          float gm1, float limit, double (&C)[NV]) {
+  using CV = CellVec<NV, double, FIELD>;
+  constexpr int H = ORDER == 7 ? 3 : 2;  // pairs j-H .. j+H
+  constexpr float bw[4] = {1.0f, ORDER == 7 ? -6.0f : -4.0f, ORDER == 7 ? 15.0f : 6.0f, -20.0f};
+  constexpr int B0 = ORDER == 5 ? 2 : 1, B1 = ORDER == 5 ? 5 : 6;
+  constexpr int ND = NV == 1 ? 1 : 3, NS = NV > 3 ? NV - 3 : 0;
+  float L[ND][NV], vt[NS > 0 ? NS : 1], K = 1.0f, feps = (NV + 16) * FLT_EPSILON;
+  if constexpr (NV > 1) {
+    double p64[NV];
+    float pl[NV], prr[NV];
+    tv.load_prims(x, p64);
+#pragma unroll
+    for (int c = 0; c < NV; ++c) pl[c] = f32_rn(p64[c]);
+    tv.load_prims(x + 1, p64);
+#pragma unroll
+    for (int c = 0; c < NV; ++c) prr[c] = f32_rn(p64[c]);
+    Eigen<NV, float> E;
+    roe_eigen<NV, float>(pl, prr, gm1, E);
+    left_row<NV, float>(E, 0, L[0]);
+    left_row<NV, float>(E, 1, L[1]);
+    left_row<NV, float>(E, NV - 1, L[2]);
+#pragma unroll
+    for (int t = 0; t < NS; ++t) {
+      vt[t] = E.vt[t];
+      K = fmaxf(K, fabsf(vt[t]));
+    }
+    // bounds on the entries from the terms they are sums of (a left row's
+    // rounding is relative to those)
+    const float q = sqrtf(E.q2);
+    K = fmaxf(K, fmaxf(fmaxf(1.0f + E.b2, 0.5f * fmaf(q, E.ic, E.b2)),
+                       fmaxf(0.5f * fmaf(E.b1, q, E.ic), E.b1 * fmaxf(q, 1.0f))));
+    feps = (NV + 8 + 8.0f * E.H * E.b1) * FLT_EPSILON;
+  } else {
+    L[0][0] = 1.0f;
+  }
+  bool ok = true;
+#pragma unroll 1
+  for (int sgn = 0; sgn < 2; ++sgn) {
+    const double* src = sgn == 0 ? tv.dfp : tv.dfm;
+    float D[NV], P = 0.0f;
+#pragma unroll
+    for (int c = 0; c < NV; ++c) D[c] = 0.0f;
+#pragma unroll
+    for (int k = -H; k <= H; ++k) {
+      double p[NV];
+      CV::load(src, tv.cells, x + k, p);
+      const float w = bw[k <= 0 ? k + H : H - k];
+#pragma unroll
+      for (int c = 0; c < NV; ++c) {
+        const float pc = f32_rn(p[c]);
+        D[c] = fmaf(w, pc, D[c]);
+        P = fmaf(fabsf(w), fabsf(pc), P);
+      }
+    }
+    float d = 0.0f;
+#pragma unroll
+    for (int v = 0; v < ND; ++v) {
+      float t = 0.0f;
+#pragma unroll
+      for (int c = 0; c < NV; ++c) t = fmaf(L[v][c], D[c], t);
+      d = fmaxf(d, fabsf(t));
+      ok = ok && t == t;  // fmaxf drops a NaN
+    }
+#pragma unroll
+    for (int t = 0; t < NS; ++t) d = fmaxf(d, fabsf(fmaf(-vt[t], D[0], D[2 + t])));
+    ok = ok && fmaf(K * feps, P, d) <= limit;  // false for NaN
+  }
+  if (!ok) return false;
+#pragma unroll
+  for (int sgn = 0; sgn < 2; ++sgn) {
+    const double* src = sgn == 0 ? tv.dfp : tv.dfm;
+    double corr[NV];
+#pragma unroll
+    for (int c = 0; c < NV; ++c) corr[c] = 0.0;
+#pragma unroll
+    for (int i = B0; i <= B1; ++i) {
+      double p[NV];
+      CV::load(src, tv.cells, x + (sgn == 0 ? i - 4 : 4 - i), p);
+      const double b = bcoef_top<ORDER, double>(i);
+#pragma unroll
+      for (int c = 0; c < NV; ++c) corr[c] = fma(b, sgn == 0 ? p[c] : -p[c], corr[c]);
+    }
+#pragma unroll
+    for (int c = 0; c < NV; ++c) C[c] = sgn == 0 ? corr[c] : C[c] + corr[c];
+  }
+  return true;
+}
+
 // The raw state of a tile staged in shared memory by TMA: conserved
 // component c of line a at extended cell e is p[c rc + a ra + (e + xoff) re]
 // (the layout of the copied box; xoff is the alignment slack of x boxes).
@@ -1343,8 +1471,9 @@ __device__ __forceinline__ void tile_const(const SweepArgs& A, double alpha_d, d
   k.alpha = (R)alpha_d;
   k.dt32 = f32_rn(dt);
   k.wdt32 = f32_rn((A.stage == 0 ? 1.0 : (A.stage == 1 ? 0.25 : 2.0 / 3.0)) * dt);
-  // below delta by more than the near-tie margin (and the bound's own rounding)
-  k.limit = A.delta_f - fmaf(A.tie_rel_f, A.delta_f, 1e-3f * A.delta_f);
+  // below delta by more than the near-tie margin (and the bound's own
+  // rounding); FP64 has no near-ties and takes a margin of its own
+  k.limit = A.delta_f - fmaf(sizeof(R) == 4 ? A.tie_rel_f : 1e-3f, A.delta_f, 1e-3f * A.delta_f);
 }
 
 // Whether the tile is the one that writes face f (the face between two tiles
@@ -1456,18 +1585,126 @@ __device__ __forceinline__ unsigned choose_face(const SweepArgs& A, const TileGe
   return fix;
 }
 
-// Phase 2 of the faces on the tile's list (FP32 bulk, kProve), one per
-// thread; their near-ties go into the list's entries.  Returns whether this
+// Lanes that share a face of a short list: one per field and sign.
+template <int NV>
+constexpr int kFaceLanes = NV == 1 ? 2 : (NV <= 4 ? 8 : 16);
+
+// choose_face of a face whose choices are spread over the kFaceLanes lanes of
+// an aligned group, lane r taking field r / 2, sign r % 2 (the operations of
+// choose_face, so the same bits): a tile's list is mostly a few faces, which
+// one per thread would leave to a few lanes, each with ten dependent
+// selections.  Every lane of the warp calls it; valid is the same over a group.
+template <int NV, int ORDER, typename R, bool COHERENT, int SHAPE>
+__device__ __forceinline__ unsigned choose_face_group(const SweepArgs& A, const TileGeo& g,
+                                                      const TileView<NV, ORDER, R, false>& tv,
+                                                      const int a, const int f, const bool valid) {
+  using CV = CellVec<NV, R, false>;
+  using GE = Geo<ORDER>;
+  constexpr int G = GE::G, W = kFaceLanes<NV>;
+  constexpr bool FP32 = sizeof(R) == 4;
+  const unsigned FULL = 0xffffffffu;
+  const int r = threadIdx.x & (W - 1);
+  const int v = r >> 1 < NV ? r >> 1 : 0, sgn = r & 1;
+  const R gm1 = bconst<R>(A.gm1, A.gm1_f);
+  const int j = G - 1 + f, x = tv.sidx(a, j);
+  Eigen<NV, R> E;
+  const bool shear = NV >= 4 && v >= 2 && v <= NV - 2;
+  R L[NV], w = R(0);
+  if constexpr (NV > 1) {
+    face_eigen<NV, ORDER, R, false>(tv, x, gm1, E);
+    left_row<NV, R>(E, v, L);
+    if constexpr (NV >= 4) w = -L[0];
+  } else {
+    L[0] = R(1);
+  }
+  R d[8], mag[8];
+  const R* src = sgn == 0 ? tv.dfp : tv.dfm;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) d[i] = mag[i] = R(0);
+#pragma unroll
+  for (int i = GE::LO; i <= GE::HI; ++i) {
+    R q[NV], acc = R(0), m = R(0);
+    CV::load(src, tv.cells, x + (sgn == 0 ? i - 4 : 4 - i), q);
+    if constexpr (NV >= 4) {
+      if (shear) {
+        const R qv = shear_comp<NV>(q, v);
+        acc = fma(-w, q[0], qv);
+        if constexpr (FP32) m = fma(rabs(w), rabs(q[0]), rabs(qv));
+      }
+    }
+    if (!shear) {
+#pragma unroll
+      for (int c = 0; c < NV; ++c) {
+        acc = fma(L[c], q[c], acc);
+        if constexpr (FP32) m = fma(rabs(L[c]), rabs(q[c]), m);
+      }
+    }
+    d[i] = sgn == 0 ? acc : -acc;
+    mag[i] = m;
+  }
+  int pick;
+  bool marg = false;
+  const R corr = eno_select<ORDER, R, FP32>(d, bconst<R>(A.delta, A.delta_f),
+                                            bconst<R>(A.tie_rel, A.tie_rel_f), mag,
+                                            R(NV + 8) * R(FLT_EPSILON), pick, marg);
+  const bool mine = valid && r < 2 * NV;
+  if ((shape_mode<SHAPE>(A) & kModeFlux) && A.idx_out && mine && owns_face(A, g, f))
+    A.idx_out[r * A.nfaces + face_index(g, a, f)] = (int8_t)pick;
+  const R cv = corr + __shfl_xor_sync(FULL, corr, 1);  // f^+ and f^- of the field
+  R C[NV];
+#pragma unroll
+  for (int c = 0; c < NV; ++c) C[c] = R(0);
+#pragma unroll
+  for (int k = 0; k < NV; ++k) {  // the fields in order
+    const R ck = __shfl_sync(FULL, cv, 2 * k, W);
+    if constexpr (NV == 1) {
+      C[0] += ck;
+    } else if (k >= 2 && k <= NV - 2) {
+      C[k] += ck;
+      C[NV - 1] = fma(E.vt[k >= 2 ? k - 2 : 0], ck, C[NV - 1]);
+    } else {
+      R Rc[NV];
+      right_col<NV, R>(E, k, Rc);
+#pragma unroll
+      for (int c = 0; c < NV; ++c) C[c] = fma(Rc[c], ck, C[c]);
+    }
+  }
+  if (valid && r == 0) CV::store(tv.Cf, tv.cells, x, C);
+  if constexpr (FP32) {
+    const unsigned all = __ballot_sync(FULL, marg && r < 2 * NV);
+    return all >> (threadIdx.x & 31 & ~(W - 1)) & ((1u << (2 * NV)) - 1u);
+  }
+  return 0u;
+}
+
+// Phase 2 of the faces on the tile's list (kProve), one per thread, or by
+// groups of lanes when the list is short enough for one round of them; their
+// near-ties go into the list's entries.  Returns whether this
 // thread met one.
-template <int NV, int ORDER, bool COHERENT, int SHAPE>
+template <int NV, int ORDER, typename R, bool COHERENT, int SHAPE>
 __device__ __forceinline__ bool listed_faces(const SweepArgs& A, const TileGeo& g,
-                                             unsigned char* smem_raw, const TileConst<float>& K,
+                                             unsigned char* smem_raw, const TileConst<R>& K,
                                              int n) {
-  const TileView<NV, ORDER, float, false> tv(smem_raw, A.ta, A.se);
+  const TileView<NV, ORDER, R, false> tv(smem_raw, A.ta, A.se);
   bool any = false;
+  constexpr int W = kFaceLanes<NV>;
+  if (n * W <= (int)blockDim.x) {  // a group of lanes per face, one round
+    const int i = threadIdx.x / W;
+    if ((int)(threadIdx.x & ~31u) < n * W) {  // warps with a face
+      const bool valid = i < n;
+      const unsigned entry = tv.list[valid ? i : 0];
+      const unsigned fix = choose_face_group<NV, ORDER, R, COHERENT, SHAPE>(
+          A, g, tv, entry_line(entry), entry_face(entry), valid);
+      if (fix && valid) {
+        if ((threadIdx.x & (W - 1)) == 0) tv.list[i] = entry | fix;
+        any = true;
+      }
+    }
+    return any;
+  }
   for (int i = threadIdx.x; i < n; i += blockDim.x) {
     const unsigned entry = tv.list[i];
-    const unsigned fix = choose_face<NV, ORDER, float, COHERENT, false, SHAPE>(
+    const unsigned fix = choose_face<NV, ORDER, R, COHERENT, false, SHAPE>(
         A, g, tv, K, entry_line(entry), entry_face(entry));
     if (fix) {
       tv.list[i] = entry | fix;
@@ -1483,7 +1720,7 @@ template <int NV, int ORDER, bool COHERENT, int SHAPE>
 __device__ __noinline__ bool listed_faces_call(const SweepArgs& A, const TileGeo& g,
                                                unsigned char* smem_raw, const TileConst<float>& K,
                                                int n) {
-  return listed_faces<NV, ORDER, COHERENT, SHAPE>(A, g, smem_raw, K, n);
+  return listed_faces<NV, ORDER, float, COHERENT, SHAPE>(A, g, smem_raw, K, n);
 }
 
 // One tile of a sweep (phases 1-3 above).  amax accumulates |u_d| + c of
@@ -1714,9 +1951,9 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& A, const TileGeo& g,
   using GE = Geo<ORDER>;
   constexpr int G = GE::G;
   constexpr bool FP32 = sizeof(R) == 4;
-  constexpr bool PROVE = kProve<R, FIELD>;
+  constexpr bool PROVE = kProve<FIELD>;
   // the code of faces not proven and of near-ties out of line
-  constexpr bool CALL = PROVE && SHAPE != kShapeAny && !COHERENT;
+  constexpr bool CALL = FP32 && PROVE && SHAPE != kShapeAny && !COHERENT;
   StepState* st = A.st;
   const int TA = A.ta, TS = A.ts;
   // row pitch A.se (>= TS + 2G), chosen on the host for conflict-free banks
@@ -1726,10 +1963,10 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& A, const TileGeo& g,
   R* const dfm = tv.dfm;
   R* const Cf = tv.Cf;
   R* const prim = tv.prim;
-  // FP32 bulk: faces on the tile's list (those not proven in phase 2a, or
-  // all with flagged choices)
+  // faces on the tile's list (those not proven in phase 2a; per field, those
+  // with flagged choices)
   __shared__ int s_nlist;
-  if (FP32 && threadIdx.x == 0) s_nlist = 0;
+  if ((FP32 || PROVE) && threadIdx.x == 0) s_nlist = 0;
 
   const int dir = A.dir;
   const bool sfast = shape_x<SHAPE>(A);
@@ -1823,7 +2060,7 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& A, const TileGeo& g,
       } else {
         CV::store(dfp, cells, sidx(a, e), fp);
         CV::store(dfm, cells, sidx(a, e), fm);
-        if constexpr (PROVE) tv.mag[sidx(a, e)] = m;
+        if constexpr (tv.MAG) tv.mag[sidx(a, e)] = m;
       }
     };
     if (sfast) {
@@ -1883,7 +2120,7 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& A, const TileGeo& g,
   __syncthreads();
   if constexpr (TMA) hook();
 
-  // ---------------- phase 2a (FP32 bulk): prove the smooth faces, list the others
+  // ---------------- phase 2a: prove the smooth faces, list the others
   const int nfaces_tile = nts + 1;
   bool any_fix = false;  // FP32 bulk: this thread flagged a near-tie
   if constexpr (PROVE) {
@@ -1891,7 +2128,7 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& A, const TileGeo& g,
       if (g.a0 + a >= g.na) return;
       const int x = sidx(a, G - 1 + f);
       R C[NV];
-      if (prove_top<NV, ORDER, FIELD>(tv, x, gm1, K.limit, C)) {
+      if (prove_top<NV, ORDER, FIELD>(tv, x, A.gm1_f, K.limit, C)) {
         CV::store(Cf, cells, x, C);
         if ((mode & kModeFlux) && A.idx_out && owns_face(A, g, f)) {
           const long long fc = face_index(g, a, f);
@@ -1911,7 +2148,7 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& A, const TileGeo& g,
         if constexpr (CALL)
           any_fix = listed_faces_call<NV, ORDER, COHERENT, SHAPE>(A, g, smem_raw, K, s_nlist);
         else
-          any_fix = listed_faces<NV, ORDER, COHERENT, SHAPE>(A, g, smem_raw, K, s_nlist);
+          any_fix = listed_faces<NV, ORDER, R, COHERENT, SHAPE>(A, g, smem_raw, K, s_nlist);
       }
     } else {
       for_items(lgTA, nfaces_tile, sfast, [&](const int a, const int f) {
@@ -1929,7 +2166,7 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& A, const TileGeo& g,
 
   // ---------------- phase 2b (FP32 bulk): the faces with flagged choices
   if constexpr (!FP32) {
-    __syncthreads();
+    if (!PROVE || s_nlist > 0) __syncthreads();
   } else if (PROVE && s_nlist == 0) {
     // every face proven: C is complete since the barrier of phase 2a
   } else if constexpr (DEFER) {
@@ -2106,9 +2343,12 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& A, const TileGeo& g,
       if constexpr (FP32) {
         bulk_state_check<NV>(A, cell, unew, mode, amax);
       } else if constexpr (NV > 1) {
-        // non-physical check and next-step alpha on the new state
+        // non-physical check and next-step alpha on the new state; its FP64
+        // operations (a division and a square root among them) only where
+        // FP32 bounds leave either open
         double s[kAmax<FIELD>];
-        if (!speeds64<NV, FIELD>(unew, A.gamma, s)) {
+        if (!FIELD && state_is_plain<NV>(unew, A.gm1_f, mode & kModeAlpha, amax)) {
+        } else if (!speeds64<NV, FIELD>(unew, A.gamma, s)) {
           atomicOr(&st->err, kErrNonPhys);
           atomicMin(&st->err_cell, cell);
         } else if (mode & kModeAlpha) {
@@ -2122,6 +2362,17 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& A, const TileGeo& g,
         }
       }
     });
+  }
+  if constexpr (!FP32 && !FIELD && NV > 1) {
+    // the maxima of a warp's lanes are each lane's from here on: the next
+    // tile's cells below them need no FP64 speeds
+    if (mode & kModeAlpha) {
+#pragma unroll
+      for (int d = 0; d < NV - 2; ++d)
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+          amax[d] = fmax(amax[d], __shfl_xor_sync(0xffffffffu, amax[d], o));
+    }
   }
   if constexpr (!TMA) hook();
   __syncthreads();
