@@ -267,7 +267,9 @@ enoao_status enoao_sync(enoao_ctx *ctx);
 /* Reads the run statistics (synchronises). */
 enoao_status enoao_get_stats(enoao_ctx *ctx, enoao_stats *out);
 
-/* Number of CUDA kernel launches one step issues (per graph replay step). */
+/* Number of CUDA kernel launches one step issues (per graph replay step); 0
+ * where one persistent launch covers every step (batched contexts, and 1D
+ * problems of up to 256 cells per SM with one alpha per step). */
 int enoao_launches_per_step(const enoao_ctx *ctx);
 
 /* Tile shape of the sweep kernels along each axis: lines per tile (ta) and

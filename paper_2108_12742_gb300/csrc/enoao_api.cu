@@ -17,7 +17,9 @@
 #include "enoao.h"
 #include "enoao_ctx.h"
 #include "enoao_internal.h"
+#include "run1d.h"
 #include "state_speed.cuh"
+#include "step_state.cuh"
 
 using namespace enoao;
 
@@ -144,73 +146,7 @@ void launch_alpha(int nv, const double* U, long long ncell, long long cstride, d
   if (nv == 5) launch_alpha_nv<5>(U, ncell, cstride, gamma, st, slot, bulk, field, blocks, s);
 }
 
-struct StepConsts {
-  int system, ndim;
-  int field;  // per-field splitting constants (Euler)
-  double adv_speed;
-  double dx[3];
-};
-
-__device__ void finalize_pending(StepState* st) {
-  if (st->pending) {
-    st->t = st->last ? st->t_end : st->t + st->dt;
-    st->steps += 1;
-    if (st->last) st->done = 1;
-    st->pending = 0;
-  }
-}
-
-// Per-field constants of the step from the running maxima of slot cur (the
-// one-alpha value, for dt, is the largest of them); clear: the other slot too.
-// alpha of axis d for the CFL rule (Euler): |u_d| + c of slot cur, which per
-// field is the larger of max |u_d - c| and max |u_d + c| (the last stage then
-// accumulates only the per-field maxima).
-__device__ double step_alpha(const StepState* st, const StepConsts& k, int cur, int d) {
-  if (k.field)
-    return fmax(__longlong_as_double((long long)st->alpha_acc_f[cur][d][0]),
-                __longlong_as_double((long long)st->alpha_acc_f[cur][d][2]));
-  return __longlong_as_double((long long)st->alpha_acc[cur][d]);
-}
-
-__device__ void load_field_alpha(StepState* st, const StepConsts& k, int cur, bool clear) {
-  if (!k.field) return;
-  for (int d = 0; d < 3; ++d)
-    for (int f = 0; f < 3; ++f) {
-      st->alpha_f[d][f] = d < k.ndim ? __longlong_as_double((long long)st->alpha_acc_f[cur][d][f]) : 0.0;
-      if (clear) st->alpha_acc_f[cur ^ 1][d][f] = 0ull;
-    }
-}
-
-// Start of a step: finalise the previous one, fix alpha from U^n and dt from
-// the CFL rule (or the fixed step), shortened to land on t_end.
-__global__ void step_begin_kernel(StepState* st, StepConsts k) {
-  finalize_pending(st);
-  if (st->done || (st->max_steps > 0 && st->steps >= st->max_steps) || st->err) {
-    st->skip = 1;
-    return;
-  }
-  st->skip = 0;
-  const int cur = (int)(st->steps & 1);
-  double s = 0.0;
-  for (int d = 0; d < k.ndim; ++d) {
-    const double a = k.system == ENOAO_EULER
-                         ? step_alpha(st, k, cur, d)
-                         : fabs(k.adv_speed);
-    st->alpha[d] = a;
-    s += a / k.dx[d];
-  }
-  st->par = cur ^ 1;
-  for (int d = 0; d < 3; ++d) st->alpha_acc[cur ^ 1][d] = st->alpha_stage[d] = 0ull;
-  load_field_alpha(st, k, cur, true);
-  double dt = st->dt_fixed > 0.0 ? st->dt_fixed : st->cfl / s;
-  st->last = 0;
-  if (st->t + dt >= st->t_end) {
-    dt = st->t_end - st->t;
-    st->last = 1;
-  }
-  st->dt = dt;
-  st->pending = 1;
-}
+__global__ void step_begin_kernel(StepState* st, StepConsts k) { begin_step(st, k); }
 
 __global__ void finalize_kernel(StepState* st) { finalize_pending(st); }
 
@@ -1160,6 +1096,33 @@ enoao_status enoao_rk_stage(enoao_ctx* c, int stage, double dt) {
   return ENOAO_OK;
 }
 
+// Whether the steps of this context run inside one persistent launch
+// (run1d.cu): 1D problems small enough for a tile per SM, one alpha per step,
+// near-ties re-decided in the sweep, no TMA staging.
+static bool persistent_run(const enoao_ctx* c) {
+  return !c->batch && !c->sub && c->cfg.ndim == 1 && !c->tma && !use_list(c) && !consts(c).field &&
+         !per_stage_alpha(c) && c->ncell <= (long long)kRun1dMaxTile * c->sms;
+}
+
+// Enqueues one persistent launch of up to cap steps.
+static enoao_status enqueue_run1d(enoao_ctx* c, long long cap) {
+  int ts, block;
+  run1d_tile(c->nv, c->ncell, c->sms, &ts, &block);
+  Run1dArgs a;
+  memset(&a, 0, sizeof a);
+  for (int stage = 0; stage < 3; ++stage) {
+    enoao_status r = fill_sweep_args(c, 0, stage, kModeCombine | (stage == 2 ? kModeAlpha : 0),
+                                     c->U[stage], c->U[stage == 2 ? 0 : stage + 1], nullptr, nullptr,
+                                     false, 1, ts, a.stage[stage]);
+    if (r != ENOAO_OK) return r;
+  }
+  a.k = consts(c);
+  a.cap = cap;
+  const cudaError_t e = run1d_launch(c->nv, c->cfg.order, fp32(c), a, block, c->sms, c->s);
+  if (e != cudaSuccess) return fail(c, ENOAO_ECUDA, "1D run launch: %s", cudaGetErrorString(e));
+  return ENOAO_OK;
+}
+
 static enoao_status run_graph_steps(enoao_ctx* c, double t_end, double cfl, double dt_fixed,
                                     long long max_steps, bool until_time, bool sync) {
   if (c->sub)
@@ -1167,15 +1130,36 @@ static enoao_status run_graph_steps(enoao_ctx* c, double t_end, double cfl, doub
                 "a sub-domain steps stage by stage (enoao_rk_stage) between halo exchanges");
   enoao_status r = enter(c);
   if (r != ENOAO_OK) return r;
-  r = build_graph(c, steps_per_graph(c));
-  if (r != ENOAO_OK) return r;
+  const bool persistent = persistent_run(c);
+  if (!persistent) {
+    r = build_graph(c, steps_per_graph(c));
+    if (r != ENOAO_OK) return r;
+  }
   CU(c, cudaMemcpyAsync(c->st_host, c->st, sizeof(StepState), cudaMemcpyDeviceToHost, c->s));
   CU(c, cudaStreamSynchronize(c->s));
   const long long start = c->st_host->steps;
   const long long limit = max_steps > 0 ? start + max_steps : 0;
   set_run_kernel<<<1, 1, 0, c->s>>>(c->st, t_end, cfl, dt_fixed, limit);
   CU(c, cudaGetLastError());
-  if (!until_time) {
+  if (persistent) {
+    // a launch ends at the step limit or end time by itself; launches of
+    // bounded length keep an open-ended run within reach of the host
+    constexpr long long kCap = 4096;
+    if (!until_time) {
+      for (long long k = 0; k < max_steps; k += kCap) {
+        r = enqueue_run1d(c, std::min(kCap, max_steps - k));
+        if (r != ENOAO_OK) return r;
+      }
+    } else {
+      for (;;) {
+        r = enqueue_run1d(c, kCap);
+        if (r == ENOAO_OK) r = read_host_state(c);
+        if (r != ENOAO_OK) return r;
+        if (c->st_host->done || c->st_host->err) break;
+        if (limit > 0 && c->st_host->steps >= limit) break;
+      }
+    }
+  } else if (!until_time) {
     const long long reps = (max_steps + c->graph_steps - 1) / c->graph_steps;
     for (long long k = 0; k < reps; ++k) CU(c, cudaGraphLaunch(c->graph, c->s));
   } else {
@@ -1246,7 +1230,7 @@ enoao_status enoao_get_stats(enoao_ctx* c, enoao_stats* out) {
 
 int enoao_launches_per_step(const enoao_ctx* c) {
   if (!c) return 0;
-  if (c->batch) return 0;  // one persistent launch covers every step
+  if (c->batch || persistent_run(c)) return 0;  // one persistent launch covers every step
   return 1 + 3 * c->cfg.ndim * (use_list(c) ? 3 : 1) + (per_stage_alpha(c) ? 2 : 0);
 }
 

@@ -37,6 +37,7 @@ struct StepState {
                                       // state stage 0 or 1 writes (bit patterns)
   unsigned int redo_epoch;        // sweeps that listed faces: tags the changed-face marks
   unsigned int redo_done;         // blocks of the running apply pass that have left it
+  unsigned int grid_count, grid_gen;  // the grid barrier of the persistent 1D run
   // per-field alpha (Euler): per axis max |u_d - c|, max |u_d|, max |u_d + c|
   double alpha_f[3][3];                   // of the current step
   unsigned long long alpha_acc_f[2][3][3];  // running maxima (bit patterns), as alpha_acc

@@ -1,0 +1,25 @@
+// The persistent run of small 1D problems (run1d.cu).
+#pragma once
+
+#include <cuda_runtime.h>
+
+#include "enoao_internal.h"
+#include "step_state.cuh"
+
+namespace enoao {
+
+struct Run1dArgs {
+  SweepArgs stage[3];  // the sweeps of the three Runge-Kutta stages
+  StepConsts k;
+  long long cap;       // steps of this launch at most
+};
+
+constexpr int kRun1dMaxTile = 256;
+
+// Cells per tile and threads per block for a problem of n cells.
+void run1d_tile(int nv, long long n, int sms, int* ts, int* block);
+// fp32: bulk precision.  One cooperative launch, a block per tile.
+cudaError_t run1d_launch(int nv, int order, int fp32, const Run1dArgs& a, int block, int sms,
+                         cudaStream_t s);
+
+}  // namespace enoao
