@@ -22,8 +22,11 @@
 namespace enoao {
 
 struct BatchArgs {
-  double* U[3];            // U^n, U1, U2; [nv][total]
-  float* inc[2];           // FP32 bulk: stage increments I0, I1; [nv][total]
+  // The sweeps of the three stages over the concatenated arrays; a problem is
+  // a range of their cells (TileGeo) with its own spacing (TileConst).  Kernel
+  // arguments: made per problem in the kernel, their constants were narrowed
+  // anew at each use (conversions on the FP64 unit).
+  SweepArgs stage[3];
   long long total;         // cells of all problems (component stride)
   int nprob;
   int nsteps;
@@ -36,12 +39,25 @@ struct BatchArgs {
   double* alpha;           // alpha of the last step per problem
   double* dt;              // last step size per problem
   int* queue;              // next queue position (reset to 0 before a launch)
-  StepState* st;           // error word and FP64 re-decision count
-  int ts;                  // cells per tile
-  int bc;
   int per_stage_alpha;     // 1: each stage splits with the alpha of its input state
-  double gamma, adv_speed, delta, tie_rel;
 };
+
+// Tile number tile of a problem of n cells from cell off on (tile_geo of a 1D
+// grid, at an offset).
+__device__ __forceinline__ TileGeo batch_geo(const SweepArgs& A, long long off, int n, int tile) {
+  TileGeo g;
+  g.s0 = (long long)tile * A.ts;
+  g.a0 = 0;
+  g.base = g.fbase = off;
+  g.stride_a = g.fstride_a = n;
+  g.stride_d = g.fstride_d = 1;
+  g.na = 1;
+  g.nd = n;
+  g.b = 0;
+  const long long left = n - g.s0;
+  g.nts = (int)(left < A.ts ? left : A.ts);
+  return g;
+}
 
 // Block-wide maximum of v (all threads get the result).
 __device__ __forceinline__ double block_max(double v, double* red) {
@@ -68,10 +84,14 @@ constexpr int batch_min_blocks() {
 }
 
 template <int NV, int ORDER, typename R>
-__global__ void __launch_bounds__(256, batch_min_blocks<R>()) batch_kernel(const BatchArgs B) {
+__global__ void __launch_bounds__(256, batch_min_blocks<R>()) batch_kernel(const __grid_constant__ BatchArgs B) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ int s_q;
   __shared__ double s_red[32];
+  __shared__ TileConst<R> s_k;
+  __shared__ TileGeo s_geo[2];
+  StepState* const st = B.stage[0].st;
+  const double gamma = B.stage[0].gamma;
   unsigned long long nfall = 0;
   for (;;) {
     __syncthreads();
@@ -84,54 +104,29 @@ __global__ void __launch_bounds__(256, batch_min_blocks<R>()) batch_kernel(const
     const int n = B.n[p];
     const double dx = B.dx[p];
 
-    SweepArgs A;
-    memset(&A, 0, sizeof A);
-    A.st = B.st;
-    A.n[0] = n;
-    A.n[1] = A.n[2] = 1;
-    A.ncell = n;
-    A.nfaces = n + 1;
-    A.cstride = B.total;
-    A.ndim = 1;
-    A.dir = 0;
-    A.bc = B.bc;
-    A.ta = 1;
-    A.ts = B.ts;
-    A.se = B.ts + 2 * Geo<ORDER>::G;  // sweep_row_pitch of a one-line x tile
-    A.tiles_s = (n + B.ts - 1) / B.ts;
-    A.tiles_a = A.tiles_b = 1;
-    A.ntiles = A.tiles_s;
-    A.inv_dx = 1.0 / dx;
-    A.gamma = B.gamma;
-    A.adv_speed = B.adv_speed;
-    A.delta = B.delta;
-    A.tie_rel = B.tie_rel;
-    set_derived_constants(A);
-    A.redo_passes = 64 * NV;
-
     // alpha of the initial state of this launch
     double alpha;
     if constexpr (NV > 1) {
       double a = 0.0;
-      const double* U = B.U[0] + off;
+      const double* U = B.stage[0].u_in + off;
       for (int i = threadIdx.x; i < n; i += blockDim.x) {
         // the speeds as a step's last stage takes them (FP32 bulk: speeds32),
         // so that launches split anywhere give the same run
         double u[NV], sp[3];
 #pragma unroll
         for (int c = 0; c < NV; ++c) u[c] = __ldcg(U + c * B.total + i);
-        const bool ok = sizeof(R) == 4 ? speeds32<NV, false>(u, B.gamma, sp)
-                                       : speeds64<NV, false>(u, B.gamma, sp);
+        const bool ok = sizeof(R) == 4 ? speeds32<NV, false>(u, gamma, sp)
+                                       : speeds64<NV, false>(u, gamma, sp);
         if (!ok) {
-          atomicOr(&B.st->err, kErrNonPhys);
-          atomicMin(&B.st->err_cell, off + i);
+          atomicOr(&st->err, kErrNonPhys);
+          atomicMin(&st->err_cell, off + i);
           continue;
         }
         a = fmax(a, sp[0]);
       }
       alpha = block_max(a, s_red);
     } else {
-      alpha = fabs(B.adv_speed);
+      alpha = fabs(B.stage[0].adv_speed);
     }
     double t = B.t[p], dt = 0.0;
     const bool per_stage = NV > 1 && B.per_stage_alpha;
@@ -142,18 +137,22 @@ __global__ void __launch_bounds__(256, batch_min_blocks<R>()) batch_kernel(const
       double a_stage = alpha;  // splitting constant of the current stage
       for (int stage = 0; stage < 3; ++stage) {
         double amax[3] = {0.0, 0.0, 0.0};
-        A.u_in = B.U[stage] + off;
-        A.u0 = B.U[0] + off;
-        A.u_out = B.U[stage == 2 ? 0 : stage + 1] + off;
-        A.inc_in = stage == 0 ? nullptr : B.inc[stage - 1] + off;
-        A.inc_out = stage == 2 ? nullptr : B.inc[stage] + off;
-        A.stage = stage;
-        set_component_pointers(A, sizeof(R) == 4);
-        A.mode = kModeCombine | (stage == 2 || per_stage ? kModeAlpha : 0);
-        TileConst<R> k;
-        tile_const<ORDER, R>(A, a_stage, dt, k);
-        for (long long tile = 0; tile < A.ntiles; ++tile)
-          sweep_tile<NV, ORDER, R, true, false, false, false, kShapeXCombine>(A, tile_geo(A, tile), smem_raw, k, amax, nfall);
+        const SweepArgs& A = B.stage[stage];
+        if (threadIdx.x == 0) {
+          tile_const<ORDER, R>(A, a_stage, dt, s_k);
+          s_k.inv_dx = (R)(1.0 / dx);
+          s_geo[0] = batch_geo(A, off, n, 0);
+        }
+        __syncthreads();
+        const int ntiles = (n + A.ts - 1) / A.ts;
+        for (int tile = 0; tile < ntiles; ++tile) {
+          auto publish = [&]() {
+            if (threadIdx.x == 0 && tile + 1 < ntiles)
+              s_geo[(tile + 1) & 1] = batch_geo(A, off, n, tile + 1);
+          };
+          sweep_tile<NV, ORDER, R, true, false, false, false, kShapeXCombine, decltype(publish)>(
+              A, s_geo[tile & 1], smem_raw, s_k, amax, nfall, RawTile{}, publish);
+        }
         if constexpr (NV > 1) {
           if (stage == 2)
             alpha = block_max(amax[0], s_red);
@@ -170,7 +169,7 @@ __global__ void __launch_bounds__(256, batch_min_blocks<R>()) batch_kernel(const
     }
   }
   if constexpr (sizeof(R) == 4) {
-    if (nfall) atomicAdd(&B.st->fallbacks, nfall);
+    if (nfall) atomicAdd(&st->fallbacks, nfall);
   }
 }
 
@@ -268,10 +267,35 @@ __global__ void batch_check_kernel(const double* U, long long total, double gamm
 
 BatchArgs make_args(enoao_ctx* c, int nsteps, double cfl) {
   BatchState* b = c->batch;
+  const int f32 = c->cfg.precision == ENOAO_FP32_BULK;
+  const bool per_stage = b->nv > 1 && c->cfg.alpha_mode == ENOAO_ALPHA_PER_STAGE;
   BatchArgs a;
   memset(&a, 0, sizeof a);
-  for (int k = 0; k < 3; ++k) a.U[k] = b->U[k];
-  for (int k = 0; k < 2; ++k) a.inc[k] = b->inc[k];
+  for (int stage = 0; stage < 3; ++stage) {
+    SweepArgs& A = a.stage[stage];
+    A.u_in = b->U[stage];
+    A.u0 = b->U[0];
+    A.u_out = b->U[stage == 2 ? 0 : stage + 1];
+    A.inc_in = stage == 0 ? nullptr : b->inc[stage - 1];
+    A.inc_out = stage == 2 ? nullptr : b->inc[stage];
+    A.st = c->st;
+    A.ndim = 1;
+    A.bc = c->cfg.bc[0];
+    A.cstride = b->total;
+    A.stage = stage;
+    A.mode = kModeCombine | (stage == 2 || per_stage ? kModeAlpha : 0);
+    A.ta = 1;
+    A.ts = b->ts;
+    A.se = sweep_row_pitch(b->nv, c->cfg.order, f32, 0, 1, b->ts);
+    A.gamma = c->cfg.gamma;
+    A.adv_speed = c->cfg.adv_speed;
+    A.delta = c->cfg.delta;
+    A.tie_rel = c->cfg.tie_rel;
+    A.inv_dx = 1.0;  // per problem
+    A.redo_passes = 64 * b->nv;
+    set_derived_constants(A);
+    set_component_pointers(A, f32);
+  }
   a.total = b->total;
   a.nprob = b->nprob;
   a.nsteps = nsteps;
@@ -284,14 +308,7 @@ BatchArgs make_args(enoao_ctx* c, int nsteps, double cfl) {
   a.alpha = b->alpha;
   a.dt = b->dt;
   a.queue = b->queue;
-  a.st = c->st;
-  a.ts = b->ts;
-  a.bc = c->cfg.bc[0];
-  a.gamma = c->cfg.gamma;
-  a.adv_speed = c->cfg.adv_speed;
-  a.delta = c->cfg.delta;
-  a.tie_rel = c->cfg.tie_rel;
-  a.per_stage_alpha = c->cfg.alpha_mode == ENOAO_ALPHA_PER_STAGE;
+  a.per_stage_alpha = per_stage;
   return a;
 }
 
@@ -374,8 +391,11 @@ enoao_status batch_create(enoao_ctx* c, const enoao_config* proto, int nprob, co
   b->total = total;
   b->nv = proto->system == ENOAO_EULER ? 3 : 1;
   b->off_h = off;
-  b->ts = 256;
+  // whole rounds: as many extended cells as threads (4096 uneven problems, FP32
+  // bulk: 248 cells on 256 threads 4.85 ms, 256 cells 5.55; 120 on 128 threads
+  // 4.96, and behind by a half where the longest problems set the time)
   b->block = 256;
+  b->ts = b->block - 2 * G;
   c->ncell = total;
   const size_t sb = (size_t)b->nv * total * sizeof(double);
   for (int k = 0; k < 3; ++k) BCU(c, cudaMalloc(&b->U[k], sb));
@@ -521,7 +541,8 @@ enoao_status batch_autotune(enoao_ctx* c) {
     return bfail(c, ENOAO_ENOMEM, "autotune scratch");
   }
   enoao_status r = stream_enter(c);
-  const int cands[][2] = {{128, 128}, {256, 128}, {256, 256}, {512, 256}};
+  const int h = 2 * (c->cfg.order / 2 + 2);  // halo cells of a tile
+  const int cands[][2] = {{128 - h, 128}, {256 - h, 128}, {256 - h, 256}, {512 - h, 256}};
   float best = 1e30f;
   int bts = b->ts, bblk = b->block;
   if (r == ENOAO_OK) {

@@ -1466,6 +1466,7 @@ struct TileConst {
   R alpha;
   float dt32, wdt32;    // FP32 bulk combine: dt and the stage's weight of dt L
   float limit;          // bound of prove_top
+  R inv_dx;
 };
 template <int ORDER, typename R>
 __device__ __forceinline__ void tile_const(const SweepArgs& A, double alpha_d, double dt,
@@ -1473,6 +1474,7 @@ __device__ __forceinline__ void tile_const(const SweepArgs& A, double alpha_d, d
   k.alpha_d = alpha_d;
   k.dt = dt;
   k.alpha = (R)alpha_d;
+  k.inv_dx = bconst<R>(A.inv_dx, A.inv_dx_f);
   k.dt32 = f32_rn(dt);
   k.wdt32 = f32_rn((A.stage == 0 ? 1.0 : (A.stage == 1 ? 0.25 : 2.0 / 3.0)) * dt);
   // below delta by more than the near-tie margin (and the bound's own
@@ -1957,7 +1959,7 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& A, const TileGeo& g,
   constexpr bool FP32 = sizeof(R) == 4;
   constexpr bool PROVE = kProve<FIELD>;
   // the code of faces not proven and of near-ties out of line
-  constexpr bool CALL = FP32 && PROVE && SHAPE != kShapeAny && !COHERENT;
+  constexpr bool CALL = FP32 && PROVE && SHAPE != kShapeAny;
   StepState* st = A.st;
   const int TA = A.ta, TS = A.ts;
   // row pitch A.se (>= TS + 2G), chosen on the host for conflict-free banks
@@ -1995,8 +1997,7 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& A, const TileGeo& g,
   const R delta = bconst<R>(A.delta, A.delta_f);
   const R tie_rel = bconst<R>(A.tie_rel, A.tie_rel_f);
   const int mode = shape_mode<SHAPE>(A);
-  const double inv_dx = A.inv_dx;
-  const R inv_dx_r = bconst<R>(inv_dx, A.inv_dx_f);
+  const R inv_dx_r = K.inv_dx;
   // FP32 bulk combine: dt and the stage's weight of dt L in FP32
   const float dt32 = K.dt32, wdt32 = K.wdt32;
   const float inc_w = A.stage == 1 ? -0.75f : -f32_rn(1.0 / 12.0);  // weight of the carried increment
