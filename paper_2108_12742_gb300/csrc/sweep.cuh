@@ -339,6 +339,36 @@ __device__ __forceinline__ R eno_select(const R (&d)[8], R delta, R tie_rel, con
   return corr;
 }
 
+// The FP64 choice on a window of FP64 differences: the indicators, their
+// comparisons and the bounds of both in FP32 (from the differences rounded
+// once, so an indicator is off by a few FP32 roundings of the magnitudes it
+// sums: 8 eps covers the deepest table), and the choice again in FP64 where
+// those bounds leave it open -- the same choice as FP64 throughout.  The value
+// is FP64.  The FP64 unit, 1/64 of the FP32 rate, is left with the 6 to 8
+// operations of the value instead of some 50 of tables and comparisons.
+template <int ORDER>
+__device__ __forceinline__ double choose64(const double (&d)[8], double delta, float delta_f,
+                                           int& pick) {
+  using GE = Geo<ORDER>;
+  float d32[8], mag[8], sum = 0.0f;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    d32[i] = f32_rn(d[i]);
+    mag[i] = fabsf(d32[i]);
+    sum += mag[i];
+  }
+  bool open;
+  eno_select<ORDER, float, true>(d32, delta_f, 1e-5f, mag, 8.0f * FLT_EPSILON, pick, open);
+  if (open || !(sum < INFINITY)) {
+    const double none[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+    return eno_select<ORDER, double, false>(d, delta, 0.0, none, 0.0, pick, open);
+  }
+  double corr = 0.0;
+#pragma unroll
+  for (int i = GE::LO; i <= GE::HI; ++i) corr = fma(bcoef<double>(pick, i), d[i], corr);
+  return corr;
+}
+
 // Conserved component stored at position c of the permuted state for a sweep
 // along axis dir (momentum along dir first, tangential momenta cyclic).
 template <int NV>
@@ -1560,8 +1590,12 @@ __device__ __forceinline__ unsigned choose_face(const SweepArgs& A, const TileGe
       tv.field_window(a, j, sgn, v, L, w, av, d, mag);
       int pick;
       bool marg = false;
-      R corr = eno_select<ORDER, R, FP32>(d, delta, tie_rel, mag, R(NV + 8) * R(FLT_EPSILON),
-                                          pick, marg);
+      R corr;
+      if constexpr (FP32)
+        corr = eno_select<ORDER, R, true>(d, delta, tie_rel, mag, R(NV + 8) * R(FLT_EPSILON), pick,
+                                          marg);
+      else
+        corr = choose64<ORDER>(d, delta, A.delta_f, pick);
       if constexpr (FP32) {
         if (marg) fix |= 1u << (v * 2 + sgn);  // re-decided in FP64 (phase 2b or the pass)
       }
@@ -1650,9 +1684,12 @@ __device__ __forceinline__ unsigned choose_face_group(const SweepArgs& A, const 
   }
   int pick;
   bool marg = false;
-  const R corr = eno_select<ORDER, R, FP32>(d, bconst<R>(A.delta, A.delta_f),
-                                            bconst<R>(A.tie_rel, A.tie_rel_f), mag,
-                                            R(NV + 8) * R(FLT_EPSILON), pick, marg);
+  R corr;
+  if constexpr (FP32)
+    corr = eno_select<ORDER, R, true>(d, A.delta_f, A.tie_rel_f, mag, R(NV + 8) * R(FLT_EPSILON),
+                                      pick, marg);
+  else
+    corr = choose64<ORDER>(d, A.delta, A.delta_f, pick);
   const bool mine = valid && r < 2 * NV;
   if ((shape_mode<SHAPE>(A) & kModeFlux) && A.idx_out && mine && owns_face(A, g, f))
     A.idx_out[r * A.nfaces + face_index(g, a, f)] = (int8_t)pick;
