@@ -393,17 +393,22 @@ __device__ __forceinline__ T comp_of(const T (&up)[NV], int k, int dir) {
   }
 }
 
+template <int NV, typename T>
+__device__ __forceinline__ T inv_density(const T (&q)[NV]) {
+  return NV > 1 ? brcp(q[0]) : T(0);
+}
+
 // Flux difference F(qb) - F(qa) along the sweep axis, written in differences
 // so that rounding scales with |dq| (Euler: F = [m, m u + p, m_t u, (E+p) u]).
+// ia, ib: 1 / density of the two cells (inv_density), which neighbouring
+// pairs share.
 template <int NV, typename T>
 __device__ __forceinline__ void flux_diff(const T (&qa)[NV], const T (&qb)[NV], const T (&dq)[NV],
-                                          T gm1, T adv, T (&dF)[NV]) {
+                                          T gm1, T adv, T ia, T ib, T (&dF)[NV]) {
   if constexpr (NV == 1) {
     dF[0] = adv * dq[0];
   } else {
     constexpr int NT = NV - 3;  // tangential components
-    const T ia = brcp(qa[0]);
-    const T ib = brcp(qb[0]);
     const T u = qa[1] * ia;
     T vt[NT > 0 ? NT : 1], dvt[NT > 0 ? NT : 1];
     const T du = fma(-u, dq[0], dq[1]) * ib;
@@ -463,9 +468,8 @@ __device__ __forceinline__ void phys_flux(const double (&q)[NV], double gm1, dou
 
 // Roe-average ingredients of one cell: sqrt(rho), velocity, total enthalpy.
 template <int NV, typename T>
-__device__ __forceinline__ void roe_prims(const T (&q)[NV], T gm1, T (&pr)[NV]) {
+__device__ __forceinline__ void roe_prims(const T (&q)[NV], T gm1, T ir, T (&pr)[NV]) {
   if constexpr (NV > 1) {
-    const T ir = brcp(q[0]);
     T ke = T(0);
 #pragma unroll
     for (int i = 1; i < NV - 1; ++i) {
@@ -695,8 +699,8 @@ __device__ __forceinline__ int redo_group(const SweepArgs& A, const TileGeo& g, 
       ql[c] = __shfl_sync(FULL, q[c], G - 1, W);
       qr[c] = __shfl_sync(FULL, q[c], G, W);
     }
-    roe_prims<NV, double>(ql, gm1, pl);
-    roe_prims<NV, double>(qr, gm1, prr);
+    roe_prims<NV, double>(ql, gm1, inv_density<NV>(ql), pl);
+    roe_prims<NV, double>(qr, gm1, inv_density<NV>(qr), prr);
     Eigen<NV, double> E;
     roe_eigen<NV, double>(pl, prr, gm1, E);
     left_row<NV, double>(E, v, L);
@@ -711,7 +715,8 @@ __device__ __forceinline__ int redo_group(const SweepArgs& A, const TileGeo& g, 
     double dq[NV], dF[NV];
 #pragma unroll
     for (int c = 0; c < NV; ++c) dq[c] = qn[c] - q[c];
-    flux_diff<NV, double>(q, qn, dq, gm1, A.adv_speed, dF);
+    const double ia = inv_density<NV>(q), ib = __shfl_down_sync(FULL, ia, 1, W);
+    flux_diff<NV, double>(q, qn, dq, gm1, A.adv_speed, ia, ib, dF);
     const double sa = sgn == 0 ? alpha : -alpha;
 #pragma unroll
     for (int c = 0; c < NV; ++c) w = fma(L[c], 0.5 * fma(sa, dq[c], dF[c]), w);
@@ -754,8 +759,8 @@ __device__ __forceinline__ int redo_lane(const SweepArgs& A, const TileGeo& g, i
     double ql[NV], qr[NV], pl[NV], prr[NV];
     load_cell(G - 1, ql);
     load_cell(G, qr);
-    roe_prims<NV, double>(ql, gm1, pl);
-    roe_prims<NV, double>(qr, gm1, prr);
+    roe_prims<NV, double>(ql, gm1, inv_density<NV>(ql), pl);
+    roe_prims<NV, double>(qr, gm1, inv_density<NV>(qr), prr);
     Eigen<NV, double> E;
     roe_eigen<NV, double>(pl, prr, gm1, E);
     left_row<NV, double>(E, v, L);
@@ -774,12 +779,13 @@ __device__ __forceinline__ int redo_lane(const SweepArgs& A, const TileGeo& g, i
     load_cell(k0, qlo);
     load_cell(k0 + 1, qhi);
   }
+  double ilo = inv_density<NV>(qlo), ihi = inv_density<NV>(qhi);
 #pragma unroll
   for (int i = GE::LO; i <= GE::HI; ++i) {
     double dq[NV], dF[NV];
 #pragma unroll
     for (int c = 0; c < NV; ++c) dq[c] = qhi[c] - qlo[c];
-    flux_diff<NV, double>(qlo, qhi, dq, gm1, A.adv_speed, dF);
+    flux_diff<NV, double>(qlo, qhi, dq, gm1, A.adv_speed, ilo, ihi, dF);
     double w = 0.0;
 #pragma unroll
     for (int c = 0; c < NV; ++c) w = fma(L[c], 0.5 * fma(sa, dq[c], dF[c]), w);
@@ -790,10 +796,14 @@ __device__ __forceinline__ int redo_lane(const SweepArgs& A, const TileGeo& g, i
 #pragma unroll
         for (int c = 0; c < NV; ++c) qlo[c] = qhi[c];
         load_cell(k + 2, qhi);
+        ilo = ihi;
+        ihi = inv_density<NV>(qhi);
       } else {
 #pragma unroll
         for (int c = 0; c < NV; ++c) qhi[c] = qlo[c];
         load_cell(k - 1, qlo);
+        ihi = ilo;
+        ilo = inv_density<NV>(qlo);
       }
     }
   }
@@ -898,11 +908,11 @@ struct CellVec {
 template <int NV, typename R>
 __device__ __forceinline__ R split_diff(const double (&qa64)[NV], const double (&qb64)[NV],
                                         const R (&qa)[NV], const R (&qb)[NV], R gm1, R adv,
-                                        R halpha, R (&fp)[NV], R (&fm)[NV]) {
+                                        R halpha, R ia, R ib, R (&fp)[NV], R (&fm)[NV]) {
   R dq[NV], dF[NV], m = R(0);
 #pragma unroll
   for (int c = 0; c < NV; ++c) dq[c] = to_bulk<R>(qb64[c] - qa64[c]);
-  flux_diff<NV, R>(qa, qb, dq, gm1, adv, dF);
+  flux_diff<NV, R>(qa, qb, dq, gm1, adv, ia, ib, dF);
 #pragma unroll
   for (int c = 0; c < NV; ++c) {
     const R hdF = R(0.5) * dF[c];
@@ -918,11 +928,11 @@ __device__ __forceinline__ R split_diff(const double (&qa64)[NV], const double (
 template <int NV, typename R>
 __device__ __forceinline__ void split_parts(const double (&qa64)[NV], const double (&qb64)[NV],
                                             const R (&qa)[NV], const R (&qb)[NV], R gm1, R adv,
-                                            R (&hdF)[NV], R (&hdq)[NV]) {
+                                            R ia, R ib, R (&hdF)[NV], R (&hdq)[NV]) {
   R dq[NV], dF[NV];
 #pragma unroll
   for (int c = 0; c < NV; ++c) dq[c] = to_bulk<R>(qb64[c] - qa64[c]);
-  flux_diff<NV, R>(qa, qb, dq, gm1, adv, dF);
+  flux_diff<NV, R>(qa, qb, dq, gm1, adv, ia, ib, dF);
 #pragma unroll
   for (int c = 0; c < NV; ++c) {
     hdF[c] = R(0.5) * dF[c];
@@ -2074,11 +2084,11 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& A, const TileGeo& g,
       }
     };
     // cell e's Roe ingredients, and the split differences of the pair (e, e+1)
-    auto prim_out = [&](int a, int e, const R (&qa)[NV]) {
+    auto prim_out = [&](int a, int e, const R (&qa)[NV], R ir) {
       if constexpr (NV > 1) {
         if (e >= G - 1 && e <= G + nts) {
           R pr[NV];
-          roe_prims<NV, R>(qa, gm1, pr);
+          roe_prims<NV, R>(qa, gm1, ir, pr);
           if constexpr (CV::kSpare) {
             dfm[4 * sidx(a, e) + 3] = pr[0];
             Cf[4 * sidx(a, e) + 3] = pr[1];
@@ -2090,12 +2100,12 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& A, const TileGeo& g,
       }
     };
     auto pair_out = [&](int a, int e, const double (&qa64)[NV], const R (&qa)[NV],
-                        const double (&qb64)[NV], const R (&qb)[NV]) {
+                        const double (&qb64)[NV], const R (&qb)[NV], R ia, R ib) {
       R fp[NV], fm[NV], m = R(0);
       if constexpr (FIELD)
-        split_parts<NV, R>(qa64, qb64, qa, qb, gm1, adv, fp, fm);  // dF/2, dq/2
+        split_parts<NV, R>(qa64, qb64, qa, qb, gm1, adv, ia, ib, fp, fm);  // dF/2, dq/2
       else
-        m = split_diff<NV, R>(qa64, qb64, qa, qb, gm1, adv, halpha, fp, fm);
+        m = split_diff<NV, R>(qa64, qb64, qa, qb, gm1, adv, halpha, ia, ib, fp, fm);
       if constexpr (CV::kSpare) {
         CV::store4(dfp, sidx(a, e), fp, m);
         CV::store(dfm, cells, sidx(a, e), fm);  // its spare value: a Roe ingredient
@@ -2114,14 +2124,15 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& A, const TileGeo& g,
         R qa[NV];
 #pragma unroll
         for (int c = 0; c < NV; ++c) qa[c] = to_bulk<R>(qa64[c]);
-        prim_out(a, e, qa);
+        const R ia = inv_density<NV>(qa);
+        prim_out(a, e, qa, ia);
         if (e + 1 < cnt) {
           double qb64[NV];
           cell_state(a, e + 1, qb64);
           R qb[NV];
 #pragma unroll
           for (int c = 0; c < NV; ++c) qb[c] = to_bulk<R>(qb64[c]);
-          pair_out(a, e, qa64, qa, qb64, qb);
+          pair_out(a, e, qa64, qa, qb64, qb, ia, inv_density<NV>(qb));
         }
       });
     } else {
@@ -2140,16 +2151,19 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& A, const TileGeo& g,
         R q[NV];
 #pragma unroll
         for (int c = 0; c < NV; ++c) q[c] = to_bulk<R>(q64[c]);
+        R ir = inv_density<NV>(q);
         for (;; ++e) {
-          prim_out(a, e, q);
+          prim_out(a, e, q, ir);
           if (e + 1 >= cnt) break;
           double n64[NV];
           cell_state(a, e + 1, n64);
           R n[NV];
 #pragma unroll
           for (int c = 0; c < NV; ++c) n[c] = to_bulk<R>(n64[c]);
-          pair_out(a, e, q64, q, n64, n);
+          const R in = inv_density<NV>(n);
+          pair_out(a, e, q64, q, n64, n, ir, in);
           if (e + 1 >= e_end) break;
+          ir = in;
 #pragma unroll
           for (int c = 0; c < NV; ++c) {
             q64[c] = n64[c];
@@ -2749,8 +2763,8 @@ __device__ __forceinline__ void face_change32(const SweepArgs& A, const TileGeo&
       ql[c] = to_bulk<float>(ql64[c]);  // the sweep's phase-1 narrowing
       qr[c] = to_bulk<float>(qr64[c]);
     }
-    roe_prims<NV, float>(ql, gm1, pl);
-    roe_prims<NV, float>(qr, gm1, prr);
+    roe_prims<NV, float>(ql, gm1, inv_density<NV>(ql), pl);
+    roe_prims<NV, float>(qr, gm1, inv_density<NV>(qr), prr);
     Eigen<NV, float> E;
     roe_eigen<NV, float, true>(pl, prr, gm1, E);
     left_row<NV, float>(E, v, L);
@@ -2776,7 +2790,8 @@ __device__ __forceinline__ void face_change32(const SweepArgs& A, const TileGeo&
       qa[c] = to_bulk<float>(qa64[c]);
       qb[c] = to_bulk<float>(qb64[c]);
     }
-    split_diff<NV, float>(qa64, qb64, qa, qb, gm1, adv, halpha, fp, fm);
+    split_diff<NV, float>(qa64, qb64, qa, qb, gm1, adv, halpha, inv_density<NV>(qa),
+                          inv_density<NV>(qb), fp, fm);
 #pragma unroll
     for (int c = 0; c < NV; ++c) x[c] = sgn == 0 ? fp[c] : fm[c];
     float acc = 0.0f;
