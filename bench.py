@@ -38,6 +38,9 @@ FLOPS_PER_FACE = 1150       # flops of one face of one axis, 2D Euler ENO-AO5 (t
                             # operation count: split, Roe eigen-system, projection of both
                             # windows, indicators, selection, back-projection)
 FLOPS_PER_FACE_COUNTED = 885  # the same path counted operation by operation in the kernel
+# FP64-unit instructions of one cell of the FP64 y sweep (2D Euler ENO-AO5, stage 0, evolved data,
+# counted by the profiler; the choices are decided in FP32), two flops each at the unit's peak
+FP64_INST_PER_CELL_Y = 143
 # y sweep, stage 0: read U^n (FP64) and L_x (FP32), write U1 (FP64) and the
 # FP32 increment I0 the later stages combine with
 BYTES_PER_CELL_Y = 32 + 16 + 32 + 16
@@ -404,10 +407,12 @@ def run_gpu(args):
                         "frac": BYTES_PER_CELL_Y * cells / t_dom / 1e9 / peaks["hbm_gbs"],
                         "algorithmic_bytes_per_launch": BYTES_PER_CELL_Y * cells,
                         "peak_kind": peak_kind}}
-    # the FP64 path's y sweep against the measured FP64 multiply-add rate
-    a64 = flops / (k_ms64[dom] / 1e3) / 1e12
+    # the FP64 path's y sweep against the measured FP64 multiply-add rate: the instructions it
+    # issues to the FP64 unit, each as a multiply-add
+    a64 = 2 * FP64_INST_PER_CELL_Y * cells / (k_ms64[dom] / 1e3) / 1e12
     roofline64 = {"bound": "fp64 alu", "achieved": a64, "peak": fma["fp64"], "unit": "TFLOP/s",
                   "frac": a64 / fma["fp64"], "kernel_ms": k_ms64[dom],
+                  "fp64_instructions_per_cell": FP64_INST_PER_CELL_Y,
                   "peak_kind": "measured: FP64 multiply-add microbenchmark on this GPU"}
 
     launches = (s32.launches_per_step() * args.steps) if rank == 0 else 0

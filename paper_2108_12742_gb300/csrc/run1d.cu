@@ -7,7 +7,8 @@
 // also paid for a launch, the sweep's prologue and a bookkeeping node (39 us a
 // step at N = 2000, FP64), and steps came in multiples of 32 to 128.  Here a
 // tile per SM spreads the cells thinnest, the barrier is one atomic and one
-// poll, and the launch ends with the run.
+// poll, and the launch ends with the run.  Advection N = 200 to t = 2 (401
+// steps) 9.0 -> 5.2 ms, Euler N = 2000 over 120 steps 10.0 -> 5.8 ms.
 //
 // Every block is resident (a cooperative launch of at most a block per SM), so
 // the barrier cannot wait for a block that has not started; its polls are
@@ -124,11 +125,15 @@ cudaError_t launch_one(const Run1dArgs& a, int block, int sms, cudaStream_t s) {
 
 }  // namespace
 
-// Small scalar problems stay in one block (a stage is a few hundred simple
-// operations, less than a grid barrier); otherwise a tile per SM, of at least
-// 15 cells (16 faces: the face groups of a tile fill one round of 128 threads).
+// Scalar problems whose extended cells fit one block's threads once stay in one
+// block: a stage is less than a grid barrier there (N = 200: 13.3 us a step, 15.3
+// in tiles of 63; N = 400: 19.0 in one block, 14.7 in tiles of 63, 18.5 of 15).
+// The Euler equations take a tile per SM, of at least 15 cells (16 faces: the
+// face groups of a tile fill one round of 128 threads).
 void run1d_tile(int nv, long long n, int sms, int* ts, int* block) {
-  long long t = nv == 1 && n <= kRun1dMaxTile * 2 ? n : std::max<long long>(15, (n + sms - 1) / sms);
+  const long long per_sm = (n + sms - 1) / sms;
+  long long t = nv == 1 ? (n <= 246 ? n : std::max<long long>(63, per_sm))
+                        : std::max<long long>(15, per_sm);
   *ts = (int)t;
   *block = t > 120 ? 256 : 128;
 }

@@ -8,7 +8,10 @@
 //            flux difference dF in difference form, Lax-Friedrichs split
 //            differences df+- = (dF +- alpha dU)/2 (Sec. 2, Eq. LF_Flux_Split);
 //            per cell: Roe-average ingredients (sqrt rho, velocity, H).
-//   phase 2  per face x_{j+1/2}: Roe average and eigenvectors (Sec. 4),
+//   phase 2a per face: one bound per field and sign shows most faces to take
+//            the top candidate everywhere and gives them their correction;
+//            the others go to the tile's face list (prove_top).
+//   phase 2  per listed face x_{j+1/2}: Roe average and eigenvectors (Sec. 4),
 //            projection of the window differences onto each characteristic
 //            field, indicators IS = MIN(delta_L, delta_R) as undivided
 //            differences (Eq. New_Smoothness_Indicator, Tables 4-5), stencil
@@ -345,7 +348,9 @@ __device__ __forceinline__ R eno_select(const R (&d)[8], R delta, R tie_rel, con
 // sums: 8 eps covers the deepest table), and the choice again in FP64 where
 // those bounds leave it open -- the same choice as FP64 throughout.  The value
 // is FP64.  The FP64 unit, 1/64 of the FP32 rate, is left with the 6 to 8
-// operations of the value instead of some 50 of tables and comparisons.
+// operations of the value instead of some 50 of tables and comparisons (scalar
+// ENO-AO7 fluxes of 4096 x 2048 cells 1.86 -> 1.02 ms, a 97 x 80 x 63 Euler step,
+// hardly any of whose faces are proven, 9.1 -> 6.7 ms).
 template <int ORDER>
 __device__ __forceinline__ double choose64(const double (&d)[8], double delta, float delta_f,
                                            int& pick) {
@@ -359,7 +364,7 @@ __device__ __forceinline__ double choose64(const double (&d)[8], double delta, f
   }
   bool open;
   eno_select<ORDER, float, true>(d32, delta_f, 1e-5f, mag, 8.0f * FLT_EPSILON, pick, open);
-  if (open || !(sum < INFINITY)) {
+  if (open || !(sum < INFINITY) || !(delta_f >= 1e-30f)) {
     const double none[8] = {0, 0, 0, 0, 0, 0, 0, 0};
     return eno_select<ORDER, double, false>(d, delta, 0.0, none, 0.0, pick, open);
   }
@@ -1032,7 +1037,8 @@ __device__ __forceinline__ int shape_mode(const SweepArgs& A) {
 
 // FP64 path: whether FP32 bounds show a new state to be physical and, when the
 // next alpha is being taken, its |u_d| + c to be no more than the maxima so
-// far.  The margins (1e-5 and 1e-6 of the summed magnitudes) cover the FP32
+// far (some 33 FP64 operations per cell of a combining sweep otherwise, of about
+// 190; 2048^2 step 8.60 -> 8.08 ms).  The margins (1e-5 and 1e-6 of the summed magnitudes) cover the FP32
 // rounding of every operation; NaN, infinities and values beyond FP32's range
 // are never shown.
 template <int NV, int KA>
@@ -1262,7 +1268,13 @@ __device__ __forceinline__ void face_eigen(const TileView<NV, ORDER, R, FIELD>& 
 // near-tie margin, principle 1 of Sec. 3.2 picks the top candidate without a
 // near-tie.  One difference decides a field instead of two per candidate and
 // their bounds; the faces of resolved flow end here (98 to 99.5 % of 2D data
-// at 2048^2 and more), the others go to the tile's face list.
+// at 2048^2 and more), the others go to the tile's face list.  The sweeps are
+// bound by issue slots: 1,440 instructions per face and cell before, 840 (x)
+// and 1,120 (y) with it; 4096^2 ENO-AO5 sweeps 0.81 -> 0.52 ms (x, 2 x 120
+// tiles) and 1.00 -> 0.69 ms (y, 16 x 15), 512^3 ENO-AO7 stage 53 -> 27 ms.
+// (Without the projection, as the FP64 path does it, they took 0.41 and 0.60
+// ms; but R (L s) and s differ by FP32 rounding, which later stages' near-ties
+// turn into other choices.)
 template <int NV, int ORDER, bool FIELD>
 __device__ __forceinline__ bool prove_top(const TileView<NV, ORDER, float, FIELD>& tv, int x,
                                           float gm1, float limit, float (&C)[NV]) {
@@ -1395,6 +1407,8 @@ __device__ __forceinline__ bool prove_top(const TileView<NV, ORDER, float, FIELD
 // (gamma-1) H / c^2 -- goes through the FP64 indicators as before.  With every
 // field on the top candidate R L = I, so the values need no projection: C is
 // a sum of FP64 differences, 8 NV (ENO-AO7: 12 NV) operations instead of 500.
+// 2048^2 ENO-AO5 sweeps: x 4.15 -> 1.13 ms, y 4.38 -> 1.20 ms (with choose64
+// and the neighbours' shared 1 / density).
 template <int NV, int ORDER, bool FIELD>
 __device__ __forceinline__ bool prove_top(const TileView<NV, ORDER, double, FIELD>& tv, int x,
                                           float gm1, float limit, double (&C)[NV]) {
@@ -1518,8 +1532,10 @@ __device__ __forceinline__ void tile_const(const SweepArgs& A, double alpha_d, d
   k.dt32 = f32_rn(dt);
   k.wdt32 = f32_rn((A.stage == 0 ? 1.0 : (A.stage == 1 ? 0.25 : 2.0 / 3.0)) * dt);
   // below delta by more than the near-tie margin (and the bound's own
-  // rounding); FP64 has no near-ties and takes a margin of its own
-  k.limit = A.delta_f - fmaf(sizeof(R) == 4 ? A.tie_rel_f : 1e-3f, A.delta_f, 1e-3f * A.delta_f);
+  // rounding); FP64 has no near-ties and takes a margin of its own.  A delta
+  // near the end of FP32's range, where narrowed differences vanish, proves
+  // nothing.
+  k.limit = !(A.delta_f >= 1e-30f) ? -1.0f : A.delta_f - fmaf(sizeof(R) == 4 ? A.tie_rel_f : 1e-3f, A.delta_f, 1e-3f * A.delta_f);
 }
 
 // Whether the tile is the one that writes face f (the face between two tiles
@@ -1643,7 +1659,9 @@ constexpr int kFaceLanes = NV == 1 ? 2 : (NV <= 4 ? 8 : 16);
 // an aligned group, lane r taking field r / 2, sign r % 2 (the operations of
 // choose_face, so the same bits): a tile's list is mostly a few faces, which
 // one per thread would leave to a few lanes, each with ten dependent
-// selections.  Every lane of the warp calls it; valid is the same over a group.
+// selections (FP64 1D sweep of 2000 cells 31 -> 19 us).  Lists longer than one
+// round of groups go one face per lane, where no lane idles and the face's
+// eigenvectors are formed once.  Every lane of the warp calls it; valid is the same over a group.
 template <int NV, int ORDER, typename R, bool COHERENT, int SHAPE>
 __device__ __forceinline__ unsigned choose_face_group(const SweepArgs& A, const TileGeo& g,
                                                       const TileView<NV, ORDER, R, false>& tv,
@@ -1845,7 +1863,9 @@ __device__ __forceinline__ void redecide_tile(const SweepArgs& A, const TileGeo&
       const int al = entry_line(entry), f = entry_face(entry);
       const int j = G - 1 + f;
       unsigned fix = entry_flags(entry);
-      // The warp's T choices in rounds.  Many left: one per lane (redo_lane),
+      // The warp's T choices in rounds (with each face's lane serving its own
+      // flags, a warp took up to ten rounds for a few choices each: 256^3
+      // ENO-AO7 x sweep 1.8 -> 1.0 ms, 800^2 0.23 -> 0.16 ms).  Many left: one per lane (redo_lane),
       // 32 in a round -- an instruction of the FP64 unit costs the same
       // whatever its active lanes.  A few left: NG per round, each by W lanes
       // together (redo_group), which takes about 2/5 (ENO-AO5) or 1/3 of the
@@ -2435,7 +2455,9 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& A, const TileGeo& g,
 }
 
 // Minimum resident blocks per SM asked of the compiler for the FP32-bulk
-// sweep (caps its registers at 65536 / (128 * min blocks)).
+// sweep (caps its registers at 65536 / (128 * min blocks): 64, a few spilled
+// around the out-of-line calls).  Six, eight and ten were within 5 % of one
+// another on 4096^2 and 256^3 data; eight led on most tiles.
 #ifndef ENOAO_FP32_MIN_BLOCKS
 #define ENOAO_FP32_MIN_BLOCKS 8
 #endif

@@ -89,3 +89,24 @@ def test_short_and_long_lists_give_the_same_bits(order, precision):
             outs.append(s.reconstruct_fluxes(0, want_idx=True))
     for F, idx in outs[1:]:
         assert np.array_equal(F, outs[0][0]) and np.array_equal(idx, outs[0][1])
+
+
+@pytest.mark.parametrize("delta", [0.0, 1e-40, 1e-3])
+@pytest.mark.parametrize("precision", [eno.FP64, eno.FP32_BULK])
+def test_other_thresholds_match_oracle(delta, precision):
+    # a threshold of zero, one below FP32's normal range, and a coarse one
+    U = np.ascontiguousarray(_data("euler2d", 4e-6, seed=11))
+    shape = SHAPES["euler2d"]
+    P = oracle.make_problem(shape, (0.0, 0.0), (1.0, 1.0), delta=delta, **_kw("euler2d", 5))
+    with eno.Solver(shape, (0.0, 0.0), (1.0, 1.0), precision=precision, delta=delta,
+                    **_kw("euler2d", 5)) as s:
+        s.init_state(U)
+        for d in range(2):
+            F, idx = s.reconstruct_fluxes(d, want_idx=True)
+            Fo, io, gap = oracle.fluxes(P, U, d, want_idx=True)
+            differ = idx != io
+            if precision == eno.FP64:
+                assert not (differ & (gap > TIE)).any(), (d, int(differ.sum()))
+            rel = np.abs(F - Fo) / np.abs(Fo).max()
+            ok = ~differ.any(axis=(0, 1))
+            assert rel[:, ok].max() <= (TOL64 if precision == eno.FP64 else TOL32), d

@@ -25,10 +25,10 @@ def _solver(system, n, order, precision, bc):
 
 
 # 11: the least; 15/16/17: one tile, the first with two; 2281: tiles of 16 on
-# 152 SMs; 512/513: the last scalar problem in one block; 18241: tiles past
+# 152 SMs; 246/247: the last scalar problem in one block; 18241: tiles past
 # 120 cells (256 threads); 38912/38913: the last persistent one, and one beyond
 @pytest.mark.parametrize("system,sizes", [(eno.EULER, (11, 15, 16, 17, 333, 2281, 18241, 38912, 38913)),
-                                          (eno.SCALAR_ADVECTION, (11, 121, 512, 513, 2281))])
+                                          (eno.SCALAR_ADVECTION, (11, 121, 246, 247, 513, 18241))])
 @pytest.mark.parametrize("order", [5, 7])
 @pytest.mark.parametrize("precision", [eno.FP64, eno.FP32_BULK])
 def test_persistent_run_equals_stages(system, sizes, order, precision):
