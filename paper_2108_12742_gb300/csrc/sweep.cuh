@@ -492,10 +492,7 @@ struct Eigen {
   T u, vt[NV > 3 ? NV - 3 : 1], H, c, ic, b1, b2, q2;
 };
 
-// PASS: the grid-wide pass's form, which fuses the other product of |v|^2 in
-// 2D; results of that mode keep its bits (a choice within a last-bit rounding
-// of a tie can then be taken as changed, or not, by the pass alone).
-template <int NV, typename T, bool PASS = false>
+template <int NV, typename T>
 __device__ __forceinline__ void roe_eigen(const T (&pl)[NV], const T (&prr)[NV], T gm1,
                                           Eigen<NV, T>& E) {
   constexpr int NT = NV - 3;
@@ -507,8 +504,7 @@ __device__ __forceinline__ void roe_eigen(const T (&pl)[NV], const T (&prr)[NV],
   T q2;
   if constexpr (NT < 2) {
     q2 = mul_rn(E.u, E.u);
-    if constexpr (NT == 1)
-      q2 = PASS ? dot2(E.u, E.u, E.vt[0], E.vt[0]) : fma(E.vt[0], E.vt[0], q2);
+    if constexpr (NT == 1) q2 = fma(E.vt[0], E.vt[0], q2);
   } else {
     q2 = fma(E.vt[1], E.vt[1], dot2(E.u, E.u, E.vt[0], E.vt[0]));
   }
@@ -2788,7 +2784,7 @@ __device__ __forceinline__ void face_change32(const SweepArgs& A, const TileGeo&
     roe_prims<NV, float>(ql, gm1, inv_density<NV>(ql), pl);
     roe_prims<NV, float>(qr, gm1, inv_density<NV>(qr), prr);
     Eigen<NV, float> E;
-    roe_eigen<NV, float, true>(pl, prr, gm1, E);
+    roe_eigen<NV, float>(pl, prr, gm1, E);
     left_row<NV, float>(E, v, L);
     right_col<NV, float>(E, v, Rc);
     if constexpr (NV >= 4) w = -L[0];

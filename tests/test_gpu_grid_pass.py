@@ -1,0 +1,49 @@
+"""The grid-wide re-decision pass against the in-sweep re-decisions: both end with
+the FP64 choice of every near-tie, so one stage from one state agrees to FP32
+rounding.  The pass re-derives the FP32 choice that the sweep made; derived with
+other roundings, a tie within them gets its change twice or not at all, and the
+cells beside the face are off by the difference of two candidates' values."""
+import numpy as np
+import pytest
+
+import paper_2108_12742_gb300 as eno
+from paper_2108_12742_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+# Either way a cell's increment is some ten FP32 operations (2^-24 each) on four
+# terms of the size of the largest increment, on up to three axes: 120 x 2^-24 = 7e-6.
+TOL = 1e-5
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _gpu():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2108_12742_gb300 import build
+    build.build()
+
+
+@pytest.mark.parametrize("order", [5, 7])
+@pytest.mark.parametrize("shape", [(200000,), (1024, 1024), (60, 60, 60)])
+def test_grid_pass_ends_with_the_choices_of_the_sweep(shape, order):
+    # white noise: among the choices of so many faces (33 million on the plane)
+    # tens are ties to the last bits
+    nd = len(shape)
+    rng = np.random.default_rng(order)
+    full = tuple(reversed(shape + (1,) * (3 - nd)))
+    rho, p, *vel = (b + 0.3 * rng.uniform(-1, 1, full) for b in [1.0, 1.0] + [0.2] * nd)
+    U = np.ascontiguousarray(inputs.conserved(rho, vel, p, 1.4).reshape((nd + 2,) + full))
+    out = []
+    for mode in (eno.REDECIDE_GRID, eno.REDECIDE_IN_SWEEP):
+        with eno.Solver(shape, (0.0,) * nd, (1.0,) * nd, system=eno.EULER, order=order,
+                        precision=eno.FP32_BULK, bc=eno.PERIODIC) as s:
+            s.set_redecide(mode)
+            s.init_state(U)
+            s.rk_stage(0, 0.1 / max(shape))
+            out.append(s.get_stage_state(1))
+            assert s.stats().fp64_fallbacks > 0
+    grid, sweep = out
+    off = np.abs(grid - sweep).max(axis=0) / np.abs(sweep - U).max()
+    assert off.max() <= TOL, (off.max(), int((off > TOL).sum()))
