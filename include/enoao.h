@@ -338,6 +338,15 @@ enoao_status enoao_set_fused_stage(enoao_ctx *ctx, int on, int x_lines, int x_ce
  * batched contexts and for limits below -1. */
 enoao_status enoao_set_redecide_pass_limit(enoao_ctx *ctx, int passes);
 
+/* Fault-injection knob for tests: bounds the polls of a block waiting for the
+ * others between the stages of a persistent 1D run (the default, -1, is a few
+ * seconds of them).  A block that reaches a smaller bound sets the device error
+ * word and leaves, and so do the others at their next wait; the call returns
+ * ENOAO_ETIMEOUT, the step they were in is not counted and the state is
+ * undefined.  Until enoao_init_state, further runs return ENOAO_ETIMEOUT at
+ * once.  ENOAO_EINVAL for batched contexts and for limits below -1. */
+enoao_status enoao_set_run_poll_limit(enoao_ctx *ctx, int polls);
+
 /* One third-order TVD Runge-Kutta step of a 1D problem that allocates no
  * device memory.  The paper has no counterpart: this is a deployment aid for
  * callers that cannot let a library allocate -- applications that reserve

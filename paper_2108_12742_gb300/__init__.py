@@ -107,6 +107,7 @@ def load():
         "enoao_set_redecide": (ctypes.c_int, [P, ctypes.c_int]),
         "enoao_uses_grid_redecide": (ctypes.c_int, [P]),
         "enoao_set_redecide_pass_limit": (ctypes.c_int, [P, ctypes.c_int]),
+        "enoao_set_run_poll_limit": (ctypes.c_int, [P, ctypes.c_int]),
         "enoao_set_tma": (ctypes.c_int, [P, ctypes.c_int]),
         "enoao_set_fused_stage": (ctypes.c_int, [P, ctypes.c_int, ctypes.c_int, ctypes.c_int,
                                                  ctypes.c_int, ctypes.c_int]),
@@ -338,6 +339,11 @@ class Solver:
     def set_redecide_pass_limit(self, passes):
         """Test knob: bound on the in-sweep FP64 re-decision passes (-1: default)."""
         self._check(self._lib.enoao_set_redecide_pass_limit(self._h, passes))
+
+    def set_run_poll_limit(self, polls):
+        """Test knob: bound on a block's polls between the stages of a persistent 1D run
+        (-1: default)."""
+        self._check(self._lib.enoao_set_run_poll_limit(self._h, polls))
 
     def uses_grid_redecide(self):
         return bool(self._lib.enoao_uses_grid_redecide(self._h))

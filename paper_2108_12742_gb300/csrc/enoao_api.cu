@@ -642,7 +642,7 @@ enoao_status check_err(enoao_ctx* c) {
   if (c->st_host->err & kErrNonPhys)
     return fail(c, ENOAO_ENONPHYS, "non-physical state (rho <= 0, p <= 0 or NaN) at cell %lld",
                 (long long)c->st_host->err_cell);
-  if (c->st_host->err & kErrTimeout) return fail(c, ENOAO_ETIMEOUT, "device wait timed out");
+  if (c->st_host->err & (kErrTimeout | kErrBarrier)) return fail(c, ENOAO_ETIMEOUT, "device wait timed out");
   if (c->st_host->err & kErrRedoFull)
     return fail(c, ENOAO_ECUDA, "internal error: re-decision list overflow");
   return ENOAO_OK;
@@ -1118,6 +1118,7 @@ static enoao_status enqueue_run1d(enoao_ctx* c, long long cap) {
   }
   a.k = consts(c);
   a.cap = cap;
+  a.polls = c->run_polls >= 0 ? (unsigned)c->run_polls : kRun1dPolls;
   const cudaError_t e = run1d_launch(c->nv, c->cfg.order, fp32(c), a, block, c->sms, c->s);
   if (e != cudaSuccess) return fail(c, ENOAO_ECUDA, "1D run launch: %s", cudaGetErrorString(e));
   return ENOAO_OK;
@@ -1218,7 +1219,8 @@ enoao_status enoao_get_stats(enoao_ctx* c, enoao_stats* out) {
   if (c->batch) return batch_stats(c, out);
   enoao_status r = read_host_state(c);
   if (r != ENOAO_OK) return r;
-  const StepState& h = *c->st_host;
+  StepState& h = *c->st_host;
+  if (h.err & kErrBarrier) h.pending = 0;  // as finalize_pending
   out->t = h.pending ? (h.last ? h.t_end : h.t + h.dt) : h.t;
   out->steps = h.steps + (h.pending ? 1 : 0);
   for (int d = 0; d < 3; ++d) out->alpha[d] = h.alpha[d];
@@ -1306,6 +1308,14 @@ enoao_status enoao_set_redecide_pass_limit(enoao_ctx* c, int passes) {
     cudaGraphExecDestroy(c->graph);
     c->graph = nullptr;
   }
+  return ENOAO_OK;
+}
+
+enoao_status enoao_set_run_poll_limit(enoao_ctx* c, int polls) {
+  if (!c) return fail(c, ENOAO_EINVAL, "NULL context");
+  if (c->batch) return fail(c, ENOAO_EINVAL, "not available for batched contexts");
+  if (polls < -1) return fail(c, ENOAO_EINVAL, "poll limit must be >= 0, or -1 for the default");
+  c->run_polls = polls;
   return ENOAO_OK;
 }
 

@@ -51,6 +51,8 @@ constexpr int kBcHalo = 2;
 constexpr int kErrNonPhys = 1;
 constexpr int kErrTimeout = 2;
 constexpr int kErrRedoFull = 4;  // re-decision list full (cannot happen: one slot per face)
+constexpr int kErrBarrier = 8;   // a block of a persistent 1D run gave up at the grid barrier:
+                                 // the pending step is not complete
 
 // Modes of a sweep launch (bit set).
 constexpr int kModeRhsStore = 1;   // write this axis' L(u) into rhs

@@ -13,6 +13,9 @@
 // Every block is resident (a cooperative launch of at most a block per SM), so
 // the barrier cannot wait for a block that has not started; its polls are
 // bounded all the same: a block that gives up sets the error word and leaves.
+// The others then run out of polls at the next barrier, which it never reaches.
+// The barrier's count is left short: until the state is set anew (which clears
+// it) a launch finds the error word and leaves at once.
 #include <algorithm>
 
 #include "run1d.h"
@@ -22,8 +25,6 @@ namespace enoao {
 
 namespace {
 
-constexpr unsigned kBarrierPolls = 1u << 22;  // a few seconds
-
 __device__ __forceinline__ unsigned load_acquire(const unsigned* p) {
   unsigned v;
   asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
@@ -32,7 +33,7 @@ __device__ __forceinline__ unsigned load_acquire(const unsigned* p) {
 
 // All threads of all blocks; false when the wait ran out.  What a block wrote
 // before it (any thread) is seen by every block's L2 reads after it.
-__device__ __forceinline__ bool grid_barrier(StepState* st) {
+__device__ __forceinline__ bool grid_barrier(StepState* st, unsigned limit) {
   __shared__ bool s_ok;
   __syncthreads();
   if (gridDim.x == 1) {
@@ -49,8 +50,8 @@ __device__ __forceinline__ bool grid_barrier(StepState* st) {
       atomicAdd(&st->grid_gen, 1u);
     } else {
       unsigned polls = 0;
-      while (load_acquire(&st->grid_gen) == gen && ok) ok = ++polls < kBarrierPolls;
-      if (!ok) atomicOr(&st->err, kErrTimeout);
+      while (load_acquire(&st->grid_gen) == gen && ok) ok = polls++ < limit;
+      if (!ok) atomicOr(&st->err, kErrBarrier);
     }
     __threadfence();
     s_ok = ok;
@@ -68,12 +69,17 @@ __global__ void __launch_bounds__(256, 1) run1d_kernel(const __grid_constant__ R
   __shared__ double s_red[8];
   StepState* st = P.stage[0].st;
   unsigned long long nfall = 0;
-  if (threadIdx.x == 0) s_geo = tile_geo(P.stage[0], blockIdx.x);
+  if (threadIdx.x == 0) {
+    s_geo = tile_geo(P.stage[0], blockIdx.x);
+    s_skip = __ldcg(&st->err) & kErrBarrier;
+  }
+  __syncthreads();
+  if (s_skip) return;
   bool ok = true;
   long long n = 0;
   for (; n < P.cap; ++n) {
     if (blockIdx.x == 0 && threadIdx.x == 0) begin_step(st, P.k);
-    ok = grid_barrier(st);
+    ok = grid_barrier(st, P.polls);
     if (!ok) break;
     if (threadIdx.x == 0) {
       s_skip = __ldcg(&st->skip);
@@ -101,7 +107,7 @@ __global__ void __launch_bounds__(256, 1) run1d_kernel(const __grid_constant__ R
             atomicMax(&st->alpha_acc[s_par][0], (unsigned long long)__double_as_longlong(v));
         }
       }
-      ok = grid_barrier(st);
+      ok = grid_barrier(st, P.polls);
     }
     if (!ok) break;
   }

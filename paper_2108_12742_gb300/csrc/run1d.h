@@ -12,9 +12,11 @@ struct Run1dArgs {
   SweepArgs stage[3];  // the sweeps of the three Runge-Kutta stages
   StepConsts k;
   long long cap;       // steps of this launch at most
+  unsigned polls;      // bound on a block's polls of the grid barrier
 };
 
 constexpr int kRun1dMaxTile = 256;
+constexpr unsigned kRun1dPolls = 1u << 22;  // a few seconds
 
 // Cells per tile and threads per block for a problem of n cells.
 void run1d_tile(int nv, long long n, int sms, int* ts, int* block);

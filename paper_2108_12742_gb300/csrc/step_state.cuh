@@ -17,6 +17,7 @@ struct StepConsts {
 };
 
 __device__ inline void finalize_pending(StepState* st) {
+  if (st->err & kErrBarrier) st->pending = 0;
   if (st->pending) {
     st->t = st->last ? st->t_end : st->t + st->dt;
     st->steps += 1;
