@@ -347,6 +347,12 @@ enoao_status enoao_set_redecide_pass_limit(enoao_ctx *ctx, int passes);
  * once.  ENOAO_EINVAL for batched contexts and for limits below -1. */
 enoao_status enoao_set_run_poll_limit(enoao_ctx *ctx, int polls);
 
+/* Knob for tests: bounds the blocks of a persistent 1D run (the default, -1,
+ * leaves it to the device).  A run that needs more, or more than the device
+ * holds at once, goes as CUDA-graph replays, to the same bits, and so do the
+ * context's later runs.  ENOAO_EINVAL for batched contexts and for limits below -1. */
+enoao_status enoao_set_run_block_limit(enoao_ctx *ctx, int blocks);
+
 /* One third-order TVD Runge-Kutta step of a 1D problem that allocates no
  * device memory.  The paper has no counterpart: this is a deployment aid for
  * callers that cannot let a library allocate -- applications that reserve

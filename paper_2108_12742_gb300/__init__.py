@@ -108,6 +108,7 @@ def load():
         "enoao_uses_grid_redecide": (ctypes.c_int, [P]),
         "enoao_set_redecide_pass_limit": (ctypes.c_int, [P, ctypes.c_int]),
         "enoao_set_run_poll_limit": (ctypes.c_int, [P, ctypes.c_int]),
+        "enoao_set_run_block_limit": (ctypes.c_int, [P, ctypes.c_int]),
         "enoao_set_tma": (ctypes.c_int, [P, ctypes.c_int]),
         "enoao_set_fused_stage": (ctypes.c_int, [P, ctypes.c_int, ctypes.c_int, ctypes.c_int,
                                                  ctypes.c_int, ctypes.c_int]),
@@ -344,6 +345,10 @@ class Solver:
         """Test knob: bound on a block's polls between the stages of a persistent 1D run
         (-1: default)."""
         self._check(self._lib.enoao_set_run_poll_limit(self._h, polls))
+
+    def set_run_block_limit(self, blocks):
+        """Test knob: bound on the blocks of a persistent 1D run (-1: none)."""
+        self._check(self._lib.enoao_set_run_block_limit(self._h, blocks))
 
     def uses_grid_redecide(self):
         return bool(self._lib.enoao_uses_grid_redecide(self._h))

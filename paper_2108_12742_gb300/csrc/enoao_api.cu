@@ -1098,14 +1098,16 @@ enoao_status enoao_rk_stage(enoao_ctx* c, int stage, double dt) {
 
 // Whether the steps of this context run inside one persistent launch
 // (run1d.cu): 1D problems small enough for a tile per SM, one alpha per step,
-// near-ties re-decided in the sweep, no TMA staging.
+// near-ties re-decided in the sweep, no TMA staging, and not found too large
+// for the device by an earlier run.
 static bool persistent_run(const enoao_ctx* c) {
   return !c->batch && !c->sub && c->cfg.ndim == 1 && !c->tma && !use_list(c) && !consts(c).field &&
-         !per_stage_alpha(c) && c->ncell <= (long long)kRun1dMaxTile * c->sms;
+         !per_stage_alpha(c) && !c->run_unfit && c->ncell <= (long long)kRun1dMaxTile * c->sms;
 }
 
-// Enqueues one persistent launch of up to cap steps.
-static enoao_status enqueue_run1d(enoao_ctx* c, long long cap) {
+// Enqueues one persistent launch of up to cap steps; fits false (and nothing
+// enqueued): its blocks cannot all be resident (SMs kept from the process, say).
+static enoao_status enqueue_run1d(enoao_ctx* c, long long cap, bool& fits) {
   int ts, block;
   run1d_tile(c->nv, c->ncell, c->sms, &ts, &block);
   Run1dArgs a;
@@ -1119,7 +1121,14 @@ static enoao_status enqueue_run1d(enoao_ctx* c, long long cap) {
   a.k = consts(c);
   a.cap = cap;
   a.polls = c->run_polls >= 0 ? (unsigned)c->run_polls : kRun1dPolls;
-  const cudaError_t e = run1d_launch(c->nv, c->cfg.order, fp32(c), a, block, c->sms, c->s);
+  const cudaError_t e =
+      run1d_launch(c->nv, c->cfg.order, fp32(c), a, block, c->sms, c->run_blocks, c->s);
+  fits = e != cudaErrorCooperativeLaunchTooLarge;
+  if (!fits) {
+    cudaGetLastError();
+    c->run_unfit = 1;
+    return ENOAO_OK;
+  }
   if (e != cudaSuccess) return fail(c, ENOAO_ECUDA, "1D run launch: %s", cudaGetErrorString(e));
   return ENOAO_OK;
 }
@@ -1131,7 +1140,7 @@ static enoao_status run_graph_steps(enoao_ctx* c, double t_end, double cfl, doub
                 "a sub-domain steps stage by stage (enoao_rk_stage) between halo exchanges");
   enoao_status r = enter(c);
   if (r != ENOAO_OK) return r;
-  const bool persistent = persistent_run(c);
+  bool persistent = persistent_run(c);
   if (!persistent) {
     r = build_graph(c, steps_per_graph(c));
     if (r != ENOAO_OK) return r;
@@ -1147,19 +1156,27 @@ static enoao_status run_graph_steps(enoao_ctx* c, double t_end, double cfl, doub
     // bounded length keep an open-ended run within reach of the host
     constexpr long long kCap = 4096;
     if (!until_time) {
-      for (long long k = 0; k < max_steps; k += kCap) {
-        r = enqueue_run1d(c, std::min(kCap, max_steps - k));
+      for (long long k = 0; k < max_steps && persistent; k += kCap) {
+        r = enqueue_run1d(c, std::min(kCap, max_steps - k), persistent);
         if (r != ENOAO_OK) return r;
       }
     } else {
       for (;;) {
-        r = enqueue_run1d(c, kCap);
+        r = enqueue_run1d(c, kCap, persistent);
+        if (r == ENOAO_OK && !persistent) break;
         if (r == ENOAO_OK) r = read_host_state(c);
         if (r != ENOAO_OK) return r;
         if (c->st_host->done || c->st_host->err) break;
         if (limit > 0 && c->st_host->steps >= limit) break;
       }
     }
+    if (!persistent) {  // the steps left, as graph replays
+      r = build_graph(c, steps_per_graph(c));
+      if (r != ENOAO_OK) return r;
+    }
+  }
+  if (persistent) {
+    // enqueued above
   } else if (!until_time) {
     const long long reps = (max_steps + c->graph_steps - 1) / c->graph_steps;
     for (long long k = 0; k < reps; ++k) CU(c, cudaGraphLaunch(c->graph, c->s));
@@ -1316,6 +1333,15 @@ enoao_status enoao_set_run_poll_limit(enoao_ctx* c, int polls) {
   if (c->batch) return fail(c, ENOAO_EINVAL, "not available for batched contexts");
   if (polls < -1) return fail(c, ENOAO_EINVAL, "poll limit must be >= 0, or -1 for the default");
   c->run_polls = polls;
+  return ENOAO_OK;
+}
+
+enoao_status enoao_set_run_block_limit(enoao_ctx* c, int blocks) {
+  if (!c) return fail(c, ENOAO_EINVAL, "NULL context");
+  if (c->batch) return fail(c, ENOAO_EINVAL, "not available for batched contexts");
+  if (blocks < -1) return fail(c, ENOAO_EINVAL, "block limit must be >= 0, or -1 for none");
+  c->run_blocks = blocks;
+  c->run_unfit = 0;
   return ENOAO_OK;
 }
 

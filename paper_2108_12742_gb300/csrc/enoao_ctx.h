@@ -57,6 +57,8 @@ struct enoao_ctx {
   long long redo_cap = 0;
   int redo_passes = -1;                // in-sweep re-decision pass bound (-1: 64 nv)
   int run_polls = -1;                  // 1D runs: bound on a barrier's polls (-1: kRun1dPolls)
+  int run_blocks = -1;                 // 1D runs: bound on the blocks of a persistent one (-1: none)
+  int run_unfit = 0;                   // 1: its blocks do not fit the device at once
   int tma = 0;                         // FP32 bulk: stage raw tiles by TMA where eligible
   // Arrays: carr cells per conserved component, the interior from cell org on.
   // A sub-domain (enoao_create_subdomain) owns layers [sub_off, sub_off + n[last])

@@ -117,14 +117,15 @@ __global__ void __launch_bounds__(256, 1) run1d_kernel(const __grid_constant__ R
 }
 
 template <int NV, int ORDER, typename R>
-cudaError_t launch_one(const Run1dArgs& a, int block, int sms, cudaStream_t s) {
+cudaError_t launch_one(const Run1dArgs& a, int block, int sms, int max_blocks, cudaStream_t s) {
   const SweepArgs& A = a.stage[0];
   const size_t smem = sweep_smem_bytes(NV, sizeof(R) == 4, 1, A.se);
   const void* kernel = reinterpret_cast<const void*>(run1d_kernel<NV, ORDER, R>);
   int per_sm = 0;
   cudaError_t e = sweep_setup(kernel, block, smem, &per_sm);
   if (e != cudaSuccess) return e;
-  if (A.ntiles > (long long)per_sm * sms) return cudaErrorCooperativeLaunchTooLarge;
+  if (A.ntiles > (long long)per_sm * sms || (max_blocks >= 0 && A.ntiles > max_blocks))
+    return cudaErrorCooperativeLaunchTooLarge;
   void* args[1] = {const_cast<Run1dArgs*>(&a)};
   return cudaLaunchCooperativeKernel(kernel, dim3((unsigned)A.ntiles), dim3(block), args, smem, s);
 }
@@ -145,16 +146,16 @@ void run1d_tile(int nv, long long n, int sms, int* ts, int* block) {
 }
 
 cudaError_t run1d_launch(int nv, int order, int fp32, const Run1dArgs& a, int block, int sms,
-                         cudaStream_t s) {
+                         int max_blocks, cudaStream_t s) {
   switch (nv * 100 + order * 10 + (fp32 ? 1 : 0)) {
-    case 150: return launch_one<1, 5, double>(a, block, sms, s);
-    case 170: return launch_one<1, 7, double>(a, block, sms, s);
-    case 151: return launch_one<1, 5, float>(a, block, sms, s);
-    case 171: return launch_one<1, 7, float>(a, block, sms, s);
-    case 350: return launch_one<3, 5, double>(a, block, sms, s);
-    case 370: return launch_one<3, 7, double>(a, block, sms, s);
-    case 351: return launch_one<3, 5, float>(a, block, sms, s);
-    case 371: return launch_one<3, 7, float>(a, block, sms, s);
+    case 150: return launch_one<1, 5, double>(a, block, sms, max_blocks, s);
+    case 170: return launch_one<1, 7, double>(a, block, sms, max_blocks, s);
+    case 151: return launch_one<1, 5, float>(a, block, sms, max_blocks, s);
+    case 171: return launch_one<1, 7, float>(a, block, sms, max_blocks, s);
+    case 350: return launch_one<3, 5, double>(a, block, sms, max_blocks, s);
+    case 370: return launch_one<3, 7, double>(a, block, sms, max_blocks, s);
+    case 351: return launch_one<3, 5, float>(a, block, sms, max_blocks, s);
+    case 371: return launch_one<3, 7, float>(a, block, sms, max_blocks, s);
     default: return cudaErrorInvalidValue;
   }
 }

@@ -20,8 +20,10 @@ constexpr unsigned kRun1dPolls = 1u << 22;  // a few seconds
 
 // Cells per tile and threads per block for a problem of n cells.
 void run1d_tile(int nv, long long n, int sms, int* ts, int* block);
-// fp32: bulk precision.  One cooperative launch, a block per tile.
+// fp32: bulk precision.  One cooperative launch, a block per tile;
+// cudaErrorCooperativeLaunchTooLarge (and nothing launched) where the blocks
+// cannot all be resident at once, or are more than max_blocks (if that is >= 0).
 cudaError_t run1d_launch(int nv, int order, int fp32, const Run1dArgs& a, int block, int sms,
-                         cudaStream_t s);
+                         int max_blocks, cudaStream_t s);
 
 }  // namespace enoao

@@ -1,6 +1,7 @@
-"""A persistent 1D run whose blocks run out of polls at the grid barrier: an error
-status, no half-taken step counted, no further run from the barrier's short
-count, and a context that is usable again once its state is set."""
+"""The limits of a persistent 1D run.  Blocks that run out of polls at the grid
+barrier: an error status, no half-taken step counted, no further run from the
+barrier's short count, and a context that is usable again once its state is set.
+Blocks that do not all fit: the same steps, to the same bits, as graph replays."""
 import numpy as np
 import pytest
 
@@ -56,8 +57,32 @@ def test_barrier_polls_run_out_as_a_timeout_status(precision):
         assert np.array_equal(s.get_state(), good)
 
 
-def test_poll_limit_rejects_bad_values():
+@pytest.mark.parametrize("precision", [eno.FP64, eno.FP32_BULK])
+def test_blocks_that_do_not_fit_step_as_graphs(precision):
+    U = inputs.titarev_toro(N)
+    with _solver(precision) as s:
+        def runs():
+            s.init_state(U)
+            s.advance_steps(37, 0.5)
+            a = s.get_state()
+            s.init_state(U)
+            t, k = s.advance(0.05, cfl=0.5)
+            assert t == 0.05
+            return a, s.get_state(), k
+        a, b, k = runs()
+        s.set_run_block_limit(1)
+        assert s.launches_per_step() == 0  # not known yet
+        for _ in range(2):
+            a1, b1, k1 = runs()
+            assert s.launches_per_step() > 0
+            assert np.array_equal(a, a1) and np.array_equal(b, b1) and k == k1
+        s.set_run_block_limit(-1)
+        assert s.launches_per_step() == 0
+
+
+def test_limits_reject_bad_values():
     with _solver(eno.FP64) as s:
-        with pytest.raises(eno.EnoaoError) as e:
-            s.set_run_poll_limit(-2)
-        assert e.value.status == EINVAL
+        for knob in (s.set_run_poll_limit, s.set_run_block_limit):
+            with pytest.raises(eno.EnoaoError) as e:
+                knob(-2)
+            assert e.value.status == EINVAL
