@@ -287,6 +287,24 @@ void default_tiles(enoao_ctx* c) {
   }
 }
 
+// Shared memory of a sweep block of axis d with tiles of ta lines x ts cells.
+size_t tile_smem(const enoao_ctx* c, int d, int ta, int ts) {
+  const int field = consts(c).field;
+  return sweep_smem_bytes(c->nv, fp32(c), ta,
+                          sweep_row_pitch(c->nv, c->cfg.order, fp32(c), d, ta, ts, field), field);
+}
+
+constexpr size_t kTileSmem = 216 * 1024;
+
+// Cells per tile of a sweep's launches: the tile's, or as many as fit a block.
+// Scalar FP64 tiles of more than 7,890 cells, whose planes fit, do not with
+// the face list (a word a cell); in parts they give the same bits.
+int launch_ts(const enoao_ctx* c, int d) {
+  int ts = c->ts[d];
+  while (tile_smem(c, d, c->ta[d], ts) > kTileSmem) ts = (ts + 1) / 2;
+  return ts;
+}
+
 enoao_status check_tiles(enoao_ctx* c, int d, int ta, int ts) {
   if (ta < 1 || ts < 1 || ta * ts > 8192)
     return fail(c, ENOAO_EINVAL, "tile %dx%d out of range", ta, ts);
@@ -294,12 +312,11 @@ enoao_status check_tiles(enoao_ctx* c, int d, int ta, int ts) {
     return fail(c, ENOAO_EINVAL, "axis %d needs 8, 16, 32 or 64 lines per tile", d);
   if (d == 0 && ta != 1 && ta != 2 && ta != 4 && ta != 8)
     return fail(c, ENOAO_EINVAL, "axis 0 needs 1, 2, 4 or 8 lines per tile");
-  const int field = consts(c).field;
-  size_t smem = sweep_smem_bytes(
-      c->nv, fp32(c), ta, sweep_row_pitch(c->nv, c->cfg.order, fp32(c), d, ta, ts, field), field);
-  // (216 KB: the tiles that fitted 200 KB before a cell took a face-list word
-  // and, in FP32 bulk, a value more)
-  if (smem > 216 * 1024)
+  const size_t smem = tile_smem(c, d, ta, ts);
+  // FP64: without the face list (launch_ts)
+  const size_t list = fp32(c) ? 0 : 4 * (size_t)tile_cells(
+      ta, sweep_row_pitch(c->nv, c->cfg.order, 0, d, ta, ts, consts(c).field));
+  if (smem > kTileSmem && (fp32(c) || smem - list > 200 * 1024))
     return fail(c, ENOAO_EINVAL, "tile %dx%d needs %zu bytes of shared memory", ta, ts, smem);
   return ENOAO_OK;
 }
@@ -481,7 +498,7 @@ enoao_status launch_sweep(enoao_ctx* c, int d, int stage, int mode, const double
                           cudaEvent_t after_sweep = nullptr) {
   SweepArgs a;
   enoao_status r0 = fill_sweep_args(c, d, stage, mode, u_in, u_out, fhat, idx, list, c->ta[d],
-                                    c->ts[d], a);
+                                    launch_ts(c, d), a);
   if (r0 != ENOAO_OK) return r0;
   CUtensorMap tmap;
   const size_t smem0 = sweep_smem_bytes(c->nv, fp32(c), a.ta, a.se, consts(c).field);
