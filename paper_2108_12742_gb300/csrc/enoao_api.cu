@@ -1440,7 +1440,10 @@ enoao_status enoao_autotune(enoao_ctx* c) {
       for (int ta : tas)
         for (int ts : tss) cands.push_back({ta, ts});
     }
+    // (the tile in use first and last: tuning does not end slower than it began)
     const int best_ta0 = c->ta[d], best_ts0 = c->ts[d];
+    cands.insert(cands.begin(), {best_ta0, best_ts0});
+    cands.push_back({best_ta0, best_ts0});
     float best = 1e30f;
     int bta = best_ta0, bts = best_ts0;
     for (auto& p : cands) {
