@@ -134,6 +134,7 @@ struct SweepArgs {
   int tma_box;          // TMA: box extent along the swept axis (cells, with alignment slack)
   unsigned tma_bytes;   // TMA: bytes of one box
   int tma_raw_bytes;    // TMA: shared memory reserved for the box (a multiple of 128)
+  int redo_spread;      // FP32 bulk: 1 where the launch has no more tiles than SMs
   int redo_passes;      // FP32 bulk: bound on the in-sweep re-decision passes of a warp
                         // round; reaching it sets kErrTimeout (64 nv by default)
   long long tiles_s;    // tiles along dir

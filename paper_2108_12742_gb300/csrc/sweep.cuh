@@ -1839,23 +1839,41 @@ __device__ __forceinline__ void redecide_tile(const SweepArgs& A, const TileGeo&
     const int bd = blockDim.x, tid = threadIdx.x, lane = tid & 31;
     // The flagged entries to the front of the list (one warp, in place: an
     // entry never moves behind one not yet read), so that the choices of a
-    // warp's 32 faces below fill its lanes.
-    __shared__ int s_nflag;
+    // warp's faces below fill its lanes.
+    __shared__ int s_nflag, s_nchoice;
     if (tid < 32) {
       int n = 0;
+      unsigned nc = 0;
       for (int base = 0; base < nlist; base += 32) {
         const unsigned e = base + lane < nlist ? tv.list[base + lane] : 0u;
         const unsigned m = __ballot_sync(FULL, entry_flags(e) != 0u);
         if (entry_flags(e)) tv.list[n + __popc(m & ((1u << lane) - 1u))] = e;
         n += __popc(m);
+        nc += __popc(entry_flags(e));
         __syncwarp();
       }
-      if (lane == 0) s_nflag = n;
+      nc = __reduce_add_sync(FULL, nc);
+      if (lane == 0) s_nflag = n, s_nchoice = (int)nc;
     }
     __syncthreads();
-    const int nflag = s_nflag;
-    for (int base = tid - lane; base < nflag; base += bd) {  // the same for every lane
-      const unsigned entry = base + lane < nflag ? tv.list[base + lane] : 0u;
+    // The warps that share them: a round of 32 choices each (redo_lane), or, of a
+    // few choices, a round of NG (redo_group), which costs no more in all and
+    // ends sooner.  In 32 faces a warp, whatever their choices, the first warps
+    // took all and each scheduler's FP64 pipe but theirs stood idle: tiles along a
+    // front then set the length of a sweep (1024^2 quadrant jumps, per-field
+    // ENO-AO7 y sweep 320 -> 182 us, one-alpha ENO-AO5 stage 186 -> 153 us;
+    // composite wave ENO-AO7 N = 400 36.8 -> 32.2 us a step).  Where a launch has no
+    // more tiles than SMs nothing else would use the pipes: as many warps as
+    // there are rounds of NG (1D ENO-AO7 noise stage 47 -> 38 us).  Without the
+    // choices' number, by faces alone, sweeps with a choice or two a tile took
+    // longer than before (512^2 noise, ENO-AO5 stage 157 -> 163 us).
+    const int nflag = s_nflag, nchoice = s_nchoice;
+    const int few = A.redo_spread ? nchoice : 3 * NG;
+    const int nw = min(bd >> 5, nchoice <= few ? (nchoice + NG - 1) / NG : (nchoice + 31) / 32);
+    const int share = min(32, (nflag + nw - 1) / nw);  // faces of a warp at a time
+    const int wid = tid >> 5;
+    for (int base = wid < nw ? wid * share : nflag; base < nflag; base += nw * share) {
+      const unsigned entry = lane < share && base + lane < nflag ? tv.list[base + lane] : 0u;
       const int al = entry_line(entry), f = entry_face(entry);
       const int j = G - 1 + f;
       unsigned fix = entry_flags(entry);
