@@ -1517,14 +1517,18 @@ struct TileConst {
   float dt32, wdt32;    // FP32 bulk combine: dt and the stage's weight of dt L
   float limit;          // bound of prove_top
   R inv_dx;
+  R af[3];              // per field: splitting constants of u-c, of entropy and shear, of u+c
 };
-template <int ORDER, typename R>
+template <int ORDER, typename R, bool FIELD = false>
 __device__ __forceinline__ void tile_const(const SweepArgs& A, double alpha_d, double dt,
                                            TileConst<R>& k) {
   k.alpha_d = alpha_d;
   k.dt = dt;
   k.alpha = (R)alpha_d;
   k.inv_dx = bconst<R>(A.inv_dx, A.inv_dx_f);
+  if constexpr (FIELD) {
+    for (int i = 0; i < 3; ++i) k.af[i] = (R)A.st->alpha_f[A.dir][i];
+  }
   k.dt32 = f32_rn(dt);
   k.wdt32 = f32_rn((A.stage == 0 ? 1.0 : (A.stage == 1 ? 0.25 : 2.0 / 3.0)) * dt);
   // below delta by more than the near-tie margin (and the bound's own
@@ -1554,7 +1558,6 @@ __device__ __forceinline__ unsigned choose_face(const SweepArgs& A, const TileGe
   using CV = CellVec<NV, R, FIELD>;
   constexpr int G = Geo<ORDER>::G;
   constexpr bool FP32 = sizeof(R) == 4;
-  const StepState* st = A.st;
   const int cells = tv.cells, mode = shape_mode<SHAPE>(A);
   R* const dfm = tv.dfm;
   R* const Cf = tv.Cf;
@@ -1563,13 +1566,10 @@ __device__ __forceinline__ unsigned choose_face(const SweepArgs& A, const TileGe
   const R delta = bconst<R>(A.delta, A.delta_f);
   const R tie_rel = bconst<R>(A.tie_rel, A.tie_rel_f);
   // splitting constant of field v: alpha, or per field max |u_d - c|, |u_d|, |u_d + c|
-  R alo = K.alpha, amid = K.alpha, ahi = K.alpha;
-  if constexpr (FIELD) {
-    alo = (R)st->alpha_f[A.dir][0];
-    amid = (R)st->alpha_f[A.dir][1];
-    ahi = (R)st->alpha_f[A.dir][2];
-  }
-  auto afield = [&](int v) { return v == 0 ? alo : (v == NV - 1 ? ahi : amid); };
+  auto afield = [&](int v) {
+    if constexpr (FIELD) return K.af[v == 0 ? 0 : (v == NV - 1 ? 2 : 1)];
+    return K.alpha;
+  };
   const int j = G - 1 + f;  // face j+1/2 in extended cells
   Eigen<NV, R> E;
   if constexpr (NV > 1) face_eigen<NV, ORDER, R, FIELD>(tv, sidx(a, j), gm1, E);
@@ -1788,6 +1788,37 @@ __device__ __noinline__ bool listed_faces_call(const SweepArgs& A, const TileGeo
                                                unsigned char* smem_raw, const TileConst<float>& K,
                                                int n) {
   return listed_faces<NV, ORDER, float, COHERENT, SHAPE>(A, g, smem_raw, K, n);
+}
+
+// Phase 2 of a tile with per-field constants: every face, one per thread; returns
+// whether this thread met a near-tie.
+template <int NV, int ORDER, typename R, bool COHERENT, int SHAPE>
+__device__ __forceinline__ bool field_faces(const SweepArgs& A, const TileGeo& g,
+                                            unsigned char* smem_raw, const TileConst<R>& K,
+                                            int lgTA, bool sfast, int* nlist) {
+  const TileView<NV, ORDER, R, true> tv(smem_raw, A.ta, A.se);
+  bool any = false;
+  for_items(lgTA, g.nts + 1, sfast, [&](const int a, const int f) {
+    if (g.a0 + a >= g.na) return;
+    const unsigned fix = choose_face<NV, ORDER, R, COHERENT, true, SHAPE>(A, g, tv, K, a, f);
+    if constexpr (sizeof(R) == 4) {
+      if (fix) {
+        tv.list[atomicAdd(nlist, 1)] = face_entry(a, f) | fix;
+        any = true;
+      }
+    }
+  });
+  return any;
+}
+// The same out of line (FP32, 2D): its two projections per window cell otherwise
+// spill in the other phases too (1024^2 ENO-AO7 x and y sweeps 133 -> 129 and
+// 139 -> 136 us).  3D (96^3 ENO-AO5 stage 615 -> 657 us) and FP64, which has the
+// registers (1.60 -> 1.68 ms), stay inline.
+template <int NV, int ORDER, bool COHERENT, int SHAPE>
+__device__ __noinline__ bool field_faces_call(const SweepArgs& A, const TileGeo& g,
+                                              unsigned char* smem_raw, const TileConst<float>& K,
+                                              int lgTA, bool sfast, int* nlist) {
+  return field_faces<NV, ORDER, float, COHERENT, SHAPE>(A, g, smem_raw, K, lgTA, sfast, nlist);
 }
 
 // One tile of a sweep (phases 1-3 above).  amax accumulates |u_d| + c of
@@ -2240,17 +2271,12 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& A, const TileGeo& g,
         else
           any_fix = listed_faces<NV, ORDER, R, COHERENT, SHAPE>(A, g, smem_raw, K, s_nlist);
       }
+    } else if constexpr (FP32 && NV == 4) {
+      any_fix = field_faces_call<NV, ORDER, COHERENT, SHAPE>(A, g, smem_raw, K, lgTA, sfast,
+                                                             &s_nlist);
     } else {
-      for_items(lgTA, nfaces_tile, sfast, [&](const int a, const int f) {
-        if (g.a0 + a >= g.na) return;
-        const unsigned fix = choose_face<NV, ORDER, R, COHERENT, FIELD, SHAPE>(A, g, tv, K, a, f);
-        if constexpr (FP32) {
-          if (fix) {
-            tv.list[atomicAdd(&s_nlist, 1)] = face_entry(a, f) | fix;
-            any_fix = true;
-          }
-        }
-      });
+      any_fix = field_faces<NV, ORDER, R, COHERENT, SHAPE>(A, g, smem_raw, K, lgTA, sfast,
+                                                           &s_nlist);
     }
   }
 
@@ -2567,7 +2593,7 @@ __global__ void __launch_bounds__(128, sweep_min_blocks<R, FIELD, TMA>())
   if (st->skip) return;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ TileConst<R> s_k;
-  if (threadIdx.x == 0) tile_const<ORDER, R>(A, st->alpha[A.dir], st->dt, s_k);
+  if (threadIdx.x == 0) tile_const<ORDER, R, FIELD>(A, st->alpha[A.dir], st->dt, s_k);
   constexpr int KA = kAmax<FIELD>;
   double amax[KA];
 #pragma unroll
