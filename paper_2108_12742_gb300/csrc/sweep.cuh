@@ -2497,19 +2497,26 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& A, const TileGeo& g,
 }
 
 // Minimum resident blocks per SM asked of the compiler for the FP32-bulk
-// sweep (caps its registers at 65536 / (128 * min blocks): 64, a few spilled
-// around the out-of-line calls).  Six, eight and ten were within 5 % of one
-// another on 4096^2 and 256^3 data; eight led on most tiles.
+// sweep, which caps its registers at 65536 / (128 * min blocks): eight (64, a few
+// spilled around the out-of-line calls) for ENO-AO5 and scalars, six (80) for
+// ENO-AO7 of the Euler equations, whose selection spills at 64 (512^3 stage 29.1 ->
+// 28.0 ms, 1024^2 jumps 237 -> 229 us, 512^2 noise, every face selected, 208 -> 201 us;
+// scalars at 80: 1024^2 sine 44 -> 48 us).
 #ifndef ENOAO_FP32_MIN_BLOCKS
 #define ENOAO_FP32_MIN_BLOCKS 8
+#endif
+#ifndef ENOAO_FP32_MIN_BLOCKS_EULER7
+#define ENOAO_FP32_MIN_BLOCKS_EULER7 6
 #endif
 // Per-field splitting keeps two projections per window cell live and takes
 // four blocks (128 registers).  With a TMA-staged raw tile a block needs more
 // shared memory, and four of them fill an SM: they get the registers (128, no
 // spills; at 96 the thread-0 copy issue spills).
-template <typename R, bool FIELD = false, bool TMA = false>
+template <int NV, int ORDER, typename R, bool FIELD = false, bool TMA = false>
 constexpr int sweep_min_blocks() {
-  return sizeof(R) == 8 ? 1 : (FIELD || TMA ? 4 : ENOAO_FP32_MIN_BLOCKS);
+  if (sizeof(R) == 8) return 1;
+  if (FIELD || TMA) return 4;
+  return NV > 1 && ORDER == 7 ? ENOAO_FP32_MIN_BLOCKS_EULER7 : ENOAO_FP32_MIN_BLOCKS;
 }
 
 // Bound on the polls of a TMA completion barrier (a copy of a few tens of KB
@@ -2588,7 +2595,7 @@ __device__ __forceinline__ void sweep_epilogue(const SweepArgs& A, double (&amax
 
 template <int NV, int ORDER, typename R, bool DEFER = false, bool FIELD = false, bool TMA = false,
           int SHAPE = kShapeAny>
-__global__ void __launch_bounds__(128, sweep_min_blocks<R, FIELD, TMA>())
+__global__ void __launch_bounds__(128, sweep_min_blocks<NV, ORDER, R, FIELD, TMA>())
     sweep_kernel(const __grid_constant__ SweepArgs A, const __grid_constant__ CUtensorMap tmap) {
   constexpr int G = Geo<ORDER>::G;
   StepState* st = A.st;
@@ -2725,8 +2732,10 @@ __global__ void __launch_bounds__(128, sweep_min_blocks<R, FIELD, TMA>())
 // blocks never wait on one another.  Ax and Ay are the two axes' arguments
 // as separate launches would take them; the host makes the 2D tile a whole
 // number of both axes' sub-tiles (Ay.ts % Ax.ta == 0, Ax.ts % Ay.ta == 0).
+// (ENO-AO7: five blocks, 96 registers for both parts in one kernel; 1024^2 jumps
+// 1.03 -> 0.92 ms a stage)
 template <int NV, int ORDER>
-__global__ void __launch_bounds__(128, sweep_min_blocks<float>())
+__global__ void __launch_bounds__(128, ORDER == 7 ? 5 : ENOAO_FP32_MIN_BLOCKS)
     fused2d_kernel(const __grid_constant__ SweepArgs Ax, const __grid_constant__ SweepArgs Ay) {
   using R = float;
   StepState* st = Ay.st;
