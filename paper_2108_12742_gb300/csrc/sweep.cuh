@@ -1271,7 +1271,12 @@ __device__ __forceinline__ void face_eigen(const TileView<NV, ORDER, R, FIELD>& 
 // (Without the projection, as the FP64 path does it, they took 0.41 and 0.60
 // ms; but R (L s) and s differ by FP32 rounding, which later stages' near-ties
 // turn into other choices.)
-template <int NV, int ORDER, bool FIELD>
+// FRONTS: return as soon as the first sign's differences fail.  For the listing
+// sweeps, whose flows leave most faces of a tile unproven (2D Riemann
+// configuration 1, 800^2, late: ENO-AO5 701 -> 691, ENO-AO7 1175 -> 1145 us a step with
+// the ENO-AO7 registers below); on resolved flow the branch costs a little (4096^2
+// ENO-AO5 step 4.47 -> 4.53 ms), so the others do without.
+template <int NV, int ORDER, bool FIELD, bool FRONTS>
 __device__ __forceinline__ bool prove_top(const TileView<NV, ORDER, float, FIELD>& tv, int x,
                                           float gm1, float limit, float (&C)[NV]) {
   using CV = CellVec<NV, float, FIELD>;
@@ -1363,6 +1368,7 @@ __device__ __forceinline__ bool prove_top(const TileView<NV, ORDER, float, FIELD
       most = fmaxf(most, fabsf(d));
       cs[t] = sgn == 0 ? corrs[t] : cs[t] + corrs[t];
     }
+    if (FRONTS && sgn == 0 && !(ok && most <= limit)) return false;
   }
   float P;
   if constexpr (ORDER == 7)
@@ -1405,7 +1411,7 @@ __device__ __forceinline__ bool prove_top(const TileView<NV, ORDER, float, FIELD
 // a sum of FP64 differences, 8 NV (ENO-AO7: 12 NV) operations instead of 500.
 // 2048^2 ENO-AO5 sweeps: x 4.15 -> 1.13 ms, y 4.38 -> 1.20 ms (with choose64
 // and the neighbours' shared 1 / density).
-template <int NV, int ORDER, bool FIELD>
+template <int NV, int ORDER, bool FIELD, bool FRONTS>
 __device__ __forceinline__ bool prove_top(const TileView<NV, ORDER, double, FIELD>& tv, int x,
                                           float gm1, float limit, double (&C)[NV]) {
   using CV = CellVec<NV, double, FIELD>;
@@ -2251,7 +2257,7 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& A, const TileGeo& g,
       if (g.a0 + a >= g.na) return;
       const int x = sidx(a, G - 1 + f);
       R C[NV];
-      if (prove_top<NV, ORDER, FIELD>(tv, x, A.gm1_f, K.limit, C)) {
+      if (prove_top<NV, ORDER, FIELD, DEFER>(tv, x, A.gm1_f, K.limit, C)) {
         CV::store(Cf, cells, x, C);
         if ((mode & kModeFlux) && A.idx_out && owns_face(A, g, f)) {
           const long long fc = face_index(g, a, f);
