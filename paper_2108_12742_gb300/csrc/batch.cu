@@ -73,18 +73,19 @@ __device__ __forceinline__ double block_max(double v, double* red) {
   return r;
 }
 
-// Resident 256-thread blocks per SM asked of the compiler: FP32 bulk four
-// (64 registers, some spilled), FP64 three (80).  4096 uneven problems,
-// against the unbounded 116 registers and two blocks: FP32 bulk 1.52e10 ->
-// 1.68e10 (three) -> 1.73e10 (four) cell-stage/s; FP64 1.37e9 at three,
-// 1.30e9 at four.
-template <typename R>
+// Resident 256-thread blocks per SM asked of the compiler: FP32 bulk four for
+// the Euler equations (64 registers, some spilled), three for scalars (80), FP64
+// three.  Chosen before the proof of faces came in, on 4096 uneven problems:
+// against the unbounded 116 registers and two blocks FP32 bulk 1.52e10 -> 1.68e10
+// (three) -> 1.73e10 (four) cell-stage/s, FP64 1.37e9 at three, 1.30e9 at four; with
+// the proof 2.33e10 and 4.33e9.
+template <int NV, typename R>
 constexpr int batch_min_blocks() {
-  return sizeof(R) == 4 ? 4 : 3;
+  return sizeof(R) == 4 && NV > 1 ? 4 : 3;
 }
 
 template <int NV, int ORDER, typename R>
-__global__ void __launch_bounds__(256, batch_min_blocks<R>()) batch_kernel(const __grid_constant__ BatchArgs B) {
+__global__ void __launch_bounds__(256, batch_min_blocks<NV, R>()) batch_kernel(const __grid_constant__ BatchArgs B) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ int s_q;
   __shared__ double s_red[32];
@@ -150,7 +151,12 @@ __global__ void __launch_bounds__(256, batch_min_blocks<R>()) batch_kernel(const
             if (threadIdx.x == 0 && tile + 1 < ntiles)
               s_geo[(tile + 1) & 1] = batch_geo(A, off, n, tile + 1);
           };
-          sweep_tile<NV, ORDER, R, true, false, false, false, kShapeXCombine, decltype(publish)>(
+          // (scalars in FP32: a face's selection costs little more than its proof, and
+          // unresolved problems paid for both: 1024 problems of white noise, ENO-AO5 and
+          // ENO-AO7, 0.90 and 1.11 -> 0.69 and 0.87 ms a step, of one sine each, 0.47 and
+          // 0.50 -> 0.40 and 0.44 ms, with three blocks instead of four)
+          sweep_tile<NV, ORDER, R, true, false, false, false, kShapeXCombine, decltype(publish),
+                     (NV > 1 || sizeof(R) == 8)>(
               A, s_geo[tile & 1], smem_raw, s_k, amax, nfall, RawTile{}, publish);
         }
         if constexpr (NV > 1) {

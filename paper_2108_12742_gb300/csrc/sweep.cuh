@@ -1796,17 +1796,17 @@ __device__ __noinline__ bool listed_faces_call(const SweepArgs& A, const TileGeo
   return listed_faces<NV, ORDER, float, COHERENT, SHAPE>(A, g, smem_raw, K, n);
 }
 
-// Phase 2 of a tile with per-field constants: every face, one per thread; returns
-// whether this thread met a near-tie.
-template <int NV, int ORDER, typename R, bool COHERENT, int SHAPE>
-__device__ __forceinline__ bool field_faces(const SweepArgs& A, const TileGeo& g,
+// Phase 2 of a tile without the proof: every face, one per thread; returns whether
+// this thread met a near-tie.
+template <int NV, int ORDER, typename R, bool COHERENT, bool FIELD, int SHAPE>
+__device__ __forceinline__ bool all_faces(const SweepArgs& A, const TileGeo& g,
                                             unsigned char* smem_raw, const TileConst<R>& K,
                                             int lgTA, bool sfast, int* nlist) {
-  const TileView<NV, ORDER, R, true> tv(smem_raw, A.ta, A.se);
+  const TileView<NV, ORDER, R, FIELD> tv(smem_raw, A.ta, A.se);
   bool any = false;
   for_items(lgTA, g.nts + 1, sfast, [&](const int a, const int f) {
     if (g.a0 + a >= g.na) return;
-    const unsigned fix = choose_face<NV, ORDER, R, COHERENT, true, SHAPE>(A, g, tv, K, a, f);
+    const unsigned fix = choose_face<NV, ORDER, R, COHERENT, FIELD, SHAPE>(A, g, tv, K, a, f);
     if constexpr (sizeof(R) == 4) {
       if (fix) {
         tv.list[atomicAdd(nlist, 1)] = face_entry(a, f) | fix;
@@ -1816,7 +1816,7 @@ __device__ __forceinline__ bool field_faces(const SweepArgs& A, const TileGeo& g
   });
   return any;
 }
-// The same out of line (FP32, 2D): its two projections per window cell otherwise
+// The same out of line (per-field constants, FP32, 2D): its two projections per window cell otherwise
 // spill in the other phases too (1024^2 ENO-AO7 x and y sweeps 133 -> 129 and
 // 139 -> 136 us).  3D (96^3 ENO-AO5 stage 615 -> 657 us) and FP64, which has the
 // registers (1.60 -> 1.68 ms), stay inline.
@@ -1824,7 +1824,7 @@ template <int NV, int ORDER, bool COHERENT, int SHAPE>
 __device__ __noinline__ bool field_faces_call(const SweepArgs& A, const TileGeo& g,
                                               unsigned char* smem_raw, const TileConst<float>& K,
                                               int lgTA, bool sfast, int* nlist) {
-  return field_faces<NV, ORDER, float, COHERENT, SHAPE>(A, g, smem_raw, K, lgTA, sfast, nlist);
+  return all_faces<NV, ORDER, float, COHERENT, true, SHAPE>(A, g, smem_raw, K, lgTA, sfast, nlist);
 }
 
 // One tile of a sweep (phases 1-3 above).  amax accumulates |u_d| + c of
@@ -2064,10 +2064,12 @@ __device__ __noinline__ void redecide_tile_call(const SweepArgs& A, const TileGe
 }
 
 // TMA: phase 1 reads the tile's raw state from rt instead of global memory.
+// PROOF: prove faces first, where the sweep can (kProve).
 // hook() runs before the tile's last barrier, with TMA once every thread is
 // past phase 1 (the raw buffer is then free for the next tile's copy).
 template <int NV, int ORDER, typename R, bool COHERENT = false, bool DEFER = false,
-          bool FIELD = false, bool TMA = false, int SHAPE = kShapeAny, typename Hook = NoHook>
+          bool FIELD = false, bool TMA = false, int SHAPE = kShapeAny, typename Hook = NoHook,
+          bool PROOF = true>
 __device__ __forceinline__ void sweep_tile(const SweepArgs& A, const TileGeo& g,
                                            unsigned char* smem_raw, const TileConst<R>& K,
                                            double (&amax)[kAmax<FIELD>],
@@ -2077,9 +2079,9 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& A, const TileGeo& g,
   using GE = Geo<ORDER>;
   constexpr int G = GE::G;
   constexpr bool FP32 = sizeof(R) == 4;
-  constexpr bool PROVE = kProve<FIELD>;
+  constexpr bool PROVE = kProve<FIELD> && PROOF;
   // the code of faces not proven and of near-ties out of line
-  constexpr bool CALL = FP32 && PROVE && SHAPE != kShapeAny;
+  constexpr bool CALL = FP32 && !FIELD && SHAPE != kShapeAny;
   StepState* st = A.st;
   const int TA = A.ta, TS = A.ts;
   // row pitch A.se (>= TS + 2G), chosen on the host for conflict-free banks
@@ -2185,7 +2187,7 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& A, const TileGeo& g,
       } else {
         CV::store(dfp, cells, sidx(a, e), fp);
         CV::store(dfm, cells, sidx(a, e), fm);
-        if constexpr (tv.MAG) tv.mag[sidx(a, e)] = m;
+        if constexpr (PROVE && tv.MAG) tv.mag[sidx(a, e)] = m;
       }
     };
     if (sfast) {
@@ -2279,12 +2281,12 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& A, const TileGeo& g,
         else
           any_fix = listed_faces<NV, ORDER, R, COHERENT, SHAPE>(A, g, smem_raw, K, s_nlist);
       }
-    } else if constexpr (FP32 && NV == 4) {
+    } else if constexpr (FIELD && FP32 && NV == 4) {
       any_fix = field_faces_call<NV, ORDER, COHERENT, SHAPE>(A, g, smem_raw, K, lgTA, sfast,
                                                              &s_nlist);
     } else {
-      any_fix = field_faces<NV, ORDER, R, COHERENT, SHAPE>(A, g, smem_raw, K, lgTA, sfast,
-                                                           &s_nlist);
+      any_fix = all_faces<NV, ORDER, R, COHERENT, FIELD, SHAPE>(A, g, smem_raw, K, lgTA, sfast,
+                                                                &s_nlist);
     }
   }
 
