@@ -267,6 +267,11 @@ void pick_tile(const enoao_ctx* c, int d, int* ta_out, int* ts_out) {
       }
     }
   }
+  // 1D: no longer than a tile per SM needs (run1d_tile; Euler fluxes of 500 cells of
+  // noise, ENO-AO7 FP32: 4 tiles of 118 45 us, 34 of 15 33 us)
+  if (c->cfg.ndim == 1)
+    *ts_out = (int)std::min<long long>(
+        *ts_out, std::max<long long>(c->nv == 1 ? 63 : 15, (nd + c->sms - 1) / c->sms));
 }
 
 // Per-field sweeps: tile lengths are 2^k - 1 cells, so that the 2^k faces of a

@@ -190,7 +190,11 @@ extern "C" enoao_status enoao_step_noalloc(const enoao_config* cfg, const double
   a.dir = 0;
   a.bc = cfg->bc[0];
   a.ta = 1;
-  a.ts = f32 ? 127 : 63;
+  // a tile per SM, as a run takes it (run1d_tile): with 63 or 127 cells always, small
+  // problems left most SMs idle, the more so since a block proves its faces and
+  // then selects (Euler ENO-AO5, N = 2000: FP32 bulk 126 -> 102, FP64 120 -> 99 us a step)
+  a.ts = (int)std::min<long long>(f32 ? 127 : 63,
+                                  std::max<long long>(nv == 1 ? 63 : 15, (n + sms - 1) / sms));
   a.se = sweep_row_pitch(nv, cfg->order, f32, 0, a.ta, a.ts);
   a.tiles_s = (n + a.ts - 1) / a.ts;
   a.tiles_a = a.tiles_b = 1;
