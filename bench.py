@@ -38,9 +38,6 @@ FLOPS_PER_FACE = 1150       # flops of one face of one axis, 2D Euler ENO-AO5 (t
                             # operation count: split, Roe eigen-system, projection of both
                             # windows, indicators, selection, back-projection)
 FLOPS_PER_FACE_COUNTED = 885  # the same path counted operation by operation in the kernel
-# FP64-unit instructions of one cell of the FP64 y sweep (2D Euler ENO-AO5, stage 0, evolved data,
-# counted by the profiler; the choices are decided in FP32), two flops each at the unit's peak
-FP64_INST_PER_CELL_Y = 143
 # y sweep, stage 0: read U^n (FP64) and L_x (FP32), write U1 (FP64) and the
 # FP32 increment I0 the later stages combine with
 BYTES_PER_CELL_Y = 32 + 16 + 32 + 16
@@ -199,9 +196,14 @@ def step_roofline(value, flops_per_cs, bytes_fused, bytes_split, peaks, hbm):
                     "bytes_per_cell_stage": {"fused": bytes_fused, "per_axis": bytes_split}}}
 
 
-def profiled_traffic(summary):
-    """DRAM bytes per launch of the dominant kernel at 4096^2, from the committed
-    ncu summary, if that summary was taken on the current kernel source."""
+TRAFFIC = r"traffic_bytes_per_launch_4096:\s*([0-9.eE+]+)"            # DRAM bytes at 4096^2
+INST = r"\| warp instructions x 32 per cell \| ([0-9.]+) \|"
+FP64_INST = r"\| FP64-unit warp instructions x 32 per cell \| ([0-9.]+) \|"
+
+
+def profiled(summary, pattern):
+    """A figure of a committed ncu summary, if that summary was taken on the
+    current kernel source (else None)."""
     import hashlib
     import re
     prof = os.path.join(ROOT, "profiles", summary)
@@ -210,12 +212,26 @@ def profiled_traffic(summary):
         return None
     text = open(prof).read()
     m = re.search(r"source_sha256:\s*([0-9a-f]{64})", text)
-    t = re.search(r"traffic_bytes_per_launch_4096:\s*([0-9.eE+]+)", text)
+    t = re.search(pattern, text)
     if not m or not t:
         return None
     if hashlib.sha256(open(src, "rb").read()).hexdigest() != m.group(1):
         return None
     return float(t.group(1))
+
+
+def fp64_roofline(kernel_ms, cells, peak, inst):
+    """The FP64 y sweep against the measured FP64 multiply-add rate: the instructions
+    per cell that the profiler counted on the FP64 unit (inst), two flops each -- the
+    unit's use, not the method's operations over the time.  inst None (no capture of
+    the present kernels): no fraction."""
+    achieved = None if inst is None else 2 * inst * cells / (kernel_ms / 1e3) / 1e12
+    return {"bound": "fp64 alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
+            "frac": None if achieved is None else achieved / peak, "kernel_ms": kernel_ms,
+            "fp64_instructions_per_cell": inst,
+            "kind": "use of the FP64 unit: its instructions per cell, from the committed profile "
+                    "of the same kernel source (2048^2 evolved data)",
+            "peak_kind": "measured: FP64 multiply-add microbenchmark on this GPU"}
 
 
 def cpu_sample(U0, sub, nthreads=0):
@@ -390,10 +406,16 @@ def run_gpu(args):
     flops = FLOPS_PER_FACE * cells
     achieved = flops / t_dom / 1e12
     achieved_counted = FLOPS_PER_FACE_COUNTED * cells / t_dom / 1e12
-    traffic = profiled_traffic("sweep_y_fp32_euler2d.md")
+    traffic = profiled("sweep_y_fp32_euler2d.md", TRAFFIC)
+    inst32 = profiled("sweep_y_fp32_euler2d.md", INST)
     roofline = {"bound": "alu", "achieved": achieved, "peak": fma["fp32"], "unit": "TFLOP/s",
                 "frac": achieved / fma["fp32"], "traffic": traffic,
                 "kernel": "sweep_kernel<4,5,float> y axis (stage 0, adds L_x, combines)",
+                "kind": "method-equivalent: the method's operations over the launch's time (most "
+                        "faces are proven to take the top candidate without all of them)",
+                "issued": None if inst32 is None else {
+                    "instructions_per_cell": inst32,
+                    "thread_instructions_per_s": inst32 * cells / t_dom},
                 "peak_kind": "measured: FP32 multiply-add microbenchmark on this GPU "
                              "(enoao_measure_fma_peak), 'of measured'",
                 "peak_clock_mhz": fma["clocks"].get("sm_mhz"),
@@ -407,13 +429,8 @@ def run_gpu(args):
                         "frac": BYTES_PER_CELL_Y * cells / t_dom / 1e9 / peaks["hbm_gbs"],
                         "algorithmic_bytes_per_launch": BYTES_PER_CELL_Y * cells,
                         "peak_kind": peak_kind}}
-    # the FP64 path's y sweep against the measured FP64 multiply-add rate: the instructions it
-    # issues to the FP64 unit, each as a multiply-add
-    a64 = 2 * FP64_INST_PER_CELL_Y * cells / (k_ms64[dom] / 1e3) / 1e12
-    roofline64 = {"bound": "fp64 alu", "achieved": a64, "peak": fma["fp64"], "unit": "TFLOP/s",
-                  "frac": a64 / fma["fp64"], "kernel_ms": k_ms64[dom],
-                  "fp64_instructions_per_cell": FP64_INST_PER_CELL_Y,
-                  "peak_kind": "measured: FP64 multiply-add microbenchmark on this GPU"}
+    roofline64 = fp64_roofline(k_ms64[dom], cells, fma["fp64"],
+                               profiled("sweep_y_fp64_euler2d.md", FP64_INST))
 
     launches = (s32.launches_per_step() * args.steps) if rank == 0 else 0
 
