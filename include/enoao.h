@@ -244,7 +244,8 @@ enoao_status enoao_rk_stage(enoao_ctx *ctx, int stage, double dt);
 /* Advances to t_end with dt = cfl / sum_d(alpha_d / dx_d), alpha from U^n of
  * each step, the last step shortened to land on t_end; or with the fixed
  * step dt_fixed when dt_fixed > 0.  Stops after max_steps steps when
- * max_steps > 0.  Steps run as CUDA-graph replays; alpha and dt never leave
+ * max_steps > 0.  Steps run as CUDA-graph replays, those of small 1D problems
+ * in one persistent launch (enoao_launches_per_step); alpha and dt never leave
  * the device.  Returns the time reached and the steps taken (nullable). */
 enoao_status enoao_advance(enoao_ctx *ctx, double t_end, double cfl, double dt_fixed,
                            int64_t max_steps, double *t_out, int64_t *steps_out);

@@ -233,8 +233,9 @@ int halo(int order) { return order / 2 + 2; }
 // 1: with the halo) or faces take over the threads of a line; the sweep takes
 // as many tiles as the resident blocks do in turn, and one more (the tail).
 // Candidates fill whole rounds, so ragged lengths and small grids -- which want
-// many small tiles -- come out of the same rule.  Tiles whose shared memory
-// would leave fewer than seven (FP64: three) blocks an SM are not considered.
+// many small tiles -- come out of the same rule.  Tiles of more than 33 KB (FP64:
+// 72), which leave fewer than six (three) blocks an SM, are not considered; the
+// model counts eight (three) an SM for all.
 // FP32 y and z tiles of 8 lines use half of each 128-byte line they touch
 // (256^3 z sweep: 8 x 31 1.18 ms, 16 x 16 0.82 ms); FP64 sweeps, bound by the
 // FP64 unit, take 8 lines for the smaller halo (2048^2 y sweep: 32 x 15 1.73,

@@ -2,6 +2,9 @@
 // ENO-AO library (not part of the public C interface).
 #pragma once
 
+#include <cuda.h>
+#include <cuda_runtime.h>
+
 #include <cstdint>
 
 namespace enoao {
@@ -181,10 +184,7 @@ __host__ __device__ inline void set_component_pointers(SweepArgs& a, bool fp32) 
 }
 
 // Host-side interface of the instantiation units.
-}  // namespace enoao
-#include <cuda.h>
-#include <cuda_runtime.h>
-namespace enoao {
+
 // The sweep kernel for a system, order, shape and variant, or NULL: FP32 bulk
 // re-deciding its near-ties in the sweep, the same with raw tiles staged by
 // TMA, FP32 bulk listing them for the grid-wide pass, FP64, and either

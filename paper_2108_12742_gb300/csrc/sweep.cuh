@@ -1404,9 +1404,14 @@ __device__ __forceinline__ bool prove_top(const TileView<NV, ORDER, float, FIELD
 // ingredients (narrowed on the integer units: the FP64 unit, 1/64 of the FP32
 // rate, bounds this path, and its issue slots are nine tenths idle), the
 // correction in FP64.  The proof only decides; what it cannot decide with its
-// margin -- the FP32 rounding of the differences, and of the left rows, which
-// the cancellation in c^2 = (gamma-1) (H - |v|^2/2) magnifies by up to
-// (gamma-1) H / c^2 -- goes through the FP64 indicators as before.  With every
+// margin goes through the FP64 indicators.  The margin, in units of eps = 2^-23:
+// D is off by at most (NV + 8) P (narrowing, and sums of five or seven weighted
+// terms), P the Pascal sum of |df|.  The left rows are off through c^2 = (gamma-1)
+// (H - |v|^2/2), whose terms are each off by a few roundings of H -- H by 1.5
+// (narrowing, weights, sum), |v|^2/2 by 5 (|u_l|, |u_r| <= sqrt(2 H), so also where
+// their average cancels) -- that is by 6.5 h relative, h = (gamma-1) H / c^2 >= 1 (E.H
+// E.b1); 8 h covers that and the entries' own products.  A row times D is then off
+// by at most K (NV + 8 + 8 h) P, K the largest term of the rows' entries.  With every
 // field on the top candidate R L = I, so the values need no projection: C is
 // a sum of FP64 differences, 8 NV (ENO-AO7: 12 NV) operations instead of 500.
 // 2048^2 ENO-AO5 sweeps: x 4.15 -> 1.13 ms, y 4.38 -> 1.20 ms (with choose64
@@ -1827,11 +1832,6 @@ __device__ __noinline__ bool field_faces_call(const SweepArgs& A, const TileGeo&
   return all_faces<NV, ORDER, float, COHERENT, true, SHAPE>(A, g, smem_raw, K, lgTA, sfast, nlist);
 }
 
-// One tile of a sweep (phases 1-3 above).  amax accumulates |u_d| + c of
-// combined states (last stage), nfall counts FP64 re-decisions.  FIELD: each
-// characteristic field splits with its own constant (st->alpha_f): phase 1
-// keeps dF/2 and dq/2, the split follows the projection, and the face's
-// centre part 1/2 R diag(alpha) L dq moves into its correction C.
 // Phase 2b of a tile (FP32 bulk, near-ties re-decided in the sweep): the
 // flagged choices are re-decided from the FP64 state by lane groups of the
 // warp (redo_group), or lane by lane when a warp has many (redo_lane), then
@@ -1870,184 +1870,180 @@ __device__ __forceinline__ void redecide_tile(const SweepArgs& A, const TileGeo&
   };
   auto field_window = [&](int a, int j, int sgn, int v, const R (&L)[NV], R w, R av, R (&d)[8],
                           R (&mag)[8]) { tv.field_window(a, j, sgn, v, L, w, av, d, mag); };
-    constexpr int W = 2 * G <= 8 ? 8 : 16;  // lanes per re-decision group
-    constexpr int NG = 32 / W;
-    const unsigned FULL = 0xffffffffu;
-    const int bd = blockDim.x, tid = threadIdx.x, lane = tid & 31;
-    // The flagged entries to the front of the list (one warp, in place: an
-    // entry never moves behind one not yet read), so that the choices of a
-    // warp's faces below fill its lanes.
-    __shared__ int s_nflag, s_nchoice;
-    if (tid < 32) {
-      int n = 0;
-      unsigned nc = 0;
-      for (int base = 0; base < nlist; base += 32) {
-        const unsigned e = base + lane < nlist ? tv.list[base + lane] : 0u;
-        const unsigned m = __ballot_sync(FULL, entry_flags(e) != 0u);
-        if (entry_flags(e)) tv.list[n + __popc(m & ((1u << lane) - 1u))] = e;
-        n += __popc(m);
-        nc += __popc(entry_flags(e));
-        __syncwarp();
-      }
-      nc = __reduce_add_sync(FULL, nc);
-      if (lane == 0) s_nflag = n, s_nchoice = (int)nc;
+  constexpr int W = 2 * G <= 8 ? 8 : 16;  // lanes per re-decision group
+  constexpr int NG = 32 / W;
+  const unsigned FULL = 0xffffffffu;
+  const int bd = blockDim.x, tid = threadIdx.x, lane = tid & 31;
+  // The flagged entries to the front of the list (one warp, in place: an
+  // entry never moves behind one not yet read), so that the choices of a
+  // warp's faces below fill its lanes.
+  __shared__ int s_nflag, s_nchoice;
+  if (tid < 32) {
+    int n = 0;
+    unsigned nc = 0;
+    for (int base = 0; base < nlist; base += 32) {
+      const unsigned e = base + lane < nlist ? tv.list[base + lane] : 0u;
+      const unsigned m = __ballot_sync(FULL, entry_flags(e) != 0u);
+      if (entry_flags(e)) tv.list[n + __popc(m & ((1u << lane) - 1u))] = e;
+      n += __popc(m);
+      nc += __popc(entry_flags(e));
+      __syncwarp();
     }
-    __syncthreads();
-    // The warps that share them: a round of 32 choices each (redo_lane), or, of a
-    // few choices, a round of NG (redo_group), which costs no more in all and
-    // ends sooner.  In 32 faces a warp, whatever their choices, the first warps
-    // took all and each scheduler's FP64 pipe but theirs stood idle: tiles along a
-    // front then set the length of a sweep (1024^2 quadrant jumps, per-field
-    // ENO-AO7 y sweep 320 -> 182 us, one-alpha ENO-AO5 stage 186 -> 153 us;
-    // composite wave ENO-AO7 N = 400 36.8 -> 32.2 us a step).  Where a launch has no
-    // more tiles than SMs nothing else would use the pipes: as many warps as
-    // there are rounds of NG (1D ENO-AO7 noise stage 47 -> 38 us).  Without the
-    // choices' number, by faces alone, sweeps with a choice or two a tile took
-    // longer than before (512^2 noise, ENO-AO5 stage 157 -> 163 us).
-    const int nflag = s_nflag, nchoice = s_nchoice;
-    const int few = A.redo_spread ? nchoice : 3 * NG;
-    const int nw = min(bd >> 5, nchoice <= few ? (nchoice + NG - 1) / NG : (nchoice + 31) / 32);
-    const int share = min(32, (nflag + nw - 1) / nw);  // faces of a warp at a time
-    const int wid = tid >> 5;
-    for (int base = wid < nw ? wid * share : nflag; base < nflag; base += nw * share) {
-      const unsigned entry = lane < share && base + lane < nflag ? tv.list[base + lane] : 0u;
-      const int al = entry_line(entry), f = entry_face(entry);
-      const int j = G - 1 + f;
-      unsigned fix = entry_flags(entry);
-      // The warp's T choices in rounds (with each face's lane serving its own
-      // flags, a warp took up to ten rounds for a few choices each: 256^3
-      // ENO-AO7 x sweep 1.8 -> 1.0 ms, 800^2 0.23 -> 0.16 ms).  Many left: one per lane (redo_lane),
-      // 32 in a round -- an instruction of the FP64 unit costs the same
-      // whatever its active lanes.  A few left: NG per round, each by W lanes
-      // together (redo_group), which takes about 2/5 (ENO-AO5) or 1/3 of the
-      // instructions of a lone re-decision.  Every round clears at least one
-      // choice, so the default bound (64 NV rounds) is never reached; a
-      // smaller bound (a test knob) can be: then the error word says so and
-      // the choices left keep their FP32 pick.
-      const int m = __popc(fix);
-      int pre = m;  // inclusive, then exclusive prefix sum over the lanes
+    nc = __reduce_add_sync(FULL, nc);
+    if (lane == 0) s_nflag = n, s_nchoice = (int)nc;
+  }
+  __syncthreads();
+  // The warps that share them: a round of 32 choices each (redo_lane), or, of a
+  // few choices, a round of NG (redo_group), which costs no more in all and
+  // ends sooner.  In 32 faces a warp, whatever their choices, the first warps
+  // took all and each scheduler's FP64 pipe but theirs stood idle: tiles along a
+  // front then set the length of a sweep (1024^2 quadrant jumps, per-field
+  // ENO-AO7 y sweep 320 -> 182 us, one-alpha ENO-AO5 stage 186 -> 153 us;
+  // composite wave ENO-AO7 N = 400 36.8 -> 32.2 us a step).  Where a launch has no
+  // more tiles than SMs nothing else would use the pipes: as many warps as
+  // there are rounds of NG (1D ENO-AO7 noise stage 47 -> 38 us).  Without the
+  // choices' number, by faces alone, sweeps with a choice or two a tile took
+  // longer than before (512^2 noise, ENO-AO5 stage 157 -> 163 us).
+  const int nflag = s_nflag, nchoice = s_nchoice;
+  const int few = A.redo_spread ? nchoice : 3 * NG;
+  const int nw = min(bd >> 5, nchoice <= few ? (nchoice + NG - 1) / NG : (nchoice + 31) / 32);
+  const int share = min(32, (nflag + nw - 1) / nw);  // faces of a warp at a time
+  const int wid = tid >> 5;
+  for (int base = wid < nw ? wid * share : nflag; base < nflag; base += nw * share) {
+    const unsigned entry = lane < share && base + lane < nflag ? tv.list[base + lane] : 0u;
+    const int al = entry_line(entry), f = entry_face(entry);
+    const int j = G - 1 + f;
+    unsigned fix = entry_flags(entry);
+    // The warp's T choices in rounds (with each face's lane serving its own
+    // flags, a warp took up to ten rounds for a few choices each: 256^3
+    // ENO-AO7 x sweep 1.8 -> 1.0 ms, 800^2 0.23 -> 0.16 ms).  Many left: one per lane (redo_lane),
+    // 32 in a round -- an instruction of the FP64 unit costs the same
+    // whatever its active lanes.  A few left: NG per round, each by W lanes
+    // together (redo_group), which takes about 2/5 (ENO-AO5) or 1/3 of the
+    // instructions of a lone re-decision.  Every round clears at least one
+    // choice, so the default bound (64 NV rounds) is never reached; a
+    // smaller bound (a test knob) can be: then the error word says so and
+    // the choices left keep their FP32 pick.
+    const int m = __popc(fix);
+    int pre = m;  // inclusive, then exclusive prefix sum over the lanes
 #pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int t = __shfl_up_sync(FULL, pre, o);
-        if (lane >= o) pre += t;
+    for (int o = 1; o < 32; o <<= 1) {
+      const int t = __shfl_up_sync(FULL, pre, o);
+      if (lane >= o) pre += t;
+    }
+    const int T = __shfl_sync(FULL, pre, 31);
+    pre -= m;
+    unsigned long long picks = 0ull;
+    int done = 0;
+    for (int pass = 0; done < T; ++pass) {
+      if (pass >= A.redo_passes) {
+        if (lane == 0) atomicOr(&st->err, kErrTimeout);
+        break;
       }
-      const int T = __shfl_sync(FULL, pre, 31);
-      pre -= m;
-      unsigned long long picks = 0ull;
-      int done = 0;
-      for (int pass = 0; done < T; ++pass) {
-        if (pass >= A.redo_passes) {
-          if (lane == 0) atomicOr(&st->err, kErrTimeout);
-          break;
-        }
-        const bool lone = T - done > (ORDER == 7 ? 3 : 2) * NG;
-        const int per = lone ? 32 : NG;
-        // this lane's (its group's) choice of the round: number ci, of the
-        // face of lane jl
-        const int ci = done + (lone ? lane : lane / W);
-        int jl = 0;
+      const bool lone = T - done > (ORDER == 7 ? 3 : 2) * NG;
+      const int per = lone ? 32 : NG;
+      // this lane's (its group's) choice of the round: number ci, of the
+      // face of lane jl
+      const int ci = done + (lone ? lane : lane / W);
+      int jl = 0;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {  // the last lane whose first choice is <= ci
-          const int pq = __shfl_sync(FULL, pre, jl + o);
-          if (pq <= ci) jl += o;
-        }
-        const unsigned mj = __shfl_sync(FULL, fix, jl);
-        const int prej = __shfl_sync(FULL, pre, jl);
-        const int aj = __shfl_sync(FULL, al, jl), fj = __shfl_sync(FULL, f, jl);
-        const bool valid = ci < T;
-        const int kb = valid ? nth_set_bit(mj, ci - prej) : 0;
-        // (a group without a choice works on the face of the last one, unused)
-        const int k = kb < 0 ? 0 : kb;
-        int pick = 0;
-        if (lone) {
-          if (valid)
-            pick = redo_lane<NV, ORDER, COHERENT>(A, g, aj, g.s0 + fj - 1, k >> 1, k & 1,
-                                                  alpha64(k >> 1));
-        } else {
-          pick = redo_group<NV, ORDER, COHERENT, W>(A, g, aj, g.s0 + fj - 1, k >> 1, k & 1,
-                                                    alpha64(k >> 1), lane & (W - 1));
-        }
-        __syncwarp();
-        // each face's lane collects its choices of the round
-        unsigned todo = fix;
-        int most = __reduce_max_sync(FULL, (unsigned)m);
-        for (int t = 0; t < most; ++t) {
-          const int c = pre + t - done;
-          const int src = c >= 0 && c < per ? (lone ? c : c * W) : 0;
-          const int got = __shfl_sync(FULL, pick, src);
-          const int kk = todo ? __ffs(todo) - 1 : 0;
-          todo &= todo - 1;
-          if (t < m && c >= 0 && c < per) {
-            picks |= (unsigned long long)got << (4 * kk);
-            ++nfall;
-          }
-        }
-        done += per;
+      for (int o = 16; o > 0; o >>= 1) {  // the last lane whose first choice is <= ci
+        const int pq = __shfl_sync(FULL, pre, jl + o);
+        if (pq <= ci) jl += o;
       }
-      // choices left by a pass bound keep their FP32 pick
-      const int have = done - pre < 0 ? 0 : (done - pre < m ? done - pre : m);
-      for (int t = m; t > have; --t) fix &= ~(1u << (31 - __clz(fix)));
-      if (!fix) continue;
-      // apply the changed choices of this face
-      Eigen<NV, R> E;
-      if constexpr (NV > 1) {
-        face_eigen<NV, ORDER, R, FIELD>(tv, sidx(al, j), gm1, E);
+      const unsigned mj = __shfl_sync(FULL, fix, jl);
+      const int prej = __shfl_sync(FULL, pre, jl);
+      const int aj = __shfl_sync(FULL, al, jl), fj = __shfl_sync(FULL, f, jl);
+      const bool valid = ci < T;
+      const int kb = valid ? nth_set_bit(mj, ci - prej) : 0;
+      // (a group without a choice works on the face of the last one, unused)
+      const int k = kb < 0 ? 0 : kb;
+      int pick = 0;
+      if (lone) {
+        if (valid)
+          pick = redo_lane<NV, ORDER, COHERENT>(A, g, aj, g.s0 + fj - 1, k >> 1, k & 1,
+                                                alpha64(k >> 1));
+      } else {
+        pick = redo_group<NV, ORDER, COHERENT, W>(A, g, aj, g.s0 + fj - 1, k >> 1, k & 1,
+                                                  alpha64(k >> 1), lane & (W - 1));
       }
-      const long long gface = g.s0 + f;
-      const bool own = (gface <= g.nd) && (f < A.ts || gface == g.nd);
-      R dC[NV];
+      __syncwarp();
+      // each face's lane collects its choices of the round
+      unsigned todo = fix;
+      int most = __reduce_max_sync(FULL, (unsigned)m);
+      for (int t = 0; t < most; ++t) {
+        const int c = pre + t - done;
+        const int src = c >= 0 && c < per ? (lone ? c : c * W) : 0;
+        const int got = __shfl_sync(FULL, pick, src);
+        const int kk = todo ? __ffs(todo) - 1 : 0;
+        todo &= todo - 1;
+        if (t < m && c >= 0 && c < per) {
+          picks |= (unsigned long long)got << (4 * kk);
+          ++nfall;
+        }
+      }
+      done += per;
+    }
+    // choices left by a pass bound keep their FP32 pick
+    const int have = done - pre < 0 ? 0 : (done - pre < m ? done - pre : m);
+    for (int t = m; t > have; --t) fix &= ~(1u << (31 - __clz(fix)));
+    if (!fix) continue;
+    // apply the changed choices of this face
+    Eigen<NV, R> E;
+    if constexpr (NV > 1) {
+      face_eigen<NV, ORDER, R, FIELD>(tv, sidx(al, j), gm1, E);
+    }
+    const bool own = owns_face(A, g, f);
+    R dC[NV];
 #pragma unroll
-      for (int c = 0; c < NV; ++c) dC[c] = R(0);
+    for (int c = 0; c < NV; ++c) dC[c] = R(0);
 #pragma unroll 1
-      for (int k = 0; k < 2 * NV; ++k) {
-        if (!(fix & (1u << k))) continue;
-        const int v = k >> 1, sgn = k & 1;
-        const int pick = (int)((picks >> (4 * k)) & 15ull);
-        const bool shear = NV >= 4 && v >= 2 && v <= NV - 2;
-        R L[NV], w = R(0);
-        if constexpr (NV > 1) {
-          left_row<NV, R>(E, v, L);
-          if constexpr (NV >= 4) w = -L[0];
+    for (int k = 0; k < 2 * NV; ++k) {
+      if (!(fix & (1u << k))) continue;
+      const int v = k >> 1, sgn = k & 1;
+      const int pick = (int)((picks >> (4 * k)) & 15ull);
+      const bool shear = NV >= 4 && v >= 2 && v <= NV - 2;
+      R L[NV], w = R(0);
+      if constexpr (NV > 1) {
+        left_row<NV, R>(E, v, L);
+        if constexpr (NV >= 4) w = -L[0];
+      } else {
+        L[0] = R(1);
+      }
+      R d[8], mag[8];
+      field_window(al, j, sgn, v, L, w, afield(v), d, mag);
+      int pick_old;
+      bool m;
+      const R nomx[8] = {R(0), R(0), R(0), R(0), R(0), R(0), R(0), R(0)};
+      const R corr_old = eno_select<ORDER, R, false>(d, delta, tie_rel, nomx, R(0), pick_old, m);
+      if (pick != pick_old) {
+        R corr = R(0);
+#pragma unroll
+        for (int i = GE::LO; i <= GE::HI; ++i) corr = fma(bcoef<R>(pick, i), d[i], corr);
+        const R dv = corr - corr_old;
+        if (shear) {
+#pragma unroll
+          for (int c = 2; c < NV - 1; ++c) dC[c] += c == v ? dv : R(0);
+          dC[NV - 1] = fma(w, dv, dC[NV - 1]);
+        } else if constexpr (NV > 1) {
+          R Rc[NV];
+          right_col<NV, R>(E, v, Rc);
+#pragma unroll
+          for (int c = 0; c < NV; ++c) dC[c] = fma(Rc[c], dv, dC[c]);
         } else {
-          L[0] = R(1);
-        }
-        R d[8], mag[8];
-        field_window(al, j, sgn, v, L, w, afield(v), d, mag);
-        int pick_old;
-        bool m;
-        const R nomx[8] = {R(0), R(0), R(0), R(0), R(0), R(0), R(0), R(0)};
-        const R corr_old = eno_select<ORDER, R, false>(d, delta, tie_rel, nomx, R(0), pick_old, m);
-        if (pick != pick_old) {
-          R corr = R(0);
-#pragma unroll
-          for (int i = GE::LO; i <= GE::HI; ++i) corr = fma(bcoef<R>(pick, i), d[i], corr);
-          const R dv = corr - corr_old;
-          if (shear) {
-#pragma unroll
-            for (int c = 2; c < NV - 1; ++c) dC[c] += c == v ? dv : R(0);
-            dC[NV - 1] = fma(w, dv, dC[NV - 1]);
-          } else if constexpr (NV > 1) {
-            R Rc[NV];
-            right_col<NV, R>(E, v, Rc);
-#pragma unroll
-            for (int c = 0; c < NV; ++c) dC[c] = fma(Rc[c], dv, dC[c]);
-          } else {
-            dC[0] += dv;
-          }
-        }
-        if ((mode & kModeFlux) && A.idx_out && own) {
-          const long long nf = A.nfaces;
-          const long long fc = g.fbase + (g.a0 + al) * g.fstride_a + gface * g.fstride_d;
-          A.idx_out[(v * 2 + sgn) * nf + fc] = (int8_t)pick;
+          dC[0] += dv;
         }
       }
-      const int sj = sidx(al, j);
-      R Cv[NV];
-      CV::load(Cf, cells, sj, Cv);
-#pragma unroll
-      for (int c = 0; c < NV; ++c) Cv[c] += dC[c];
-      CV::store(Cf, cells, sj, Cv);
+      if ((mode & kModeFlux) && A.idx_out && own)
+        A.idx_out[(v * 2 + sgn) * A.nfaces + face_index(g, al, f)] = (int8_t)pick;
     }
+    const int sj = sidx(al, j);
+    R Cv[NV];
+    CV::load(Cf, cells, sj, Cv);
+#pragma unroll
+    for (int c = 0; c < NV; ++c) Cv[c] += dC[c];
+    CV::store(Cf, cells, sj, Cv);
+  }
   __syncthreads();
 }
 
@@ -2061,6 +2057,11 @@ __device__ __noinline__ void redecide_tile_call(const SweepArgs& A, const TileGe
   redecide_tile<NV, ORDER, COHERENT, FIELD, SHAPE>(A, g, smem_raw, nlist, alpha_d, nfall);
 }
 
+// One tile of a sweep (phases 1-3 above).  amax accumulates |u_d| + c of
+// combined states (last stage), nfall counts FP64 re-decisions.  FIELD: each
+// characteristic field splits with its own constant (st->alpha_f): phase 1
+// keeps dF/2 and dq/2, the split follows the projection, and the face's
+// centre part 1/2 R diag(alpha) L dq moves into its correction C.
 // TMA: phase 1 reads the tile's raw state from rt instead of global memory.
 // PROOF: prove faces first, where the sweep can (kProve).
 // hook() runs before the tile's last barrier, with TMA once every thread is
@@ -2081,8 +2082,8 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& A, const TileGeo& g,
   // the code of faces not proven and of near-ties out of line
   constexpr bool CALL = FP32 && !FIELD && SHAPE != kShapeAny;
   StepState* st = A.st;
-  const int TA = A.ta, TS = A.ts;
-  // row pitch A.se (>= TS + 2G), chosen on the host for conflict-free banks
+  const int TA = A.ta;
+  // row pitch A.se (>= A.ts + 2G), chosen on the host for conflict-free banks
   const TileView<NV, ORDER, R, FIELD> tv(smem_raw, TA, A.se);
   const int cells = tv.cells;
   R* const dfp = tv.dfp;
@@ -2099,23 +2100,8 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& A, const TileGeo& g,
   const double alpha_d = K.alpha_d, dt = K.dt;
   const R alpha = K.alpha;
   const R halpha = R(0.5) * alpha;
-  // splitting constant of field v: alpha, or per field max |u_d - c|, |u_d|, |u_d + c|
-  R alo = alpha, amid = alpha, ahi = alpha;
-  if constexpr (FIELD) {
-    alo = (R)st->alpha_f[A.dir][0];
-    amid = (R)st->alpha_f[A.dir][1];
-    ahi = (R)st->alpha_f[A.dir][2];
-  }
-  auto afield = [&](int v) { return v == 0 ? alo : (v == NV - 1 ? ahi : amid); };
-  // the same in FP64, for the re-decisions of near-ties
-  auto alpha64 = [&](int v) {
-    if constexpr (FIELD) return field_alpha<NV>(st, A.dir, v);
-    return alpha_d;
-  };
   const R gm1 = bconst<R>(A.gm1, A.gm1_f);
   const R adv = bconst<R>(A.adv_speed, A.adv_f);
-  const R delta = bconst<R>(A.delta, A.delta_f);
-  const R tie_rel = bconst<R>(A.tie_rel, A.tie_rel_f);
   const int mode = shape_mode<SHAPE>(A);
   const R inv_dx_r = K.inv_dx;
   // FP32 bulk combine: dt and the stage's weight of dt L in FP32
@@ -2127,11 +2113,6 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& A, const TileGeo& g,
   auto sidx = [&](int a, int e) { return tv.sidx(a, e); };
   using CV = CellVec<NV, R, FIELD>;
   const int lgTA = __ffs(TA) - 1;  // TA is a power of two (checked on the host)
-  (void)TS;
-  // Projected window of field v (the same arithmetic in phase 2 and in the
-  // phase-2b check of a flagged choice, which must reproduce its pick).
-  auto field_window = [&](int a, int j, int sgn, int v, const R (&L)[NV], R w, R av, R (&d)[8],
-                          R (&mag)[8]) { tv.field_window(a, j, sgn, v, L, w, av, d, mag); };
   const int nts = g.nts;
   const int sext = nts + 2 * G;  // extended cells in use
   // extended cell e of line a is cell ext0 + a sa + e sd, except ghosts of a
@@ -2328,8 +2309,8 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& A, const TileGeo& g,
     const long long nf = A.nfaces;
     for_items(lgTA, cnt, sfast, [&](const int a, const int f) {
       if (g.a0 + a >= g.na) return;
+      if (!owns_face(A, g, f)) return;
       const long long gface = g.s0 + f;
-      if (!((gface <= g.nd) && (f < A.ts || gface == g.nd))) return;
       const int j = G - 1 + f;
       const long long la = g.base + (g.a0 + a) * g.stride_a;
       double ql[NV], qr[NV], Fl[NV], Fr[NV];
@@ -2337,7 +2318,7 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& A, const TileGeo& g,
       load_state<NV, COHERENT>(A, la + bc_map(gface, g.nd, A.bc) * g.stride_d, qr);
       phys_flux<NV>(ql, A.gm1, A.adv_speed, Fl);
       phys_flux<NV>(qr, A.gm1, A.adv_speed, Fr);
-      const long long fc = g.fbase + (g.a0 + a) * g.fstride_a + gface * g.fstride_d;
+      const long long fc = face_index(g, a, f);
       R Cv[NV];
       CV::load(Cf, cells, sidx(a, j), Cv);
 #pragma unroll
@@ -2530,12 +2511,6 @@ constexpr int sweep_min_blocks() {
 // the error word and returns instead of spinning on.
 constexpr long long kTmaPollLimit = 1ll << 24;
 
-// TMA: the tile's raw state (every component, the tile's lines, its cells and
-// halo along the swept axis) is one box of the tensor map tmap, copied into
-// the first A.tma_raw_bytes of dynamic shared memory by thread 0; the copy of
-// the next tile is issued as soon as phase 1 of the current one is done, so
-// it lands while phases 2 and 3 run.  Ghost cells outside the grid (the box
-// reads zeros there) are then filled from the boundary map with plain loads.
 // The end of a sweep launch, for every block: the last block to leave resets
 // the tile queue (and the re-decision epoch), the FP64 re-decision count is
 // added up, and the block's maxima of the new state's speeds go to alpha.
@@ -2599,6 +2574,12 @@ __device__ __forceinline__ void sweep_epilogue(const SweepArgs& A, double (&amax
   }
 }
 
+// TMA: the tile's raw state (every component, the tile's lines, its cells and
+// halo along the swept axis) is one box of the tensor map tmap, copied into
+// the first A.tma_raw_bytes of dynamic shared memory by thread 0; the copy of
+// the next tile is issued as soon as phase 1 of the current one is done, so
+// it lands while phases 2 and 3 run.  Ghost cells outside the grid (the box
+// reads zeros there) are then filled from the boundary map with plain loads.
 template <int NV, int ORDER, typename R, bool DEFER = false, bool FIELD = false, bool TMA = false,
           int SHAPE = kShapeAny>
 __global__ void __launch_bounds__(128, sweep_min_blocks<NV, ORDER, R, FIELD, TMA>())
