@@ -298,7 +298,7 @@ BatchArgs make_args(enoao_ctx* c, int nsteps, double cfl) {
     A.delta = c->cfg.delta;
     A.tie_rel = c->cfg.tie_rel;
     A.inv_dx = 1.0;  // per problem
-    A.redo_spread = b->nprob <= c->sms;
+    A.redo_split = b->nprob <= c->sms ? kSplitAll : kSplitDense;
     A.redo_passes = 64 * b->nv;
     set_derived_constants(A);
     set_component_pointers(A, f32);

@@ -489,7 +489,7 @@ enoao_status fill_sweep_args(enoao_ctx* c, int d, int stage, int mode, const dou
     a.tiles_b = d == 1 ? c->cfg.n[2] : c->cfg.n[1];
   }
   a.ntiles = a.tiles_s * a.tiles_a * a.tiles_b;
-  a.redo_spread = a.ntiles <= c->sms;
+  a.redo_split = a.ntiles <= c->sms ? kSplitAll : kSplitSweep;
   if (a.ntiles >= (1ll << 31)) return fail(c, ENOAO_EINVAL, "too many tiles for axis %d", d);
   a.inv_dx = 1.0 / c->dx[d];
   a.gamma = c->cfg.gamma;

@@ -100,6 +100,11 @@ inline int sweep_shape(int dir, int mode) {
   return kShapeAny;
 }
 
+// How a tile's re-decisions are split over the warps of its block (redecide_tile):
+// for the least work in all (batches), ending sooner for little more (sweeps), or
+// soonest (launches with no more tiles than SMs).
+enum RedoSplit { kSplitDense, kSplitSweep, kSplitAll };
+
 struct SweepArgs {
   ComponentPtrs comp;
   const double* u_in;   // U^(s): stencil source, [nv][N]
@@ -137,7 +142,7 @@ struct SweepArgs {
   int tma_box;          // TMA: box extent along the swept axis (cells, with alignment slack)
   unsigned tma_bytes;   // TMA: bytes of one box
   int tma_raw_bytes;    // TMA: shared memory reserved for the box (a multiple of 128)
-  int redo_spread;      // FP32 bulk: 1 where the launch has no more tiles than SMs
+  int redo_split;       // FP32 bulk: how a tile's re-decisions go to its warps (RedoSplit)
   int redo_passes;      // FP32 bulk: bound on the in-sweep re-decision passes of a warp
                         // round; reaching it sets kErrTimeout (64 nv by default)
   long long tiles_s;    // tiles along dir

@@ -199,7 +199,7 @@ extern "C" enoao_status enoao_step_noalloc(const enoao_config* cfg, const double
   a.tiles_s = (n + a.ts - 1) / a.ts;
   a.tiles_a = a.tiles_b = 1;
   a.ntiles = a.tiles_s;
-  a.redo_spread = a.ntiles <= sms;
+  a.redo_split = a.ntiles <= sms ? kSplitAll : kSplitSweep;
   a.inv_dx = 1.0 / ((cfg->hi[0] - cfg->lo[0]) / (double)n);
   a.gamma = cfg->gamma;
   a.adv_speed = cfg->adv_speed;

@@ -1872,6 +1872,7 @@ __device__ __forceinline__ void redecide_tile(const SweepArgs& A, const TileGeo&
                           R (&mag)[8]) { tv.field_window(a, j, sgn, v, L, w, av, d, mag); };
   constexpr int W = 2 * G <= 8 ? 8 : 16;  // lanes per re-decision group
   constexpr int NG = 32 / W;
+  constexpr int kFewRounds = ORDER == 7 ? 3 : 2;  // rounds of redo_group that cost a lone one
   const unsigned FULL = 0xffffffffu;
   const int bd = blockDim.x, tid = threadIdx.x, lane = tid & 31;
   // The flagged entries to the front of the list (one warp, in place: an
@@ -1894,19 +1895,24 @@ __device__ __forceinline__ void redecide_tile(const SweepArgs& A, const TileGeo&
   }
   __syncthreads();
   // The warps that share them: a round of 32 choices each (redo_lane), or, of a
-  // few choices, a round of NG (redo_group), which costs no more in all and
+  // few choices, a round of NG (redo_group), which costs little more in all and
   // ends sooner.  In 32 faces a warp, whatever their choices, the first warps
   // took all and each scheduler's FP64 pipe but theirs stood idle: tiles along a
   // front then set the length of a sweep (1024^2 quadrant jumps, per-field
-  // ENO-AO7 y sweep 320 -> 182 us, one-alpha ENO-AO5 stage 186 -> 153 us;
-  // composite wave ENO-AO7 N = 400 36.8 -> 32.2 us a step).  Where a launch has no
-  // more tiles than SMs nothing else would use the pipes: as many warps as
-  // there are rounds of NG (1D ENO-AO7 noise stage 47 -> 38 us).  Without the
-  // choices' number, by faces alone, sweeps with a choice or two a tile took
-  // longer than before (512^2 noise, ENO-AO5 stage 157 -> 163 us).
+  // ENO-AO7 y sweep 309 -> 179 us, one-alpha ENO-AO5 stage 186 -> 152 us; composite
+  // wave ENO-AO7 N = 400 33.3 -> 28.3 us a step).  Where a launch has no more tiles
+  // than SMs nothing else would use the pipes: as many warps as there are
+  // rounds of NG.  In a batch the blocks' other problems do: no more rounds in
+  // all than one warp would take (1024 uneven problems, ENO-AO5: 1.00 ms a step
+  // either way, 1.09 split as sweeps are).  By faces alone, without the choices'
+  // number, sweeps with a choice or two a tile took longer than in one warp
+  // (512^2 noise, ENO-AO5 stage 157 -> 163 us).
   const int nflag = s_nflag, nchoice = s_nchoice;
-  const int few = A.redo_spread ? nchoice : 3 * NG;
-  const int nw = min(bd >> 5, nchoice <= few ? (nchoice + NG - 1) / NG : (nchoice + 31) / 32);
+  const bool dense = A.redo_split == kSplitDense;
+  const int few = A.redo_split == kSplitAll ? nchoice : (dense ? kFewRounds : 3) * NG;
+  const int rounds = nchoice <= few ? (nchoice + NG - 1) / NG
+                     : dense ? max(nchoice / 32, (nflag + 31) / 32) : (nchoice + 31) / 32;
+  const int nw = min(bd >> 5, rounds);
   const int share = min(32, (nflag + nw - 1) / nw);  // faces of a warp at a time
   const int wid = tid >> 5;
   for (int base = wid < nw ? wid * share : nflag; base < nflag; base += nw * share) {
@@ -1940,7 +1946,7 @@ __device__ __forceinline__ void redecide_tile(const SweepArgs& A, const TileGeo&
         if (lane == 0) atomicOr(&st->err, kErrTimeout);
         break;
       }
-      const bool lone = T - done > (ORDER == 7 ? 3 : 2) * NG;
+      const bool lone = T - done > kFewRounds * NG;
       const int per = lone ? 32 : NG;
       // this lane's (its group's) choice of the round: number ci, of the
       // face of lane jl
