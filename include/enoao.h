@@ -275,7 +275,8 @@ int enoao_launches_per_step(const enoao_ctx *ctx);
 
 /* Tile shape of the sweep kernels along each axis: lines per tile (ta) and
  * faces per tile (ts).  Set by the autotuner or by hand; 0 keeps the current
- * value.  Errors: ENOAO_EINVAL for shapes the kernels do not support.  (1D
+ * value.  Until then enoao_set_redecide may choose other defaults for its mode.
+ * Errors: ENOAO_EINVAL for shapes the kernels do not support.  (1D
  * runs in one persistent launch choose their tile themselves.) */
 enoao_status enoao_set_tiles(enoao_ctx *ctx, int dir, int ta, int ts);
 enoao_status enoao_get_tiles(const enoao_ctx *ctx, int dir, int *ta, int *ts);

@@ -279,12 +279,27 @@ void pick_tile(const enoao_ctx* c, int d, int* ta_out, int* ts_out) {
 // line fill whole warps in the per-face phase.  (FP64 y and z: 32 x 15 took a
 // whole SM for one block in 3D: 96^3 ENO-AO5 y sweep 2.00 -> 1.58 ms, 256^3 36.4 ->
 // 27.6 ms, 1024^2 1.46 -> 1.32 ms.)
+// With the grid-wide pass (2D Euler, eight tiles an SM and more), whose flows list
+// many faces: whole rounds of 128 listed faces, y 8 x 31 and, where ENO-AO7's
+// selection counts, x no less than 4 x 63 (2D Riemann configuration 2, 800^2, late:
+// ENO-AO7 x 2 x 54 92.6 -> 86.6 us, y 16 x 14 103 -> 94, ENO-AO5 y 16 x 15 73.7 -> 71.8; on
+// 800^2 fronts of a cell or two ENO-AO7 51 + 59 -> 46 + 59 us, ENO-AO5 y 49.6 -> 50.4).
+bool use_list(const enoao_ctx* c);
 void default_tiles(enoao_ctx* c) {
   const bool f32 = fp32(c), prove = !consts(c).field;
+  const bool lists = use_list(c) && c->nv == 4;
+  const auto tiles = [&](int lines, int cells, int ta, int ts) {
+    return (long long)((c->cfg.n[lines] + ta - 1) / ta) * ((c->cfg.n[cells] + ts - 1) / ts);
+  };
   for (int d = 0; d < c->cfg.ndim; ++d) {
+    if (c->tiles_set[d]) continue;
     c->block[d] = 128;
     if (prove) {
       pick_tile(c, d, &c->ta[d], &c->ts[d]);
+      if (lists && d == 0 && c->cfg.order == 7 && c->ta[0] * c->ts[0] < 4 * 63 &&
+          tiles(1, 0, 4, 63) >= 8 * c->sms)
+        c->ta[0] = 4, c->ts[0] = 63;
+      if (lists && d == 1 && tiles(0, 1, 8, 31) >= 8 * c->sms) c->ta[1] = 8, c->ts[1] = 31;
     } else if (d == 0) {
       c->ta[d] = c->cfg.ndim == 1 ? 1 : 4;
       c->ts[d] = 63;
@@ -1292,6 +1307,7 @@ enoao_status enoao_set_redecide(enoao_ctx* c, int mode) {
     c->redecide = prev;
     return r;
   }
+  if (!c->batch) default_tiles(c);
   if (c->graph) {
     cudaGraphExecDestroy(c->graph);
     c->graph = nullptr;
@@ -1380,6 +1396,7 @@ enoao_status enoao_set_tiles(enoao_ctx* c, int dir, int ta, int ts) {
   if (r != ENOAO_OK) return r;
   c->ta[dir] = ta;
   c->ts[dir] = ts;
+  c->tiles_set[dir] = 1;
   if (c->graph) {
     cudaGraphExecDestroy(c->graph);
     c->graph = nullptr;
@@ -1433,7 +1450,6 @@ enoao_status enoao_autotune(enoao_ctx* c) {
   enoao_status r = enter(c);
   if (r != ENOAO_OK) return r;
   CU(c, cudaMemcpyAsync(c->U[2], c->U[0], bytes, cudaMemcpyDeviceToDevice, c->s));
-  const bool f32 = fp32(c);
   const bool list = use_list(c);  // candidates timed with the pass steps launch after them
   for (int d = 0; d < c->cfg.ndim; ++d) {
     std::vector<std::pair<int, int>> cands;
@@ -1482,7 +1498,7 @@ enoao_status enoao_autotune(enoao_ctx* c) {
     }
     c->ta[d] = bta;
     c->ts[d] = bts;
-    (void)f32;
+    c->tiles_set[d] = 1;
   }
   if (c->graph) {
     cudaGraphExecDestroy(c->graph);

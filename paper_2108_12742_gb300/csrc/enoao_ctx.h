@@ -43,6 +43,7 @@ struct enoao_ctx {
   enoao::StepState* st = nullptr;       // device
   enoao::StepState* st_host = nullptr;  // pinned mirror
   int ta[3] = {0, 0, 0}, ts[3] = {0, 0, 0}, block[3] = {128, 128, 128};
+  int tiles_set[3] = {0, 0, 0};         // 1: ta, ts chosen by the caller or the autotuner
   int sms = 0;
   cudaGraphExec_t graph = nullptr;
   int graph_steps = 0;

@@ -81,3 +81,26 @@ def test_grid_pass_on_ties_that_rounding_decides(shape, order):
     grid, sweep = out
     off = np.abs(grid - sweep).max(axis=0) / np.abs(sweep - U).max()
     assert off.max() <= TOL, (off.max(), int((off > TOL).sum()))
+
+
+@pytest.mark.parametrize("order", [5, 7])
+def test_tiles_of_the_mode_do_not_show_and_callers_tiles_stay(order):
+    shape = (800, 400)  # eight tiles an SM and more
+    U = inputs.riemann2d(2, *shape)
+    out = []
+    for own in (None, ((2, 63), (16, 15))):
+        with eno.Solver(shape, (-1.0, -1.0), (1.0, 1.0), system=eno.EULER, order=order,
+                        precision=eno.FP32_BULK, bc=eno.TRANSMISSIVE) as s:
+            before = [s.get_tiles(d) for d in range(2)]
+            if own:
+                for d, t in enumerate(own):
+                    s.set_tiles(d, *t)
+            s.set_redecide(eno.REDECIDE_GRID)
+            if own:
+                assert [s.get_tiles(d) for d in range(2)] == list(own)
+            s.init_state(U)
+            s.advance_steps(10, 0.5)
+            out.append(s.get_state())
+            s.set_redecide(eno.REDECIDE_IN_SWEEP)
+            assert [s.get_tiles(d) for d in range(2)] == (list(own) if own else before)
+    assert np.array_equal(*out)
