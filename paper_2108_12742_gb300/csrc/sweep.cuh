@@ -1265,9 +1265,9 @@ __device__ __forceinline__ void face_eigen(const TileView<NV, ORDER, R, FIELD>& 
 // near-tie.  One difference decides a field instead of two per candidate and
 // their bounds; the faces of resolved flow end here (98 to 99.5 % of 2D data
 // at 2048^2 and more), the others go to the tile's face list.  The sweeps are
-// bound by issue slots: 1,440 instructions per face and cell before, 840 (x)
-// and 1,120 (y) with it; 4096^2 ENO-AO5 sweeps 0.81 -> 0.52 ms (x, 2 x 120
-// tiles) and 1.00 -> 0.69 ms (y, 16 x 15), 512^3 ENO-AO7 stage 53 -> 27 ms.
+// bound by issue slots: 1,440 instructions per face and cell before, 815 (x)
+// and 1,060 (y) with it; 4096^2 ENO-AO5 sweeps 0.81 -> 0.52 ms (x, 2 x 120
+// tiles) and 1.00 -> 0.69 ms (y, 16 x 15), 512^3 ENO-AO7 stage 54 -> 28 ms.
 // (Without the projection, as the FP64 path does it, they took 0.41 and 0.60
 // ms; but R (L s) and s differ by FP32 rounding, which later stages' near-ties
 // turn into other choices.)
@@ -2494,7 +2494,8 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& A, const TileGeo& g,
 // spilled around the out-of-line calls) for ENO-AO5 and scalars, six (80) for
 // ENO-AO7 of the Euler equations, whose selection spills at 64 (512^3 stage 29.1 ->
 // 28.0 ms, 1024^2 jumps 237 -> 229 us, 512^2 noise, every face selected, 208 -> 201 us;
-// scalars at 80: 1024^2 sine 44 -> 48 us).
+// where it was slower: 96^3 noise 0.99 -> 1.01 ms; scalars at 80: 1024^2 sine 44 ->
+// 48 us).
 #ifndef ENOAO_FP32_MIN_BLOCKS
 #define ENOAO_FP32_MIN_BLOCKS 8
 #endif
@@ -2726,7 +2727,7 @@ __global__ void __launch_bounds__(128, sweep_min_blocks<NV, ORDER, R, FIELD, TMA
 // as separate launches would take them; the host makes the 2D tile a whole
 // number of both axes' sub-tiles (Ay.ts % Ax.ta == 0, Ax.ts % Ay.ta == 0).
 // (ENO-AO7: five blocks, 96 registers for both parts in one kernel; 1024^2 jumps
-// 1.03 -> 0.92 ms a stage)
+// 1.04 -> 0.94 ms a stage)
 template <int NV, int ORDER>
 __global__ void __launch_bounds__(128, ORDER == 7 ? 5 : ENOAO_FP32_MIN_BLOCKS)
     fused2d_kernel(const __grid_constant__ SweepArgs Ax, const __grid_constant__ SweepArgs Ay) {
