@@ -1528,18 +1528,28 @@ struct TileConst {
   float dt32, wdt32;    // FP32 bulk combine: dt and the stage's weight of dt L
   float limit;          // bound of prove_top
   R inv_dx;
-  R af[3];              // per field: splitting constants of u-c, of entropy and shear, of u+c
 };
-template <int ORDER, typename R, bool FIELD = false>
+// With per-field constants also those of u-c, of entropy and shear, of u+c (a
+// struct of its own: the longer one cost batches 0.5 %).
+template <typename R>
+struct FieldConst : TileConst<R> {
+  R af[3];
+};
+template <bool FIELD, typename R>
+struct SweepConst {
+  using type = TileConst<R>;
+};
+template <typename R>
+struct SweepConst<true, R> {
+  using type = FieldConst<R>;
+};
+template <int ORDER, typename R>
 __device__ __forceinline__ void tile_const(const SweepArgs& A, double alpha_d, double dt,
                                            TileConst<R>& k) {
   k.alpha_d = alpha_d;
   k.dt = dt;
   k.alpha = (R)alpha_d;
   k.inv_dx = bconst<R>(A.inv_dx, A.inv_dx_f);
-  if constexpr (FIELD) {
-    for (int i = 0; i < 3; ++i) k.af[i] = (R)A.st->alpha_f[A.dir][i];
-  }
   k.dt32 = f32_rn(dt);
   k.wdt32 = f32_rn((A.stage == 0 ? 1.0 : (A.stage == 1 ? 0.25 : 2.0 / 3.0)) * dt);
   // below delta by more than the near-tie margin (and the bound's own
@@ -1578,7 +1588,8 @@ __device__ __forceinline__ unsigned choose_face(const SweepArgs& A, const TileGe
   const R tie_rel = bconst<R>(A.tie_rel, A.tie_rel_f);
   // splitting constant of field v: alpha, or per field max |u_d - c|, |u_d|, |u_d + c|
   auto afield = [&](int v) {
-    if constexpr (FIELD) return K.af[v == 0 ? 0 : (v == NV - 1 ? 2 : 1)];
+    if constexpr (FIELD)
+      return static_cast<const FieldConst<R>&>(K).af[v == 0 ? 0 : (v == NV - 1 ? 2 : 1)];
     return K.alpha;
   };
   const int j = G - 1 + f;  // face j+1/2 in extended cells
@@ -2595,8 +2606,12 @@ __global__ void __launch_bounds__(128, sweep_min_blocks<NV, ORDER, R, FIELD, TMA
   StepState* st = A.st;
   if (st->skip) return;
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  __shared__ TileConst<R> s_k;
-  if (threadIdx.x == 0) tile_const<ORDER, R, FIELD>(A, st->alpha[A.dir], st->dt, s_k);
+  __shared__ typename SweepConst<FIELD, R>::type s_k;
+  if (threadIdx.x == 0) {
+    tile_const<ORDER, R>(A, st->alpha[A.dir], st->dt, s_k);
+    if constexpr (FIELD)
+      for (int i = 0; i < 3; ++i) s_k.af[i] = (R)st->alpha_f[A.dir][i];
+  }
   constexpr int KA = kAmax<FIELD>;
   double amax[KA];
 #pragma unroll
